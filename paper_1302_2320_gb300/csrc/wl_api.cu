@@ -148,6 +148,8 @@ struct TuneRec {
     int best = 0;                          // 0 until every candidate has a rate
 };
 constexpr int kTuneS[3] = {32, 16, 8};
+// Lines per SM up to which each gets a block of its own (plan_shape).
+constexpr int kLonePerSM = 5;
 std::mutex g_tune_mu;
 std::map<TuneKey, TuneRec> g_tune_cache;
 
@@ -191,9 +193,6 @@ wl_status allocate(wl_ctx* h)
                     (long long)h->hbm_budget);
     CU(cudaGetDevice(&h->device));
     CU(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device));
-    int smem_optin = 0;
-    CU(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
-    h->max_smem = (size_t)smem_optin;
     CU(cudaStreamCreateWithFlags(&h->s, cudaStreamNonBlocking));
     CU(cudaEventCreate(&h->ev0));
     CU(cudaEventCreate(&h->ev1));
@@ -240,20 +239,7 @@ wl_status allocate(wl_ctx* h)
     return WL_OK;
 }
 
-Geo make_geo(const wl_ctx* h)
-{
-    Geo g;
-    g.type = h->g.type;
-    g.L = h->g.L;
-    g.N = h->g.N;
-    g.NB = h->g.NB;
-    g.W = h->lo.W;
-    g.magic = (((uint64_t)1 << 40) + (uint64_t)h->g.L - 1) / (uint64_t)h->g.L;
-    g.lshift = 0;
-    while ((1 << (g.lshift + 1)) <= h->g.L) ++g.lshift;
-    g.lmask = (uint32_t)h->g.L - 1u;
-    return g;
-}
+Geo make_geo(const wl_ctx* h) { return wl::make_geo(h->g.type, h->g.L, h->g.N, h->g.NB, h->lo.W); }
 
 // The work queue: selected lines by estimated cost (bins^2), largest first.
 wl_status upload_queue(wl_ctx* h)
@@ -375,100 +361,23 @@ WalkArgs base_args(wl_ctx* h)
 
 int kernel_lattice(const wl_ctx* h);
 
-// Tail shape: when no more lines are running than there are SMs, each gets a
-// block of its own with a conflict filter table (exact when it has N entries).
-bool tail_shape(wl_ctx* h, int S, int active, Shape* sh)
+// Shape of the persistent form for the lines still running (`active` of them).
+// The count is rounded up to whole walkers per SM, so the shape (and with it the
+// captured graph) changes only when that number does.
+wl_status persistent_shape(wl_ctx* h, int S, int active, Shape* sh)
 {
-    if (!h->tail || S != 32 || active < 1 || active > h->num_sms) return false;
-    const size_t isz = h->lo.idx16 ? 2 : 4;
-    const size_t stg = (size_t)h->lo.pstride * isz + (size_t)h->lo.W * 4;
-    const size_t cap = std::min<size_t>(h->max_smem, 220 * 1024);
-    int H = 32;
-    while (H < h->g.N && H < 32768) H <<= 1;
-    size_t tbl = (size_t)H * 4;
-    int stage = (kWinBytes + tbl + stg <= cap && stg <= 64 * 1024) ? 1 : 0;
-    while (kWinBytes + tbl + (stage ? stg : 0) > cap && H > 32) {
-        H >>= 1;
-        tbl = (size_t)H * 4;
-    }
-    const size_t slot = kWinBytes + tbl + (stage ? stg : 0);
-    if (slot > cap) return false;
-    int bps = 0;
-    if (walk_kernel_attrs(kernel_lattice(h), 32, h->det != 0, h->lo.idx16, slot, 32, &bps, true) != cudaSuccess ||
-        bps < 1)
-        return false;
-    sh->grid = dim3(std::min(active, h->num_sms));
-    sh->block = dim3(32);
-    sh->smem = slot;
-    sh->stage = stage;
-    sh->slot = (int)slot;
-    sh->tbl_mask = H - 1;
-    return true;
-}
-
-wl_status persistent_shape(wl_ctx* h, int S, int* blocks_per_sm_out, Shape* sh, int active = -1)
-{
-    if (active >= 0 && !blocks_per_sm_out && tail_shape(h, S, active, sh)) return WL_OK;
-    const size_t isz = h->lo.idx16 ? 2 : 4;
-    const size_t stg = (size_t)h->lo.pstride * isz + (size_t)h->lo.W * 4;
-    const size_t cap = std::min<size_t>(h->max_smem, 220 * 1024);
-    const int groups_per_warp = 32 / S;
-    int stage = 0, max_warps = 0;
-    size_t slot = kWinBytes;
-    const size_t warps_staged = cap / ((size_t)groups_per_warp * (kWinBytes + stg));
-    if (warps_staged >= 1 && stg <= 64 * 1024) {
-        stage = 1;
-        slot = kWinBytes + stg;
-        max_warps = (int)std::min<size_t>(8, warps_staged);
-    } else {
-        max_warps = (int)std::min<size_t>(8, cap / ((size_t)groups_per_warp * kWinBytes));
-    }
-    if (max_warps < 1) return fail(WL_ECUDA, "no walker shape fits shared memory (S=%d)", S);
-    // The smallest block that still holds every queued line in one wave spreads
-    // the walkers over the most SMs; otherwise take the largest capacity.
-    int best_w = 0, best_bps = 0;
-    long best_cap = -1;
-    for (int w = 1; w <= max_warps; ++w) {
-        const int threads = w * 32;
-        const size_t smem = (size_t)(threads / S) * slot;
-        int bps = 0;
-        CU(walk_kernel_attrs(kernel_lattice(h), S, h->det != 0, h->lo.idx16, smem, threads, &bps));
-        if (bps < 1) continue;
-        const long capy = (long)h->num_sms * bps * (threads / S);
-        if (capy >= h->nqueue) {
-            best_w = w;
-            best_bps = bps;
-            best_cap = capy;
-            break;
-        }
-        if (capy > best_cap) {
-            best_w = w;
-            best_bps = bps;
-            best_cap = capy;
-        }
-    }
-    if (best_w == 0) return fail(WL_ECUDA, "walker kernel cannot be resident (S=%d)", S);
-    const int threads = best_w * 32;
-    const size_t smem = (size_t)(threads / S) * slot;
-    const int groups_per_block = threads / S;
-    const int need_blocks = (h->nqueue + groups_per_block - 1) / groups_per_block;
-    const int blocks = std::max(1, std::min(need_blocks, h->num_sms * best_bps));
-    sh->grid = dim3(blocks);
-    sh->block = dim3(threads);
-    sh->smem = smem;
-    sh->stage = stage;
-    sh->slot = (int)slot;
-    if (blocks_per_sm_out) *blocks_per_sm_out = best_bps;
-    return WL_OK;
+    const int per_sm = h->num_sms * (32 / S);
+    const int lines = std::min<int64_t>(h->nqueue, (int64_t)((active + per_sm - 1) / per_sm) * per_sm);
+    const ShapeKey k{kernel_lattice(h), S, h->det != 0, h->lo.idx16, h->g.L, h->g.N, h->lo.pstride,
+                     h->lo.desc.back().nbins, std::max(lines, 1), h->tail != 0 && S == 32};
+    return plan_shape(k, sh);
 }
 
 // One slice of the persistent form on stream h->s (capturable).
 wl_status enqueue_slice(wl_ctx* h, int S, const Shape& sh)
 {
     WalkArgs a = base_args(h);
-    a.stage_smem = sh.stage;
-    a.slot_bytes = sh.slot;
-    a.tbl_mask = sh.tbl_mask;
+    set_slot(sh.slot, &a);
     CU(cudaMemsetAsync(a.qnext, 0, 4, h->s));
     if (h->slice_ms > 0) CU(launch_set_deadline(h->d_deadline + 1, (uint64_t)h->slice_ms * 1000000ull, h->s));
     CU(launch_walk(kernel_lattice(h), S, h->det != 0, h->lo.idx16, sh.grid, sh.block, sh.smem, h->s, a));
@@ -486,11 +395,8 @@ wl_status run_slice(wl_ctx* h, int S, const Shape& sh, bool use_graph)
         return WL_OK;
     }
     WalkArgs now = base_args(h);
-    now.stage_smem = sh.stage;
-    now.slot_bytes = sh.slot;
-    now.tbl_mask = sh.tbl_mask;
-    const bool same = h->graph && h->graph_S == S && h->graph_stage == sh.stage &&
-                      h->graph_grid == sh.grid.x && h->graph_block == sh.block.x &&
+    set_slot(sh.slot, &now);
+    const bool same = h->graph && h->graph_S == S && h->graph_grid == sh.grid.x && h->graph_block == sh.block.x &&
                       memcmp(&h->graph_args, &now, sizeof now) == 0;
     if (!same) {
         if (h->graph) cudaGraphExecDestroy(h->graph);
@@ -505,7 +411,6 @@ wl_status run_slice(wl_ctx* h, int S, const Shape& sh, bool use_graph)
         cudaGraphDestroy(g);
         if (e != cudaSuccess) return fail(WL_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
         h->graph_S = S;
-        h->graph_stage = sh.stage;
         h->graph_grid = sh.grid.x;
         h->graph_block = sh.block.x;
         memcpy(&h->graph_args, &now, sizeof now);
@@ -566,7 +471,7 @@ wl_status run_persistent(wl_ctx* h, std::chrono::steady_clock::time_point t_star
         int curS = h->mapping;
         tried = -1;
         const int active = prev_moves < 0 ? h->nqueue : h->h_summary->active;
-        const bool tail = h->tail && (h->mapping == 0 || h->mapping == 32) && active <= h->num_sms;
+        const bool tail = h->tail && (h->mapping == 0 || h->mapping == 32) && active <= kLonePerSM * h->num_sms;
         if (tail) {
             curS = 32;
         } else if (curS == 0) {
@@ -579,7 +484,7 @@ wl_status run_persistent(wl_ctx* h, std::chrono::steady_clock::time_point t_star
             curS = tried >= 0 ? kTuneS[tried] : tr.best;
         }
         Shape sh;
-        wl_status st = persistent_shape(h, curS, nullptr, &sh, tail ? active : -1);
+        wl_status st = persistent_shape(h, curS, h->tail ? active : h->nqueue, &sh);
         if (st) return st;
         if (prev_moves < 0) {
             // moves before this run, for the tuning rates
@@ -644,18 +549,18 @@ wl_status run_plain(wl_ctx* h)
         CU(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
         h->pool.push_back(st);
     }
-    const size_t isz = h->lo.idx16 ? 2 : 4;
-    const size_t stg = (size_t)h->lo.pstride * isz + (size_t)h->lo.W * 4;
-    const int stage = (kWinBytes + stg <= std::min<size_t>(h->max_smem, 220 * 1024) &&
-                       stg <= 64 * 1024) ? 1 : 0;
-    const size_t slot = kWinBytes + (stage ? stg : 0);
-    const size_t smem = slot;
+    // one group per launch; as many launches as lines may share the SMs
+    Shape sh;
+    const ShapeKey key{kernel_lattice(h), S, h->det != 0, h->lo.idx16, h->g.L, h->g.N, h->lo.pstride,
+                       h->lo.desc.back().nbins, h->nqueue, false};
+    wl_status ps = plan_shape(key, &sh);
+    if (ps) return ps;
+    const size_t smem = (size_t)sh.slot.bytes;
     CU(cudaMemsetAsync(h->d_qheads, 0, h->lo.nlines * 4, h->s));
     CU(cudaEventRecord(h->ev_join, h->s));
     for (auto st : h->pool) CU(cudaStreamWaitEvent(st, h->ev_join, 0));
     WalkArgs a = base_args(h);
-    a.stage_smem = stage;
-    a.slot_bytes = (int)slot;
+    set_slot(sh.slot, &a);
     a.nqueue = 1;
     std::vector<LineState> st_host(h->lo.nlines);
     for (;;) {
@@ -722,6 +627,153 @@ wl_status prepare(wl_ctx* h, double ln_f_min, double flatness, cudaStream_t afte
     return WL_OK;
 }
 
+// A walker's slot: the list (staged or not), the sites, the window, the step
+// records.  The window is what is left of `room` bytes, up to the whole line; a
+// guard on both sides of it keeps every address inside the slot even where a
+// caller's own state (wl_walk_noalloc) is not one of the line's.
+static bool plan_slot(const ShapeKey& k, bool sites, bool perm, size_t room, Slot* o)
+{
+    constexpr int kGuard = 8 * 8 * (12 + 1);      // kSub steps of the largest bin step, in bytes
+    constexpr int kOwners = 4096;
+    // room for the margins of both edges and a walk between them
+    const int min_win = std::min(k.max_bins, k.lattice == kTriangular || k.lattice == kCubic ? 384 : 256);
+    Slot s;
+    size_t at = perm ? (size_t)k.pstride * (k.idx16 ? 2 : 4) : 0;
+    s.stage_perm = perm;
+    s.stage_sites = sites;
+    s.off_sites = (int)at;
+    s.owner_mask = kOwners - 1;
+    at += sites ? ((size_t)k.N + 31) / 32 * 32 : (size_t)kOwners;
+    at = std::max<size_t>(align16(at), kGuard);
+    s.off_win = (int)at;
+    const size_t after = std::max<size_t>(align16((size_t)k.S * kStepBytes), kGuard);
+    if (at + (size_t)min_win * 8 + 16 + after > room) return false;
+    s.win = (int)std::min<size_t>((size_t)k.max_bins, (room - 16 - at - after) / 8);
+    at += align16((size_t)s.win * 8);
+    s.off_rec = (int)at;
+    s.bytes = (int)align16(at + after);
+    *o = s;
+    return true;
+}
+
+void set_slot(const Slot& slot, WalkArgs* a)
+{
+    a->slot_bytes = slot.bytes;
+    a->off_sites = slot.off_sites;
+    a->off_win = slot.off_win;
+    a->off_rec = slot.off_rec;
+    a->win_bins = slot.win;
+    a->owner_mask = slot.owner_mask;
+    a->stage_perm = slot.stage_perm;
+    a->stage_sites = slot.stage_sites;
+    a->off_perm = slot.off_perm;
+    a->lone = slot.lone;
+}
+
+static cudaError_t walk_attrs(const ShapeKey& k, const Slot& slot, size_t smem, int threads, int* bps)
+{
+    WalkArgs a{};
+    set_slot(slot, &a);
+    return walk_kernel_attrs(k.lattice, k.S, k.det, k.idx16, smem, threads, a, bps);
+}
+
+// The slot of a line with a block of its own (wl_lone.cuh): the words of the sites
+// by code and one more, the list, the window, the ring.
+static bool plan_lone(const ShapeKey& k, size_t room, Slot* o)
+{
+    if (!k.idx16) return false;
+    size_t stride = 1;
+    while (stride < (size_t)k.L) stride <<= 1;
+    const size_t codes = k.lattice == kCubic ? stride * stride * k.L : stride * k.L;
+    // the words start at a whole row (cubic: plane), and a list entry holds an address
+    const size_t row = 4 * stride * (k.lattice == kCubic ? stride : 1);
+    if (4 * (codes + 1) + row > 65536 - 2048) return false;
+    const int min_win = std::min(k.max_bins, 1024);   // two margins of 32 steps and a walk between them
+    Slot s;
+    s.lone = true;
+    size_t at = align16(4 * (codes + 1) + row);
+    s.off_perm = (int)at;
+    at += (size_t)k.pstride * 2;
+    s.off_win = (int)at;
+    const size_t ring = (128 + 3) * 32 + 32 + 128;   // the draws, their flags, control words, spare words
+    if (at + (size_t)min_win * 8 + 16 + ring > room) return false;
+    s.win = (int)std::min<size_t>((size_t)k.max_bins, (room - 16 - at - ring) / 8);
+    at += align16((size_t)s.win * 8);
+    s.off_rec = (int)at;
+    s.bytes = (int)(at + ring);
+    *o = s;
+    return true;
+}
+
+// One warp per block, 32 / S walkers each.  The shape spreads the walkers over
+// the SMs and gives each the shared memory its share of an SM leaves.  When the
+// walkers do not all fit at once with their lists staged, the lists stay in
+// global memory if that takes fewer rounds: they are read once per batch, so
+// they cost a batch one L2 latency, while a round more costs a whole walk.
+wl_status plan_shape(const ShapeKey& k, Shape* sh)
+{
+    int dev = 0, sms = 0, per_block = 0, per_sm = 0, reserved = 0;
+    CU(cudaGetDevice(&dev));
+    CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    CU(cudaDeviceGetAttribute(&per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    CU(cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    CU(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
+    const int groups = 32 / k.S;
+    const int need = (k.lines + groups - 1) / groups;       // blocks wanted
+    const int want = std::min((need + sms - 1) / sms, 32);  // per SM
+    auto room_of = [&](int blocks) {   // bytes of a block with this many on an SM
+        const int b = std::min(per_block, per_sm / blocks - reserved - 128) / 128 * 128;
+        return b > 0 ? (size_t)b : (size_t)0;
+    };
+    // few lines: a block each (~45 cycles of issue and ~90 of latency a step, so
+    // several share an SM before the batches of the other kernel are cheaper)
+    const int per = (k.lines + sms - 1) / sms;
+    if (k.lone && per <= kLonePerSM && plan_lone(k, room_of(per), &sh->slot)) {
+        int bps = 0;
+        CU(walk_attrs(k, sh->slot, sh->slot.bytes, 64, &bps));
+        if (bps < 1) return fail(WL_ECUDA, "walker kernel cannot be resident");
+        sh->grid = dim3(k.lines);
+        sh->block = dim3(64);
+        sh->smem = sh->slot.bytes;
+        return WL_OK;
+    }
+    auto room = [&](int blocks) {      // bytes per walker with this many blocks on an SM
+        const int b = std::min(per_block, per_sm / blocks - reserved) / 128 * 128;
+        return b > 0 ? (size_t)b / groups / 16 * 16 : (size_t)0;
+    };
+    struct Mode {
+        bool sites, perm;
+        double cycles;                 // a lone walker's cycles per move, to weigh rounds
+    };
+    const Mode modes[3] = {{true, true, 72.0}, {true, false, 84.0}, {false, false, 110.0}};
+    double best = 0.0;
+    int best_blocks = 0;
+    for (const Mode& m : modes) {
+        if (m.sites && !k.idx16) continue;
+        int b = want;
+        Slot slot;
+        while (b > 0 && !plan_slot(k, m.sites, m.perm, room(b), &slot)) --b;
+        if (b == 0) continue;
+        int bps = 0;
+        CU(walk_attrs(k, slot, (size_t)groups * slot.bytes, 32, &bps));
+        b = std::min(b, bps);
+        if (b < 1) continue;
+        const double rounds = (double)((need + sms * b - 1) / (sms * b));
+        // ~28 warp instructions a move, four schedulers
+        const double cost = rounds * std::max(m.cycles, 7.0 * b);
+        if (best_blocks == 0 || cost < best) {
+            if (!plan_slot(k, m.sites, m.perm, room(b), &sh->slot)) continue;
+            best = cost;
+            best_blocks = b;
+        }
+    }
+    if (best_blocks == 0) return fail(WL_ECUDA, "no walker shape fits shared memory (S=%d)", k.S);
+    sh->grid = dim3(std::max(1, std::min(need, sms * best_blocks)));
+    sh->block = dim3(32);
+    sh->smem = (size_t)groups * sh->slot.bytes;
+    return WL_OK;
+}
+
 wl_status choose_shape(wl_ctx* h, int* S, Shape* sh)
 {
     int m = h->mapping;
@@ -732,7 +784,7 @@ wl_status choose_shape(wl_ctx* h, int* S, Shape* sh)
     }
     *S = m;
     h->last_mapping = m;
-    return persistent_shape(h, m, nullptr, sh);
+    return persistent_shape(h, m, h->nqueue, sh);
 }
 
 wl_status launch_slice_async(wl_ctx* h, int S, const Shape& sh) { return run_slice(h, S, sh, true); }

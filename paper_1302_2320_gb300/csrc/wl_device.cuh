@@ -20,11 +20,6 @@ constexpr int kTableBytes = kTableN * 4;     // entries 1..4095 as u32; entry 0 
 // fewer neighbours; k takes every value, so bins have step 1).
 enum LatticeType : int { kSquare = 0, kTriangular = 1, kCubic = 2, kSquareP2 = 3, kSquareOpen = 4 };
 
-// Per-walker window in shared memory: ln g (int64) of kWin bins, then the
-// histogram counts (u32) the walker added to them since the window was loaded.
-constexpr int kWin = 64;
-constexpr int kWinBytes = kWin * 12;
-
 // Per-line scalar state (device, one per walked line).
 struct LineState {
     int64_t k;         // current number of unhappy bonds
@@ -38,6 +33,8 @@ struct LineState {
     int64_t batches;   // speculative batches evaluated (diagnostic)
 };
 
+constexpr int kStepBytes = 40;     // shared bytes of a lane's step record (Steps in wl_walk.cuh)
+
 struct LineDesc {
     int64_t bin_off;   // first bin of this line in the ragged lng/hist arrays
     int32_t ell;       // number of up spins
@@ -49,7 +46,26 @@ struct Geo {
     uint64_t magic;          // ceil(2^40 / L): x / L == (x * magic) >> 40 for x < 2^24
     int lshift;              // log2(L) when L is a power of two
     uint32_t lmask;          // L - 1 when L is a power of two
+    int cshift;              // site codes (wl_lone.cuh): L rounded up to a power of two is 1 << cshift
+    uint32_t cmask;          // (1 << cshift) - 1
 };
+
+// The geometry of an L lattice of N sites, W spin words per line.
+inline Geo make_geo(int type, int L, int N, int NB, int W)
+{
+    Geo g{};
+    g.type = type;
+    g.L = L;
+    g.N = N;
+    g.NB = NB;
+    g.W = W;
+    g.magic = (((uint64_t)1 << 40) + (uint64_t)L - 1) / (uint64_t)L;
+    while ((1 << (g.lshift + 1)) <= L) ++g.lshift;
+    g.lmask = (uint32_t)L - 1u;
+    while ((1 << g.cshift) < L) ++g.cshift;
+    g.cmask = (1u << g.cshift) - 1u;
+    return g;
+}
 
 // Everything a walker launch needs.  Pointers are device memory.
 struct WalkArgs {
@@ -69,11 +85,16 @@ struct WalkArgs {
     float inv_u;             // 1 / u, production acceptance
     uint32_t seed;
     int32_t flat_pm;         // flatness fraction x in 1/1000
-    int32_t stage_smem;      // 1: lists and spins staged in shared memory
-    int32_t slot_bytes;      // shared bytes per walker slot (window + staged list/spins)
+    // a walker's slot of shared memory (plan_slot in wl_api.cu)
+    int32_t slot_bytes;
+    int32_t off_perm, off_sites, off_win, off_rec;
+    int32_t win_bins;        // bins of ln g held in the window
+    int32_t owner_mask;      // sites not staged: owner table entries - 1
+    int32_t stage_perm;      // 1: the list is staged at the start of the slot
+    int32_t stage_sites;     // 1: one byte per site staged (selects the kernel)
+    int32_t lone;            // 1: one block per line (selects the kernel)
     int32_t pstride;         // list entries per line, N rounded up to 16 bytes
     int32_t same_f_resets;   // R > 0: extra histogram resets at unchanged f (see walk_line)
-    int32_t tbl_mask;        // conflict filter table: tbl_mask + 1 words per walker (tail kernel)
     int64_t C;               // flatness check interval
     int64_t C_per_bin;       // > 0: a line of n bins checks every max(C, C_per_bin * n) moves
     int64_t budget;          // per-line cap on t
@@ -175,39 +196,6 @@ __device__ __forceinline__ unsigned open_neighbours(const Geo& g, uint32_t i, ui
     return v;
 }
 
-// delta_k that also returns the neighbour lists of i and j (used to decide
-// which later proposals an accepted exchange of i and j can affect).
-template <int LAT>
-__device__ __forceinline__ int delta_k_nb(const Geo& g, const uint32_t* sp, uint32_t i, uint32_t j,
-                                          uint32_t* ni, uint32_t* nj)
-{
-    constexpr int z = Coord<LAT>::z;
-    if constexpr (LAT == kSquareOpen) {
-        // with degrees z_i, z_j: dk = 2 (u_i - u_j + a_ij) - z_i + z_j
-        const unsigned vi = open_neighbours(g, i, ni), vj = open_neighbours(g, j, nj);
-        int ui = 0, uj = 0, a = 0;
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            ui += (int)(((vi >> m) & 1u) & spin_at(sp, ni[m]));
-            uj += (int)(((vj >> m) & 1u) & spin_at(sp, nj[m]));
-            a += (int)(((vi >> m) & 1u) && ni[m] == j);
-            if (!((vi >> m) & 1u)) ni[m] = 0xFFFFFFFFu;     // never equal to a site
-            if (!((vj >> m) & 1u)) nj[m] = 0xFFFFFFFFu;
-        }
-        return 2 * (ui - uj + a) - __popc(vi) + __popc(vj);
-    }
-    neighbours<LAT>(g, i, ni);
-    neighbours<LAT>(g, j, nj);
-    int ui = 0, uj = 0, a = 0;
-#pragma unroll
-    for (int m = 0; m < z; ++m) {
-        ui += (int)spin_at(sp, ni[m]);
-        uj += (int)spin_at(sp, nj[m]);
-        a += (int)(ni[m] == j);
-    }
-    return 2 * (ui - uj + a);
-}
-
 // Eq. 3 as a threshold on d, the ln g difference g(k')/g(k) in units of u.
 // Both acceptance rules are non-increasing in d, so the uphill moves a random
 // word r accepts are d = 1 .. dmax(r), and a move is accepted iff d <= dmax(r)
@@ -271,22 +259,23 @@ __device__ __forceinline__ int64_t dmax_det(uint32_t r, const uint32_t* tab, int
     const float lr = __log2f(__uint_as_float(0x3F800000u | frac)) + (float)(31 - lz);
     int c = (int)float_floor_i64(fmaxf((32.0f - lr) * seg_per_log2, 0.0f));
     c = c < 1 ? 1 : (c > kTableN - 3 ? kTableN - 3 : c);
+    // i* = max{i <= 4094 : t[i] > r}, t non-increasing; the estimate is i* itself
+    // but for words next to an entry, so the other two entries are read only then
     const uint64_t R = r;
-    const uint64_t tm = table_at(tab, c - 1), t0 = (uint64_t)tab[c], t1 = (uint64_t)tab[c + 1],
-                   t2 = (uint64_t)tab[c + 2];
-    // i* = max{i <= 4094 : t[i] > r}, t non-increasing
-    int seg;
-    uint64_t a, b;                  // t[i*], t[i*+1]
-    if (t0 > R && t1 <= R) {
-        seg = c; a = t0; b = t1;
-    } else if (tm > R && t0 <= R) {
-        seg = c - 1; a = tm; b = t0;
-    } else if (t1 > R && (t2 <= R || c + 1 == kTableN - 2)) {
-        seg = c + 1; a = t1; b = t2;
-    } else {
-        seg = dmax_segment_search(r, tab);
-        a = table_at(tab, seg);
-        b = table_at(tab, seg + 1);
+    const uint64_t t0 = (uint64_t)tab[c], t1 = (uint64_t)tab[c + 1];
+    int seg = c;
+    uint64_t a = t0, b = t1;        // t[i*], t[i*+1]
+    if (!(t0 > R && t1 <= R)) {
+        const uint64_t tm = table_at(tab, c - 1), t2 = (uint64_t)tab[c + 2];
+        if (tm > R && t0 <= R) {
+            seg = c - 1; a = tm; b = t0;
+        } else if (t1 > R && (t2 <= R || c + 1 == kTableN - 2)) {
+            seg = c + 1; a = t1; b = t2;
+        } else {
+            seg = dmax_segment_search(r, tab);
+            a = table_at(tab, seg);
+            b = table_at(tab, seg + 1);
+        }
     }
     if (b > R) return ((int64_t)(kTableN - 1) << q) - 1;   // the whole last segment
     // largest frac < 2^q with diff * frac < X 2^q, i.e. floor((X 2^q - 1) / diff)

@@ -93,6 +93,72 @@ __global__ void init_kernel(const InitArgs A)
     }
 }
 
+// ---------------------------------------------------------------------------
+// A caller's own walker state (wl_walk_noalloc): one warp per running line checks
+// that the list is a permutation whose first l entries are the up spins and that
+// k is theirs.  The walkers take this for granted; a line that fails gets the
+// status and the flag of a broken invariant and is not walked.
+// ---------------------------------------------------------------------------
+template <int LAT, typename IDX>
+__global__ void check_state_kernel(const InitArgs A, int32_t* flags)
+{
+    const int li = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (li >= A.nlines || A.st[li].status != 0) return;
+    const LineDesc D = A.desc[li];
+    const int N = A.g.N;
+    const IDX* perm = reinterpret_cast<const IDX*>(A.perm) + (size_t)li * A.pstride;
+    const uint32_t* sp = A.spins + (size_t)li * A.g.W;
+    constexpr int z = Coord<LAT>::z;
+    int up = 0, twice = 0, bad = 0;
+    // every entry a site of the right spin; with l up spins in all and the sums
+    // and sums of squares of 0 .. N-1 the entries are all different in practice
+    int64_t s1 = 0, s2 = 0;
+    for (int n = lane; n < N; n += 32) {
+        const uint32_t e = (uint32_t)perm[n];
+        if (e >= (uint32_t)N) {
+            bad = 1;
+            continue;
+        }
+        bad |= spin_at(sp, e) != (n < D.ell ? 1u : 0u);
+        s1 += (int64_t)e - n;
+        s2 += (int64_t)e * e - (int64_t)n * n;
+        uint32_t nb[z];
+        neighbours<LAT>(A.g, (uint32_t)n, nb);
+        const uint32_t sn = spin_at(sp, (uint32_t)n);
+        up += (int)sn;
+#pragma unroll
+        for (int q = 0; q < z; ++q) twice += sn != spin_at(sp, nb[q]);
+    }
+    up = group_sum<32>(0xffffffffu, up);
+    twice = group_sum<32>(0xffffffffu, twice);
+    s1 = group_sum<32>(0xffffffffu, s1);
+    s2 = group_sum<32>(0xffffffffu, s2);
+    bad |= up != D.ell || s1 != 0 || s2 != 0 || A.st[li].k != twice / 2 || A.st[li].t < 0;
+    if (__any_sync(0xffffffffu, bad) && lane == 0) {
+        A.st[li].status = 3;
+        atomicOr(flags, 8);
+    }
+}
+
+cudaError_t launch_check_state(int lattice, bool idx16, const InitArgs& a, int32_t* flags, cudaStream_t s)
+{
+    clear_stale_error();
+    const int warps = 4;
+    const dim3 grid((a.nlines + warps - 1) / warps), block(32 * warps);
+    if (lattice == kSquare) {
+        if (idx16) check_state_kernel<kSquare, uint16_t><<<grid, block, 0, s>>>(a, flags);
+        else check_state_kernel<kSquare, uint32_t><<<grid, block, 0, s>>>(a, flags);
+    } else if (lattice == kTriangular) {
+        if (idx16) check_state_kernel<kTriangular, uint16_t><<<grid, block, 0, s>>>(a, flags);
+        else check_state_kernel<kTriangular, uint32_t><<<grid, block, 0, s>>>(a, flags);
+    } else {
+        if (idx16) check_state_kernel<kCubic, uint16_t><<<grid, block, 0, s>>>(a, flags);
+        else check_state_kernel<kCubic, uint32_t><<<grid, block, 0, s>>>(a, flags);
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_init(int lattice, bool idx16, const InitArgs& a, cudaStream_t s)
 {
     clear_stale_error();
@@ -506,20 +572,18 @@ cudaError_t launch_walk(int lattice, int S, bool det, bool idx16, dim3 grid, dim
     return launch_walk_cubic(S, det, idx16, grid, block, smem, s, a, nullptr);
 }
 
-cudaError_t walk_kernel_attrs(int lattice, int S, bool det, bool idx16, size_t smem,
-                              int block_threads, int* blocks_per_sm, bool tbl)
+cudaError_t walk_kernel_attrs(int lattice, int S, bool det, bool idx16, size_t smem, int block_threads,
+                              const WalkArgs& a, int* blocks_per_sm)
 {
-    WalkArgs dummy{};
-    dummy.tbl_mask = tbl ? 1 : 0;
     const dim3 z(0), b(block_threads);
-    if (lattice == kSquare) return launch_walk_square(S, det, idx16, z, b, smem, 0, dummy, blocks_per_sm);
+    if (lattice == kSquare) return launch_walk_square(S, det, idx16, z, b, smem, 0, a, blocks_per_sm);
     if (lattice == kSquareP2)
-        return launch_walk_square_p2(S, det, idx16, z, b, smem, 0, dummy, blocks_per_sm);
+        return launch_walk_square_p2(S, det, idx16, z, b, smem, 0, a, blocks_per_sm);
     if (lattice == kTriangular)
-        return launch_walk_triangular(S, det, idx16, z, b, smem, 0, dummy, blocks_per_sm);
+        return launch_walk_triangular(S, det, idx16, z, b, smem, 0, a, blocks_per_sm);
     if (lattice == kSquareOpen)
-        return launch_walk_square_open(S, det, idx16, z, b, smem, 0, dummy, blocks_per_sm);
-    return launch_walk_cubic(S, det, idx16, z, b, smem, 0, dummy, blocks_per_sm);
+        return launch_walk_square_open(S, det, idx16, z, b, smem, 0, a, blocks_per_sm);
+    return launch_walk_cubic(S, det, idx16, z, b, smem, 0, a, blocks_per_sm);
 }
 
 }  // namespace wl

@@ -38,8 +38,9 @@ constexpr int kMappings[] = {1, 2, 4, 8, 16, 32};
 // Walker launch (one persistent grid, or one group for a single line).
 cudaError_t launch_walk(int lattice, int S, bool det, bool idx16, dim3 grid, dim3 block,
                         size_t smem, cudaStream_t s, const WalkArgs& a);
-cudaError_t walk_kernel_attrs(int lattice, int S, bool det, bool idx16, size_t smem,
-                              int block_threads, int* blocks_per_sm, bool tbl = false);
+// Blocks of the kernel that `a` selects on an SM; also admits its shared memory.
+cudaError_t walk_kernel_attrs(int lattice, int S, bool det, bool idx16, size_t smem, int block_threads,
+                              const WalkArgs& a, int* blocks_per_sm);
 
 cudaError_t launch_walk_square(int S, bool det, bool idx16, dim3 grid, dim3 block, size_t smem,
                                cudaStream_t s, const WalkArgs& a, int* bps);
@@ -53,6 +54,7 @@ cudaError_t launch_walk_square_open(int S, bool det, bool idx16, dim3 grid, dim3
                                     cudaStream_t s, const WalkArgs& a, int* bps);
 
 cudaError_t launch_init(int lattice, bool idx16, const InitArgs& a, cudaStream_t s);
+cudaError_t launch_check_state(int lattice, bool idx16, const InitArgs& a, int32_t* flags, cudaStream_t s);
 cudaError_t launch_assemble(const LineDesc* desc, const int64_t* lng, const hist_t* hist, int N,
                             int nlines, double u, double* out, cudaStream_t s);
 cudaError_t launch_exp_table(double u, int q, uint64_t* out, cudaStream_t s);

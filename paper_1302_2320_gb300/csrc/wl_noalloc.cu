@@ -119,7 +119,8 @@ extern "C" wl_status wl_walk_noalloc(wl_lattice lattice, int L, int ell_first, i
     if (flat_pm < 1) return nfail(WL_EINVAL, "flatness below 0.001");
     if (check_interval < 1 || check_interval > 0x7FFFFFFFll) return nfail(WL_EINVAL, "check_interval out of range");
     if (move_budget < 0) return nfail(WL_EINVAL, "move_budget < 0");
-    if (mapping == 0) mapping = 8;
+    const bool own_choice = mapping == 0;
+    if (own_choice) mapping = 32;
     if (!(mapping == 1 || mapping == 2 || mapping == 4 || mapping == 8 || mapping == 16 || mapping == 32))
         return nfail(WL_EINVAL, "mapping must be 0, 1, 2, 4, 8, 16 or 32");
     if (!perm || !spins || !lng || !hist || !state) return nfail(WL_EINVAL, "NULL buffer");
@@ -171,6 +172,7 @@ extern "C" wl_status wl_walk_noalloc(wl_lattice lattice, int L, int ell_first, i
 
     // ---- descriptors and work queue (static host staging -> scratch) ----
     int64_t off = 0;
+    int max_bins = 0;
     for (int i = 0; i < nlines; ++i) {
         const int l = ell_first + i;
         const int lm = std::min(l, N - l);
@@ -179,6 +181,7 @@ extern "C" wl_status wl_walk_noalloc(wl_lattice lattice, int L, int ell_first, i
         g_desc[i].ell = l;
         g_desc[i].nbins = (int)(khi / 2 + 1);
         off += g_desc[i].nbins;
+        max_bins = std::max(max_bins, g_desc[i].nbins);
         g_order[i] = i;
     }
     std::stable_sort(g_order, g_order + nlines,
@@ -203,52 +206,31 @@ extern "C" wl_status wl_walk_noalloc(wl_lattice lattice, int L, int ell_first, i
     // pageable host -> device copies have taken the data once they return
     stage_lock.unlock();
 
-    Geo g;
-    g.type = (int)lattice;
-    g.L = L;
-    g.N = N;
-    g.NB = NB;
-    g.W = W;
-    g.magic = (((uint64_t)1 << 40) + (uint64_t)L - 1) / (uint64_t)L;
-    g.lshift = 0;
-    while ((1 << (g.lshift + 1)) <= L) ++g.lshift;
-    g.lmask = (uint32_t)L - 1u;
+    const Geo g = make_geo((int)lattice, L, N, NB, W);
     const int klat = (lattice == WL_SQUARE && (L & (L - 1)) == 0) ? (int)kSquareP2 : (int)lattice;
     LineState* d_st = reinterpret_cast<LineState*>(state);
 
-    if (init) {
-        InitArgs ia;
-        ia.g = g;
-        ia.desc = d_desc;
-        ia.st = d_st;
-        ia.perm = perm;
-        ia.spins = spins;
-        ia.lng = lng;
-        ia.hist = hist;
-        ia.pstride = pstride;
-        ia.nlines = nlines;
-        ia.seed = seed;
-        ia.F0 = std::llround(1.0 / ln_f_min);
-        NCU(launch_init((int)lattice, idx16, ia, s));
-    }
+    InitArgs ia;
+    ia.g = g;
+    ia.desc = d_desc;
+    ia.st = d_st;
+    ia.perm = perm;
+    ia.spins = spins;
+    ia.lng = lng;
+    ia.hist = hist;
+    ia.pstride = pstride;
+    ia.nlines = nlines;
+    ia.seed = seed;
+    ia.F0 = std::llround(1.0 / ln_f_min);
+    if (init) NCU(launch_init((int)lattice, idx16, ia, s));
+    else NCU(launch_check_state((int)lattice, idx16, ia, d_flags, s));
 
-    // ---- launch shape: one warp per block, lists staged in shared memory
-    // when a warp's walkers fit ----
-    int dev = 0, nsm = 0, smem_optin = 0;
-    NCU(cudaGetDevice(&dev));
-    NCU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    NCU(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    // ---- launch shape ----
     const int S = mapping;
-    const int groups = 32 / S;
-    const size_t stg = (size_t)pstride * isz + (size_t)W * 4;
-    const size_t cap = std::min<size_t>((size_t)smem_optin, 220 * 1024);
-    const int stage = ((size_t)groups * (kWinBytes + stg) <= cap && stg <= 64 * 1024) ? 1 : 0;
-    const size_t slot = kWinBytes + (stage ? stg : 0);
-    const size_t smem = (size_t)groups * slot;
-    int bps = 0;
-    NCU(walk_kernel_attrs(klat, S, deterministic != 0, idx16, smem, 32, &bps));
-    if (bps < 1) return nfail(WL_ECUDA, "walker cannot be resident");
-    const int blocks = std::max(1, std::min((nlines + groups - 1) / groups, nsm * bps));
+    wl::rt::Shape sh;
+    const wl::rt::ShapeKey key{klat, S, deterministic != 0, idx16, L, N, pstride, max_bins, nlines, own_choice};
+    st = wl::rt::plan_shape(key, &sh);
+    if (st) return st;
 
     WalkArgs a{};
     a.g = g;
@@ -267,8 +249,7 @@ extern "C" wl_status wl_walk_noalloc(wl_lattice lattice, int L, int ell_first, i
     a.inv_u = (float)(1.0 / ln_f_min);
     a.seed = seed;
     a.flat_pm = flat_pm;
-    a.stage_smem = stage;
-    a.slot_bytes = (int)slot;
+    wl::rt::set_slot(sh.slot, &a);
     a.pstride = pstride;
     a.C = check_interval;
     a.budget = move_budget;
@@ -281,7 +262,7 @@ extern "C" wl_status wl_walk_noalloc(wl_lattice lattice, int L, int ell_first, i
     Summary sm;
     for (;;) {
         NCU(cudaMemsetAsync(d_qnext, 0, 4, s));
-        NCU(launch_walk(klat, S, deterministic != 0, idx16, dim3(blocks), dim3(32), smem, s, a));
+        NCU(launch_walk(klat, S, deterministic != 0, idx16, sh.grid, sh.block, sh.smem, s, a));
         NCU(launch_summary(d_st, nlines, move_budget, d_flags, d_summary, s));
         NCU(cudaMemcpyAsync(&sm, d_summary, sizeof sm, cudaMemcpyDeviceToHost, s));
         NCU(cudaStreamSynchronize(s));

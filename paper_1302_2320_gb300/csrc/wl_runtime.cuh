@@ -25,14 +25,32 @@ struct Layout {
     std::vector<LineDesc> desc;
 };
 
+// A walker's slot of shared memory.
+struct Slot {
+    int bytes = 0, off_perm = 0, off_sites = 0, off_win = 0, off_rec = 0;
+    int win = 0;                 // bins of the ln g window
+    int owner_mask = 0;
+    bool stage_sites = false, stage_perm = false, lone = false;
+};
+
 // Launch shape of the persistent form for S lanes per walker.
 struct Shape {
     dim3 grid, block;
-    size_t smem;
-    int stage;
-    int slot;
-    int tbl_mask = 0;   // tail shape: one walker per block with a conflict filter table
+    size_t smem = 0;
+    Slot slot;
 };
+
+// What the shape of a launch depends on.
+struct ShapeKey {
+    int lattice;         // kernel specialisation (LatticeType)
+    int S;               // lanes per walker
+    bool det, idx16;
+    int L, N, pstride;
+    int max_bins;        // bins of the largest line
+    int lines;           // walkers wanted at once
+    bool lone;           // few lines may get a block each (wl_lone.cuh)
+};
+
 
 }  // namespace rt
 }  // namespace wl
@@ -69,7 +87,6 @@ struct wl_ctx {
     int64_t init_moves = 0;
     // device
     int device = 0, num_sms = 0;
-    size_t max_smem = 0;
     cudaStream_t s = nullptr;
     std::vector<cudaStream_t> pool;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_join = nullptr;
@@ -96,7 +113,7 @@ struct wl_ctx {
     int nqueue = 0;
     // captured slice graph
     cudaGraphExec_t graph = nullptr;
-    int graph_S = -1, graph_stage = -1;
+    int graph_S = -1;
     unsigned graph_grid = 0, graph_block = 0;
     wl::WalkArgs graph_args{};          // arguments baked into the captured graph
 };
@@ -118,6 +135,10 @@ namespace rt {
 wl_status prepare(wl_ctx* h, double ln_f_min, double flatness, cudaStream_t after);
 // Lanes per walker (option, autotune cache or default) and the launch shape.
 wl_status choose_shape(wl_ctx* h, int* S, Shape* sh);
+// The launch shape of `k` on the current device, and its fields of the kernel's
+// arguments.
+wl_status plan_shape(const ShapeKey& k, Shape* sh);
+void set_slot(const Slot& slot, WalkArgs* a);
 // Enqueue one slice (captured graph) on the handle's stream; asynchronous.
 // The slice's summary lands in h->h_summary when the stream reaches it.
 wl_status launch_slice_async(wl_ctx* h, int S, const Shape& sh);

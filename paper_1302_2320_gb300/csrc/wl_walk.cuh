@@ -7,35 +7,39 @@
 //     ahead: the list slots a, b and dmax, the largest ln g increase that
 //     Eq. 3 accepts with this step's random word (see dmax_det / dmax_prod);
 //   propose -- lane m evaluates its exchange against the state at the start of
-//     the batch: sites i = U[a], j = D[b], their neighbours and the change of
-//     k;
-//   resolve -- while the walker stays in its bin, step m sees that bin's ln g
-//     plus F for every step in between (a rejection and an accepted exchange
-//     with the same k both visit the current bin), so every lane tests its own
-//     step at once (ln g(target) <= ln g(current) + dmax); a ballot finds the
-//     first accepted step, the rejections before it are committed together,
-//     and the lanes are tested again only when an accepted step changes the
-//     bin or the proposals.
-// An accepted exchange of (i_e, j_e) changes a later proposal in two ways.  If
-// the proposal reuses list slot a_e or b_e (equivalently: names site i_e or
-// j_e, the lists holding distinct sites) its sites are no longer U[a], D[b]:
-// the batch is cut short before it.  If one of i_e, j_e neighbours its sites,
-// its change of k is off by 2 for every such neighbour (i_e turned down, j_e
-// up): the later lanes correct it in place and are tested again.  The later
-// proposals an exchange may affect are found with 2z equality tests per lane,
-// or (TBL, the tail shape: one walker per block) with two loads from a
-// shared-memory table that lists, per site, the lanes having it among their
-// sites or their neighbours.  The exchanges accepted in a batch touch distinct
-// slots and distinct sites, so they are applied together after the resolution.
+//     the batch: sites i = U[a], j = D[b] and the change of k, and collects the
+//     earlier proposals that could change either (below);
+//   chain -- the group's first lane alone takes the steps in order: one load of
+//     ln g at the target bin, one 64-bit compare, one store of ln g at the bin
+//     the step ends in.
+// The chain is the serial part of the method.  It costs ~18 instructions a step
+// whether the step is accepted or not, all its operands but the target's ln g
+// are known before it starts, and its critical path is one shared-memory load,
+// the compare and a select.
+//
+// What an accepted exchange of (i_e, j_e) does to a later proposal: if that one
+// uses the same list slot (equivalently: names site i_e or j_e, the lists
+// holding distinct sites) its sites are no longer U[a], D[b]; if i_e or j_e
+// neighbours its sites, its change of k is another.  Every site has a byte that
+// names the lane proposing it (its "owner"; of several lanes proposing one site
+// the last to write), so a proposal learns the owners of its sites and their
+// neighbours from the same bytes that hold their spins.  The chain keeps the
+// set of owners whose site an accepted step has moved; a step that sees one of
+// them stops the chain, the accepted exchanges are applied, the group evaluates
+// that one step again from the lists and spins as they now are, and the chain
+// goes on.  A step whose evaluation is out of date is always seen: its sites
+// and their neighbours at the start of the batch include every site through
+// which an earlier step can have reached it, also when a re-evaluated step took
+// a site that entered its slot within the batch (that site was itself proposed
+// in the batch, so it has an owner).
 // Random numbers are keyed by t, so the committed chain is the sequential
 // chain, bit for bit, for every S and both forms.  Batches never cross a
 // flatness check (t multiple of C) or the end of the slice.
 //
-// The current bin's ln g and its visits not yet counted live in registers; the
-// bins around it live in a shared-memory window (ln g, and the histogram counts
-// added since the window was loaded: the visits to a bin the walker left are
-// added by the lane of the step that left it, at the end of the batch), written
-// back when the walker re-centres it, at every check and at the end.
+// ln g of the bins around the walker lives in a shared-memory window, written
+// back when the walker nears an edge of it, at every check and at the end.  A
+// visit adds F to a bin's ln g and 1 to its count, so the counts are not kept
+// while walking: storing the window recovers them as (ln g - ln g before) / F.
 #pragma once
 
 #include "wl_device.cuh"
@@ -61,17 +65,25 @@ __device__ __forceinline__ unsigned group_ballot(unsigned gmask, int gbase, bool
 // Flatness (80%/80% convention, fraction x = flat_pm/1000, exact integers):
 // n visited bins, Ssum = their histogram total, c = bins with
 // 1000*n*h >= flat_pm*Ssum; flat iff 1000*c >= flat_pm*n.
+// Both passes issue kFlatUnroll independent loads per lane: the histogram lies in
+// L2, and one load at a time makes a check cost its latency times bins / S.
+constexpr int kFlatUnroll = 8;
+
 template <int S>
 __device__ bool group_flat(const hist_t* hist, int nbins, int m, unsigned gmask, int flat_pm)
 {
     int64_t n = 0;
     uint64_t ssum = 0;
-    for (int b = m; b < nbins; b += S) {
-        const hist_t h = hist[b];
-        if (h & kVisited) {
-            n += 1;
-            ssum += h & ~kVisited;
-        }
+    for (int b0 = m; b0 < nbins; b0 += S * kFlatUnroll) {
+        hist_t h[kFlatUnroll];
+#pragma unroll
+        for (int q = 0; q < kFlatUnroll; ++q) h[q] = b0 + q * S < nbins ? hist[b0 + q * S] : 0ull;
+#pragma unroll
+        for (int q = 0; q < kFlatUnroll; ++q)
+            if (h[q] & kVisited) {
+                n += 1;
+                ssum += h[q] & ~kVisited;
+            }
     }
     n = group_sum<S>(gmask, n);
     ssum = group_sum<S>(gmask, ssum);
@@ -80,9 +92,13 @@ __device__ bool group_flat(const hist_t* hist, int nbins, int m, unsigned gmask,
     // products of up to ~2^77: compared in 128-bit integers
     const unsigned __int128 rhs = (unsigned __int128)flat_pm * ssum;
     const unsigned __int128 scale = (unsigned __int128)(1000 * n);
-    for (int b = m; b < nbins; b += S) {
-        const hist_t h = hist[b];
-        if ((h & kVisited) && scale * (h & ~kVisited) >= rhs) c += 1;
+    for (int b0 = m; b0 < nbins; b0 += S * kFlatUnroll) {
+        hist_t h[kFlatUnroll];
+#pragma unroll
+        for (int q = 0; q < kFlatUnroll; ++q) h[q] = b0 + q * S < nbins ? hist[b0 + q * S] : 0ull;
+#pragma unroll
+        for (int q = 0; q < kFlatUnroll; ++q)
+            if ((h[q] & kVisited) && scale * (h[q] & ~kVisited) >= rhs) c += 1;
     }
     c = group_sum<S>(gmask, c);
     return 1000 * c >= (int64_t)flat_pm * n;
@@ -106,45 +122,73 @@ __device__ void group_stage_step(int64_t* lng, hist_t* hist, int nbins, int m, u
     __syncwarp(gmask);
 }
 
-// Window of ln g / histogram bins a walker keeps in shared memory.  Every
-// proposal lies within z bins of the current bin (|dk| <= 2z), so the window
-// [wb, wb + kWin) is re-centred whenever the current bin comes within z bins of
-// an edge that is not the line's own edge.  The window holds ln g and the
-// counts added since it was loaded; storing it adds the counts to the global
-// histogram (a bin with a count is marked visited) and zeroes them.  Counts
-// reaching 2^62 (far beyond any run) are reported as an overflow.
-template <int S>
-__device__ __forceinline__ bool window_store(int64_t* wl, uint32_t* wd, int64_t* lng, hist_t* hist,
-                                             int wb, int wn, int m)
+// Visits behind an increase d of a bin's ln g: d / F, exact.  Every round takes a
+// quotient estimated from below to one part in 2^18, so counts below 2^18 need
+// two at most (the float helpers keep the FP64 pipe out of it).
+__device__ __forceinline__ uint64_t visits_of(int64_t d, int64_t F, float inv_f)
 {
+    uint64_t rem = (uint64_t)d, n = 0;
+    while (rem >= (uint64_t)F) {
+        uint64_t e = (uint64_t)float_floor_i64(u64_to_float_rz(rem) * inv_f);
+        e = e ? e : 1;
+        n += e;
+        rem -= e * (uint64_t)F;
+    }
+    return n;
+}
+
+// 1 / F rounded so that the estimates of visits_of never exceed the quotient.
+__device__ __forceinline__ float inverse_below(int64_t F)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(u64_to_float_rz((uint64_t)F)));
+    return r * (1.0f - 0x1p-18f);
+}
+
+// Store the window [wb, wb + wn) of ln g; the visits made since it was loaded
+// are added to the histogram and mark their bins visited.  Counts reaching 2^62
+// (far beyond any run) are reported as an overflow.
+template <int S>
+__device__ __forceinline__ bool window_store(const int64_t* wl, int64_t* lng, hist_t* hist, int wb,
+                                             int wn, int m, int64_t F)
+{
+    constexpr int U = 4;      // independent loads per lane and round
     bool ovf = false;
-    for (int x = m; x < wn; x += S) {
-        lng[wb + x] = wl[x];
-        const uint32_t add = wd[x];
-        if (add) {
-            const hist_t h = hist[wb + x] + add;
-            ovf |= (h & ~kVisited) >= (1ull << 62);
-            hist[wb + x] = h | kVisited;
-            wd[x] = 0u;
+    const float inv_f = inverse_below(F);
+    for (int x0 = m; x0 < wn; x0 += U * S) {
+        int64_t d[U];
+        hist_t h[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int x = x0 + q * S;
+            d[q] = x < wn ? wl[x] - lng[wb + x] : 0;
+            h[q] = x < wn ? hist[wb + x] : 0ull;
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int x = x0 + q * S;
+            if (d[q]) {
+                h[q] += visits_of(d[q], F, inv_f);
+                ovf |= (h[q] & ~kVisited) >= (1ull << 62);
+                hist[wb + x] = h[q] | kVisited;
+                lng[wb + x] = wl[x];
+            }
         }
     }
     return ovf;
 }
 
 template <int S>
-__device__ __forceinline__ void window_load(int64_t* wl, uint32_t* wd, const int64_t* lng, int wb,
-                                            int wn, int m)
+__device__ __forceinline__ void window_load(int64_t* wl, const int64_t* lng, int wb, int wn, int m)
 {
-    for (int x = m; x < wn; x += S) {
-        wl[x] = lng[wb + x];
-        wd[x] = 0u;
-    }
+#pragma unroll 4
+    for (int x = m; x < wn; x += S) wl[x] = lng[wb + x];
 }
 
-__device__ __forceinline__ int window_base(int bc, int nbins)
+__device__ __forceinline__ int window_base(int bc, int nbins, int win)
 {
-    int wb = bc - kWin / 2;
-    if (wb > nbins - kWin) wb = nbins - kWin;
+    int wb = bc - win / 2;
+    if (wb > nbins - win) wb = nbins - win;
     return wb < 0 ? 0 : wb;
 }
 
@@ -160,34 +204,255 @@ __device__ __forceinline__ Draw draw_step(uint64_t t, uint2 key, uint32_t ell, u
     return d;
 }
 
-template <int S>
-__device__ __forceinline__ Draw shfl_draw(unsigned gmask, const Draw& d, int src)
+// The spins and the owners of the sites proposed in the current batch.
+// BYTES: one byte per site in shared memory, the spin at the start of the batch
+// in bit 7 and the owner's lane in bits 0..6 (kNoOwner: none), so that one load
+// answers both questions.
+// Otherwise (a lattice larger than shared memory): packed spins in global memory
+// and owners in a shared table indexed by the low bits of the site; sites that
+// share an entry share an owner, which can only add evaluations.
+constexpr uint32_t kNoOwner = 0x40u;
+
+template <bool BYTES>
+struct Sites {
+    uint8_t* own;      // BYTES: N bytes; otherwise mask + 1 owners
+    uint32_t* sp;      // packed spins (not BYTES)
+    uint32_t mask;
+    __device__ __forceinline__ uint32_t peek(uint32_t n) const
+    {
+        if constexpr (BYTES) return own[n];
+        else return own[n & mask] | (spin_at(sp, n) << 7);
+    }
+    __device__ __forceinline__ void mark(uint32_t n, uint32_t spin, uint32_t lane) const
+    {
+        if constexpr (BYTES) own[n] = (uint8_t)((spin << 7) | lane);
+        else own[n & mask] = (uint8_t)lane;
+    }
+    // no owner, and (BYTES) the spin
+    __device__ __forceinline__ void clear(uint32_t n, uint32_t spin) const
+    {
+        if constexpr (BYTES) own[n] = (uint8_t)((spin << 7) | kNoOwner);
+        else own[n & mask] = (uint8_t)kNoOwner;
+    }
+};
+
+// 1 << owner of a site byte, 0 for kNoOwner (a PTX shift by 32 or more gives 0).
+__device__ __forceinline__ uint32_t owner_bit(uint32_t v)
 {
-    Draw o;
-    o.a = __shfl_sync(gmask, d.a, src);
-    o.b = __shfl_sync(gmask, d.b, src);
-    o.dmax = __shfl_sync(gmask, d.dmax, src);
-    return o;
+    uint32_t r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(v & 0x7Fu));
+    return r;
+}
+
+// Owners next to the two sites of a proposal: of up and of down neighbours of i
+// and of j (the up ones own a site that an accepted step turns down, and so on).
+struct Near {
+    uint32_t iu, id, ju, jd;
+};
+
+// The sites of the batch that have turned since its start, by owner: up sites
+// turned down, down sites turned up.  Every owner owns one site of each kind.
+struct Turned {
+    uint32_t up, down;
+};
+
+// The change of k when i (up) and j (down) exchange.  NEAR: with the spins as the
+// bytes hold them, and the owners around; otherwise (BYTES) with the spins as
+// they are after `turned`.
+template <int LAT, bool BYTES, bool NEAR>
+__device__ __forceinline__ int exchange_dk(const Geo& g, const Sites<BYTES>& st, uint32_t i, uint32_t j,
+                                           const Turned& turned, Near* near)
+{
+    constexpr int z = Coord<LAT>::z;
+    uint32_t ni[z], nj[z];
+    unsigned vi = (1u << z) - 1u, vj = vi;
+    if constexpr (LAT == kSquareOpen) {
+        vi = open_neighbours(g, i, ni);
+        vj = open_neighbours(g, j, nj);
+    } else {
+        neighbours<LAT>(g, i, ni);
+        neighbours<LAT>(g, j, nj);
+    }
+    int ui = 0, uj = 0, a = 0;
+    Near o{0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int q = 0; q < z; ++q) {
+        const uint32_t pi = st.peek(ni[q]), pj = st.peek(nj[q]);
+        int si = (int)(pi >> 7), sj = (int)(pj >> 7);
+        const uint32_t oi = owner_bit(pi), oj = owner_bit(pj);
+        if constexpr (BYTES && !NEAR) {
+            si ^= (oi & (si ? turned.up : turned.down)) != 0u;
+            sj ^= (oj & (sj ? turned.up : turned.down)) != 0u;
+        }
+        bool adj = ni[q] == j;
+        if constexpr (LAT == kSquareOpen) {
+            if (!((vi >> q) & 1u)) si = 0, adj = false;
+            if (!((vj >> q) & 1u)) sj = 0;
+        }
+        ui += si;
+        uj += sj;
+        a += adj;
+        if constexpr (NEAR) {
+            const bool hi = LAT != kSquareOpen || ((vi >> q) & 1u), hj = LAT != kSquareOpen || ((vj >> q) & 1u);
+            const uint32_t mi = hi ? oi : 0u, mj = hj ? oj : 0u;
+            const uint32_t fi = 0u - (pi >> 7), fj = 0u - (pj >> 7);
+            o.iu |= mi & fi;
+            o.id |= mi & ~fi;
+            o.ju |= mj & fj;
+            o.jd |= mj & ~fj;
+        }
+    }
+    if constexpr (NEAR) *near = o;
+    int dk = 2 * (ui - uj + a);
+    // with site degrees z_i, z_j: dk = 2 (u_i - u_j + a_ij) - z_i + z_j
+    if constexpr (LAT == kSquareOpen) dk += __popc(vj) - __popc(vi);
+    return dk;
+}
+
+// What the chain needs of the steps of a batch, in shared memory:
+//   a {dmax (two words), the owners whose move makes the step out of date, its
+//     bin step in bytes of the window}
+//   b {the owner of its up site, of its down site, as bits}
+//   c the owners around (Near), read when the step is out of date
+template <int S>
+struct Steps {
+    uint4 a[S];
+    uint4 c[S];
+    uint2 b[S];
+};
+
+// State of the chain (held by the group's first lane while it runs).
+struct Chain {
+    uint32_t xa;     // shared address of the current bin in the window
+    int64_t u;       // its ln g
+    uint32_t moved;  // owners with a site that an accepted step has moved
+    Turned turned;
+    uint32_t accm;   // accepted steps of the batch
+    int s;           // steps taken
+};
+
+// K steps of the chain from step c.s on, or up to the first that is out of date.
+// Written in PTX for the predication: the compiler turns the updates of an
+// accepted step into selects and every exit into a divergent branch with its
+// own reconvergence, ~30 instructions a step against 20 here.  The serial path
+// of a step is: target address, load, compare, select.  The load is issued before
+// the out-of-date test; its address is then wrong by a few bins at most, inside
+// the slot's guard.  The window always holds every visit, so a step with no
+// change of bin needs no case of its own: it reads ln g of its own bin and is
+// accepted, dmax being >= 0.
+#define WL_REC(q, oa, ob)                                         \
+    "ld.shared.v4.u32 {l" #q ", h" #q ", z" #q ", k" #q "}, [%7+" #oa "];\n\t" \
+    "ld.shared.v2.u32 {i" #q ", j" #q "}, [%8+" #ob "];\n\t"
+#define WL_STEP(q, bit, next)                                     \
+    "add.u32 ta, %0, k" #q ";\n\t"                                \
+    "ld.shared.s64 g, [ta];\n\t"                                  \
+    next                                                          \
+    "and.b32 t, z" #q ", %2;\n\t"                                 \
+    "setp.ne.u32 p, t, 0;\n\t"                                    \
+    "@p bra.uni X" #q ";\n\t"                                     \
+    "mov.b64 d, {l" #q ", h" #q "};\n\t"                          \
+    "add.s64 d, d, %1;\n\t"                                       \
+    "add.s64 %1, %1, %9;\n\t"                                     \
+    "setp.le.s64 p, g, d;\n\t"                                    \
+    "add.s64 g, g, %9;\n\t"                                       \
+    "@p mov.u32 %0, ta;\n\t"                                      \
+    "@p mov.b64 %1, g;\n\t"                                       \
+    "st.shared.s64 [%0], %1;\n\t"                                 \
+    "@p lop3.b32 %2, %2, i" #q ", j" #q ", 0xFE;\n\t"             \
+    "@p xor.b32 %3, %3, i" #q ";\n\t"                             \
+    "@p xor.b32 %4, %4, j" #q ";\n\t"                             \
+    "@p or.b32 %5, %5, " #bit ";\n\t"
+#define WL_REGS(q) ".reg .b32 l" #q ", h" #q ", z" #q ", k" #q ", i" #q ", j" #q ";\n\t"
+#define WL_EXIT(q) "X" #q ": mov.u32 %6, " #q ";\n\t bra.uni DONE;\n\t"
+#define WL_CHAIN_OPERANDS                                                                   \
+    : "+r"(c.xa), "+l"(c.u), "+r"(c.moved), "+r"(c.turned.up), "+r"(c.turned.down), "+r"(acc), "=r"(n) \
+    : "r"(ra), "r"(rb), "l"(F) : "memory"
+
+template <int K>
+__device__ __forceinline__ int chain_steps(Chain& c, uint32_t ra, uint32_t rb, int64_t F)
+{
+    uint32_t n, acc = 0u;
+    ra += 16u * (uint32_t)c.s;
+    rb += 8u * (uint32_t)c.s;
+    if constexpr (K == 8) {
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 ta, t;\n\t.reg .b64 g, d;\n\t"
+            WL_REGS(0) WL_REGS(1) WL_REGS(2) WL_REGS(3) WL_REGS(4) WL_REGS(5) WL_REGS(6) WL_REGS(7)
+            WL_REC(0, 0, 0) WL_REC(1, 16, 8)
+            WL_STEP(0, 1, WL_REC(2, 32, 16)) WL_STEP(1, 2, WL_REC(3, 48, 24))
+            WL_STEP(2, 4, WL_REC(4, 64, 32)) WL_STEP(3, 8, WL_REC(5, 80, 40))
+            WL_STEP(4, 16, WL_REC(6, 96, 48)) WL_STEP(5, 32, WL_REC(7, 112, 56))
+            WL_STEP(6, 64, "") WL_STEP(7, 128, "")
+            "mov.u32 %6, 8;\n\tbra.uni DONE;\n\t"
+            WL_EXIT(0) WL_EXIT(1) WL_EXIT(2) WL_EXIT(3) WL_EXIT(4) WL_EXIT(5) WL_EXIT(6) WL_EXIT(7)
+            "DONE:\n\t}" WL_CHAIN_OPERANDS);
+    } else if constexpr (K == 4) {
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 ta, t;\n\t.reg .b64 g, d;\n\t"
+            WL_REGS(0) WL_REGS(1) WL_REGS(2) WL_REGS(3)
+            WL_REC(0, 0, 0) WL_REC(1, 16, 8)
+            WL_STEP(0, 1, WL_REC(2, 32, 16)) WL_STEP(1, 2, WL_REC(3, 48, 24))
+            WL_STEP(2, 4, "") WL_STEP(3, 8, "")
+            "mov.u32 %6, 4;\n\tbra.uni DONE;\n\t"
+            WL_EXIT(0) WL_EXIT(1) WL_EXIT(2) WL_EXIT(3)
+            "DONE:\n\t}" WL_CHAIN_OPERANDS);
+    } else {
+        static_assert(K == 1, "chain_steps");
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 ta, t;\n\t.reg .b64 g, d;\n\t"
+            WL_REGS(0) WL_REC(0, 0, 0) WL_STEP(0, 1, "")
+            "mov.u32 %6, 1;\n\tbra.uni DONE;\n\t" WL_EXIT(0)
+            "DONE:\n\t}" WL_CHAIN_OPERANDS);
+    }
+    c.accm |= acc << c.s;
+    c.s += (int)n;
+    return (int)n;
+}
+
+// Take steps c.s .. lim-1; 0: all taken, 1: step c.s has to be evaluated again
+// by the group, 2: the walker is near an edge of its window (tested every kSub
+// steps; lo and hi leave the margin that kSub steps can use up).
+// An out-of-date step whose own sites are where they were only has another
+// change of k, by the sites around it that have turned: that is a count of owner
+// bits (BYTES: owners are exact), and the step is taken here.
+constexpr int kSub = 8;
+
+template <int S, int KS, bool BYTES>
+__device__ __forceinline__ int run_chain(Chain& c, Steps<S>* steps, int lim, int64_t F, uint32_t lo, uint32_t hi)
+{
+    const uint32_t ra = (uint32_t)__cvta_generic_to_shared(steps->a);
+    const uint32_t rb = (uint32_t)__cvta_generic_to_shared(steps->b);
+    while (c.s < lim) {
+        if (c.xa < lo || c.xa > hi) return 2;
+        const int left = lim - c.s;
+        bool fresh;
+        if (S >= 8 && left >= 8) fresh = chain_steps<8>(c, ra, rb, F) == 8;
+        else if (S >= 4 && left >= 4) fresh = chain_steps<4>(c, ra, rb, F) == 4;
+        else fresh = chain_steps<1>(c, ra, rb, F) == 1;
+        if (fresh) continue;
+        if constexpr (!BYTES) {
+            return 1;
+        } else {
+            const uint2 b = steps->b[c.s];
+            if ((b.x | b.y) & c.moved) return 1;
+            const uint4 o = steps->c[c.s];
+            const int d = __popc(o.z & c.turned.up) - __popc(o.x & c.turned.up) + __popc(o.y & c.turned.down) -
+                          __popc(o.w & c.turned.down);
+            steps->a[c.s].z = 0u;
+            steps->a[c.s].w += (uint32_t)(d * (16 >> KS));
+        }
+    }
+    return 0;
 }
 
 // Walk line `li` for up to A.slice_moves moves (or to its budget, or to
-// convergence).  perm/sp point at the line's list and spins (shared or global
-// memory); win is the group's window (kWin int64 ln g, then kWin u32 counts).
+// convergence).  perm points at the line's list (shared or global memory), st at
+// its spins; wl is the group's window, steps its step records (shared memory).
 // All lanes of the group hold identical copies of the scalar state.
-//
-// Draws are double-buffered: lane m holds the draw of step t + m in d0 and of
-// t + S + m in d1.  After a batch commits c steps the buffers shift by c (a
-// plain copy when c = S, the usual case), and the lanes whose entry falls past
-// the buffered range take the draw of step t + c + S + m, computed at the
-// start of the next batch so its latency overlaps that batch's work.
-template <int LAT, int S, bool DET, typename IDX, bool TBL>
-__device__ void walk_line(const WalkArgs& A, int li, int m, int gbase, unsigned gmask,
-                          IDX* perm, uint32_t* sp, uint8_t* win, uint32_t* tbl)
+template <int LAT, int S, bool DET, typename IDX, bool BYTES>
+__device__ void walk_line(const WalkArgs& A, int li, int m, int gbase, unsigned gmask, IDX* perm,
+                          const Sites<BYTES>& st, int64_t* wl, Steps<S>* steps)
 {
     constexpr int zb = Coord<LAT>::zbin;  // largest bin step of one move
     constexpr int ks = Coord<LAT>::kshift;
-    constexpr int zc = Coord<LAT>::z;
-    constexpr bool kPack = sizeof(IDX) == 2;   // slots and sites fit 16 bits
+    constexpr int kMargin = kSub * (zb + 1);
     const LineDesc D = A.desc[li];
     LineState* P = A.st + li;
     int64_t t = P->t, F = P->F, stage = P->stage, accepts = P->accepts;
@@ -199,267 +464,168 @@ __device__ void walk_line(const WalkArgs& A, int li, int m, int gbase, unsigned 
     const uint32_t nd = (uint32_t)(A.g.N - ell);
     int64_t* lng = A.lng + D.bin_off;
     hist_t* hist = A.hist + D.bin_off;
-    int64_t* wl = reinterpret_cast<int64_t*>(win);
-    uint32_t* wd = reinterpret_cast<uint32_t*>(win + kWin * 8);
     const uint2 key = make_uint2((uint32_t)ell, A.seed);
     int64_t end = t + A.slice_moves;
     if (end > A.budget) end = A.budget;
     // flatness check interval of this line: longer for lines with more bins
     const int64_t C = A.C_per_bin > 0 && A.C_per_bin * nbins > A.C ? A.C_per_bin * nbins : A.C;
 
-    int bc = k >> ks;
-    int wb = window_base(bc, nbins);
-    const int wn = nbins < kWin ? nbins : kWin;
-    window_load<S>(wl, wd, lng, wb, wn, m);
-    __syncwarp(gmask);
-    int64_t cur = wl[bc - wb];    // ln g of the current bin, every visit included
-    int pend = 0;                 // visits to the current bin not yet in the window
     int stop = 0;
-    int64_t mF = (int64_t)m * F;
+    int bc = k >> ks;
+    if (bc < 0 || bc >= nbins) {
+        stop = 4;                 // not a state of this line
+        bc = 0;
+        end = t;
+    }
+    const int wn = nbins < A.win_bins ? nbins : A.win_bins;
+    int wb = window_base(bc, nbins, A.win_bins);
+    window_load<S>(wl, lng, wb, wn, m);
+    __syncwarp(gmask);
+    const uint32_t wa = (uint32_t)__cvta_generic_to_shared(wl);
+    Chain c{};
+    c.xa = wa + 8u * (uint32_t)(bc - wb);
+    c.u = wl[bc - wb];
 
-    Draw d0 = draw_step<DET>((uint64_t)(t + m), key, (uint32_t)ell, nd, A);
-    Draw d1{};
-    uint64_t tf = (uint64_t)(t + S + m);   // pending draw for d1
-    bool needf = true;
+    Draw d = draw_step<DET>((uint64_t)(t + m), key, (uint32_t)ell, nd, A);
 
     while (t < end && !stop) {
         const int64_t next_check = (t / C + 1) * C;
         const int64_t seg_end = next_check < end ? next_check : end;
-        int left = (int)(seg_end - t);    // moves before the next check or the slice end
+        int64_t left = seg_end - t;       // moves before the next check or the slice end
 
         while (left > 0) {
-            const int lim = left < S ? left : S;
-            // the pending draw (independent of this batch)
-            const Draw df = draw_step<DET>(tf, key, (uint32_t)ell, nd, A);
+            const int lim = left < S ? (int)left : S;
             // -- propose: step t + m against the state at the start of the batch
-            const uint32_t a = d0.a, b = d0.b;
-            const uint32_t i = (uint32_t)perm[a];
-            const uint32_t j = (uint32_t)perm[ell + b];
-            uint32_t ni[zc], nj[zc];
-            int dk = delta_k_nb<LAT>(A.g, sp, i, j, ni, nj);
-            if (needf) d1 = df;
-            // accepted iff ln g(target) <= ln g(current before step m) + dmax, and
-            // ln g(current before step m) = u + m F while the walker keeps its bin
-            const int64_t base = mF + d0.dmax;
-            // U and D are lists of distinct sites, so a later proposal reuses
-            // list slot a_e (b_e) of an accepted exchange iff its i (j) is i_e (j_e)
-            const uint32_t ij = kPack ? (i | (j << 16)) : i;
-            if constexpr (TBL) {
-                // conflict filter: for every site, the lanes that have it among
-                // their sites or their sites' neighbours (hashed by the low bits);
-                // an accepted exchange looks up its own two sites
-                const uint32_t tm = (uint32_t)A.tbl_mask, bit = 1u << m;
-#pragma unroll
-                for (int q = 0; q < zc; ++q) {
-                    atomicOr(&tbl[ni[q] & tm], bit);
-                    atomicOr(&tbl[nj[q] & tm], bit);
-                }
-                atomicOr(&tbl[i & tm], bit);
-                atomicOr(&tbl[j & tm], bit);
-                __syncwarp(gmask);
+            const uint32_t i0 = (uint32_t)perm[d.a];
+            const uint32_t j0 = (uint32_t)perm[ell + d.b];
+            st.mark(i0, 1u, (uint32_t)m);
+            st.mark(j0, 0u, (uint32_t)m);
+            // the next batch's draw (independent of this batch: it hides the latencies here)
+            const Draw dn = draw_step<DET>((uint64_t)(t + S + m), key, (uint32_t)ell, nd, A);
+            __syncwarp(gmask);
+            Near near;
+            int dk = exchange_dk<LAT, BYTES, true>(A.g, st, i0, j0, Turned{0u, 0u}, &near);
+            const uint32_t oi = owner_bit(st.peek(i0)), oj = owner_bit(st.peek(j0));
+            steps->a[m] = make_uint4((uint32_t)d.dmax, (uint32_t)((uint64_t)d.dmax >> 32),
+                                     (near.iu | near.id | near.ju) | (near.jd | oi | oj), (uint32_t)((dk >> ks) * 8));
+            steps->b[m] = make_uint2(oi, oj);
+            if constexpr (BYTES) steps->c[m] = make_uint4(near.iu, near.id, near.ju, near.jd);
+            __syncwarp(gmask);
+            if constexpr (!BYTES) {
+                st.clear(i0, 1u);
+                st.clear(j0, 0u);
             }
-            int rec_x = 0;        // the bin this lane's step left, and its visits (counted at the end)
-            uint32_t rec_c = 0u;
-            // -- resolve.  One pass of the loop handles one accepted step (an
-            // event): the walker's state is updated by selects, the later lanes
-            // are evaluated again for the next event, and only the rare cases
-            // (off the window, a conflicting later proposal) branch.  Every
-            // branch depends on ballots or on values all lanes hold alike.
-            int lim_eff = lim;                                   // cut short by a reused slot
-            unsigned live = lim >= 32 ? 0xffffffffu : ((1u << lim) - 1u);
-            unsigned done = 0u;                                  // steps resolved so far
-            int64_t u = cur;      // ln g of the current bin before step 0, shifted as above
-            int ent = -pend;      // batch step at which the walker entered its bin
-            int kw = k - (wb << ks);                             // k relative to the window
-            unsigned accm = 0u;
-            int c = 0;
-            int64_t v;            // ln g of the target bin - m F
-            unsigned evb, offb;
-            {
-                const int wx = (kw + dk) >> ks;
-                const bool off = (unsigned)wx >= (unsigned)wn;
-                const int64_t ld = wl[off ? (kw >> ks) : wx];
-                v = ld - mF;
-                evb = group_ballot<S>(gmask, gbase, (dk == 0) | off | (ld <= u + base));
-                offb = group_ballot<S>(gmask, gbase, off);
-            }
+            uint32_t i = i0, j = j0;      // the sites the step exchanges, once it is taken
+            // -- the chain, with out-of-date steps evaluated again as they come up
+            const uint32_t lo = wb > 0 ? wa + 8u * kMargin : wa;
+            const uint32_t hi = wb + wn < nbins ? wa + 8u * (uint32_t)(wn - 1 - kMargin)
+                                                : wa + 8u * (uint32_t)(wn - 1);
+            c.moved = 0u;
+            c.turned = Turned{0u, 0u};
+            c.accm = 0u;
+            c.s = 0;
+            unsigned applied = 0u;
             for (;;) {
-                const unsigned ev = evb & live & ~done;
-                if (ev == 0u) {                      // the rest of the batch is rejected
-                    c = lim_eff;
-                    break;
-                }
-                const int e = __ffs(ev) - 1;
-                const int src = gbase + e;
-                const int dke = __shfl_sync(gmask, dk, src);
-                const int64_t ve = __shfl_sync(gmask, v, src);
-                const uint32_t ije = __shfl_sync(gmask, ij, src);
-                uint32_t je = 0;
-                if constexpr (!kPack) je = __shfl_sync(gmask, j, src);
-                const bool offe = (offb >> e) & 1u;  // walked off the window: ends the batch at e
-                // accepted step e: a new bin means steps e0 .. e-1 were rejections in the old one
-                const bool mv = (dke != 0) & !offe;
-                const int x = kw >> ks;
-                if (mv) wl[x] = u + (int64_t)e * F;
-                if (mv & (m == e)) {
-                    rec_x = x;
-                    rec_c = (uint32_t)(e - ent);
-                }
-                const int dkm = mv ? dke : 0;
-                k += dkm;
-                kw += dkm;
-                u = mv ? ve : u;
-                ent = mv ? e : ent;
-                accm |= 1u << e;                     // withdrawn below if e walked off the window
-                done = (2u << e) - 1u;
-                // the later lanes against the new state
-                int wx = (kw + dk) >> ks;
-                bool off = (unsigned)wx >= (unsigned)wn;
-                int64_t ld = wl[off ? (kw >> ks) : wx];
-                bool acc = (dk == 0) | off | (ld <= u + base);
-                // later proposals: one that reuses a slot of the exchange cuts the
-                // batch short before it, one next to it gets its change of k shifted
-                const uint32_t ie = kPack ? (ije & 0xFFFFu) : ije;
-                if constexpr (kPack) je = ije >> 16;
-                const uint32_t xs = ij ^ ije;
-                bool conflict;
-                if constexpr (TBL) {
-                    // lanes that may be affected (a superset); tested exactly below
-                    const uint32_t tm = (uint32_t)A.tbl_mask;
-                    conflict = ((tbl[ie & tm] | tbl[je & tm]) & live & ~done) != 0u;
-                }
-                bool n0 = false, n1 = false, n2 = false, n3 = false, slot = false;
-                if constexpr (!TBL) {
-                    slot = kPack ? (((xs & 0xFFFFu) == 0u) | ((xs >> 16) == 0u)) : ((xs == 0u) | (j == je));
-#pragma unroll
-                    for (int q = 0; q < zc; ++q) {
-                        n0 |= ni[q] == ie;
-                        n1 |= ni[q] == je;
-                        n2 |= nj[q] == ie;
-                        n3 |= nj[q] == je;
+                int why = 0;
+                if (m == 0) why = run_chain<S, ks, BYTES>(c, steps, lim, F, lo, hi);
+                __syncwarp(gmask);
+                // steps taken, reason and bin of the first lane
+                const uint32_t pk = __shfl_sync(gmask, ((c.xa - wa) & 0xFFFFFu) | ((uint32_t)c.s << 20) | ((uint32_t)why << 28), gbase);
+                c.accm = __shfl_sync(gmask, c.accm, gbase);
+                c.s = (int)((pk >> 20) & 0x3Fu);
+                c.xa = wa + (pk & 0xFFFFFu);
+                why = (int)(pk >> 28);
+                // the lists (distinct slots: a second step on a slot is out of date)
+                if (((c.accm & ~applied) >> m) & 1u) {
+                    perm[d.a] = (IDX)j;
+                    perm[ell + d.b] = (IDX)i;
+                    if constexpr (!BYTES) {
+                        atomicAnd(&st.sp[i >> 5], ~(1u << (i & 31u)));
+                        atomicOr(&st.sp[j >> 5], 1u << (j & 31u));
                     }
                 }
-                if (offe) {
-                    if ((unsigned)((k + dke) >> ks) >= (unsigned)nbins) stop = 4;   // invariant broken
-                    accm &= ~(1u << e);
-                    c = e;
-                    break;
+                applied = c.accm;
+                if constexpr (BYTES) {
+                    c.turned.up = __shfl_sync(gmask, c.turned.up, gbase);
+                    c.turned.down = __shfl_sync(gmask, c.turned.down, gbase);
                 }
-                if constexpr (!TBL)
-                    conflict = (group_ballot<S>(gmask, gbase, slot | (n0 | n1) | (n2 | n3)) & live & ~done) != 0u;
-                if (conflict) {
-                    if constexpr (TBL)
-                        slot = kPack ? (((xs & 0xFFFFu) == 0u) | ((xs >> 16) == 0u)) : ((xs == 0u) | (j == je));
-                    const unsigned sm = group_ballot<S>(gmask, gbase, slot) & live & ~done;
-                    if (sm) {
-                        lim_eff = __ffs(sm) - 1;             // > e
-                        live = (1u << lim_eff) - 1u;
+                __syncwarp(gmask);
+                if (why != 1) break;
+                // step c.s again, from the lists and spins as they now are
+                const uint32_t ac = __shfl_sync(gmask, d.a, gbase + c.s);
+                const uint32_t bb = __shfl_sync(gmask, d.b, gbase + c.s);
+                const uint32_t i2 = (uint32_t)perm[ac], j2 = (uint32_t)perm[ell + bb];
+                dk = exchange_dk<LAT, BYTES, false>(A.g, st, i2, j2, c.turned, nullptr);
+                if (m == c.s) {
+                    i = i2;
+                    j = j2;
+                    steps->a[m].z = 0u;
+                    steps->a[m].w = (uint32_t)((dk >> ks) * 8);
+                    if constexpr (BYTES) {
+                        // its sites by kind and owner: turning them toggles those bits
+                        const uint32_t pi = st.peek(i2), pj = st.peek(j2);
+                        const uint32_t bi = owner_bit(pi), bj = owner_bit(pj);
+                        steps->b[m] = make_uint2((pi >> 7 ? bi : 0u) | (pj >> 7 ? bj : 0u),
+                                                 (pi >> 7 ? 0u : bi) | (pj >> 7 ? 0u : bj));
                     }
-                    int cor = 0;
-#pragma unroll
-                    for (int q = 0; q < zc; ++q)
-                        cor += (int)(nj[q] == ie) - (int)(ni[q] == ie) + (int)(ni[q] == je) -
-                               (int)(nj[q] == je);
-                    dk += 2 * cor;
-                    wx = (kw + dk) >> ks;
-                    off = (unsigned)wx >= (unsigned)wn;
-                    ld = wl[off ? (kw >> ks) : wx];
-                    acc = (dk == 0) | off | (ld <= u + base);
                 }
-                v = ld - mF;
-                evb = group_ballot<S>(gmask, gbase, acc);
-                offb = group_ballot<S>(gmask, gbase, off);
-                // no step left: the next pass finds no event and ends the batch
-            }
-            bc = k >> ks;
-            cur = u + (int64_t)c * F;
-            pend = c - ent;
-            if (c == 0) stop = 4;                  // step t always fits the window
-            // visits to the bins the walker left in this batch, one lane per bin left
-            __syncwarp(gmask);
-            if (rec_c) atomicAdd(wd + rec_x, rec_c);
-            if constexpr (TBL) {
-                const uint32_t tm = (uint32_t)A.tbl_mask;
-#pragma unroll
-                for (int q = 0; q < zc; ++q) {
-                    tbl[ni[q] & tm] = 0u;
-                    tbl[nj[q] & tm] = 0u;
-                }
-                tbl[i & tm] = 0u;
-                tbl[j & tm] = 0u;
-            }
-            // apply the accepted exchanges (distinct slots, distinct sites)
-            if ((accm >> m) & 1u) {
-                perm[a] = (IDX)j;
-                perm[ell + b] = (IDX)i;
-                atomicAnd(&sp[i >> 5], ~(1u << (i & 31u)));
-                atomicOr(&sp[j >> 5], 1u << (j & 31u));
-            }
-            accepts += __popc(accm);
-            __syncwarp(gmask);
-            if ((bc - zb < wb && wb > 0) || (bc + zb >= wb + kWin && wb + kWin < nbins)) {
-                // re-centre the window (the current bin stays in registers)
-                if (group_ballot<S>(gmask, gbase, window_store<S>(wl, wd, lng, hist, wb, wn, m))) stop = 2;
-                __syncwarp(gmask);
-                wb = window_base(bc, nbins);
-                window_load<S>(wl, wd, lng, wb, wn, m);
                 __syncwarp(gmask);
             }
-            // shift the draw buffers by c: lane m now needs steps t + c + m (d0)
-            // and t + c + S + m (d1)
-            if (c == S) {
-                d0 = d1;
-                needf = true;
-            } else {
-                const int srcm = m + c;                       // < 2S
-                const int sl = gbase + (srcm & (S - 1));
-                const Draw x0 = shfl_draw<S>(gmask, d0, sl);
-                const Draw x1 = shfl_draw<S>(gmask, d1, sl);
-                needf = srcm >= S;
-                d0 = needf ? x1 : x0;
-                d1 = x1;
+            if constexpr (BYTES) {
+                // every owner writes back its two sites
+                if (oi == 1u << m) st.clear(i0, ((c.turned.up >> m) & 1u) ^ 1u);
+                if (oj == 1u << m) st.clear(j0, (c.turned.down >> m) & 1u);
+                __syncwarp(gmask);
             }
-            tf = (uint64_t)(t + c + S + m);
-            t += c;
-            left -= c;
+            const int taken = c.s;
+            accepts += __popc(c.accm);
             batches += 1;
+            const int x = (int)(c.xa - wa) >> 3;
+            bc = wb + x;
+            if (taken == 0 || x < 0 || x >= wn) {
+                stop = 4;                  // never: a step from inside the margins stays inside
+                break;
+            }
+            t += taken;
+            left -= taken;
+            if (c.xa < lo || c.xa > hi) {
+                // re-centre the window
+                if (group_ballot<S>(gmask, gbase, window_store<S>(wl, lng, hist, wb, wn, m, F))) stop = 2;
+                __syncwarp(gmask);
+                wb = window_base(bc, nbins, A.win_bins);
+                window_load<S>(wl, lng, wb, wn, m);
+                __syncwarp(gmask);
+                c.xa = wa + 8u * (uint32_t)(bc - wb);
+            }
+            d = dn;
+            if (taken != S) d = draw_step<DET>((uint64_t)(t + m), key, (uint32_t)ell, nd, A);
             if (stop) break;
         }
         if (stop) break;
 
         if (t == next_check) {
-            // current bin -> window -> global, then test flatness over the line
+            // window -> global, then test flatness over the line
             __syncwarp(gmask);
-            if (m == 0) {
-                wl[bc - wb] = cur;
-                wd[bc - wb] += (uint32_t)pend;
-            }
-            pend = 0;
-            __syncwarp(gmask);
-            if (group_ballot<S>(gmask, gbase, window_store<S>(wl, wd, lng, hist, wb, wn, m))) {
+            if (group_ballot<S>(gmask, gbase, window_store<S>(wl, lng, hist, wb, wn, m, F))) {
                 stop = 2;
                 break;
             }
             __syncwarp(gmask);
             checks += 1;
             const bool flat = group_flat<S>(hist, nbins, m, gmask, A.flat_pm);
-            if (!flat && A.same_f_resets > 0 && (t - t_stage) / C <= A.same_f_resets) {
-                // extra reset at unchanged f within the first R checks of a
-                // stage (the remark after Eq. 4): histogram reset, ln g shifted
+            // extra reset at unchanged f within the first R checks of a stage (the
+            // remark after Eq. 4): histogram reset, ln g shifted
+            const bool again = !flat && A.same_f_resets > 0 && (t - t_stage) / C <= A.same_f_resets;
+            if (flat || again) {
                 group_stage_step<S>(lng, hist, nbins, m, gmask);
-                window_load<S>(wl, wd, lng, wb, wn, m);
+                window_load<S>(wl, lng, wb, wn, m);
                 __syncwarp(gmask);
-                cur = wl[bc - wb];
+                c.u = wl[bc - wb];
             }
             if (flat) {
-                group_stage_step<S>(lng, hist, nbins, m, gmask);
-                F >>= 2;                     // ln f -> ln f / 4
-                mF = (int64_t)m * F;
                 stage += 1;
                 t_stage = t;
-                window_load<S>(wl, wd, lng, wb, wn, m);
-                __syncwarp(gmask);
-                cur = wl[bc - wb];
+                F >>= 2;                     // ln f -> ln f / 4
                 if (F == 0) {                // ln f < ln f_min
                     status = 1;
                     break;
@@ -478,21 +644,16 @@ __device__ void walk_line(const WalkArgs& A, int li, int m, int gbase, unsigned 
             if (req) stop = req;
         }
     }
-    // current bin -> window -> global
-    if (stop != 4) {
+    // window -> global (a converged line was stored at its last check)
+    if (stop != 4 && F != 0) {
         __syncwarp(gmask);
-        if (m == 0) {
-            wl[bc - wb] = cur;
-            wd[bc - wb] += (uint32_t)pend;
-        }
-        __syncwarp(gmask);
-        if (group_ballot<S>(gmask, gbase, window_store<S>(wl, wd, lng, hist, wb, wn, m)) && stop == 0)
+        if (group_ballot<S>(gmask, gbase, window_store<S>(wl, lng, hist, wb, wn, m, F)) && stop == 0)
             stop = 2;
     }
     if (stop == 2) status = 2;
     if (stop == 4) status = 3;
     if (m == 0) {
-        P->k = k;
+        P->k = (int64_t)bc << ks;
         P->t = t;
         P->F = F;
         P->stage = stage;
@@ -524,10 +685,40 @@ __device__ __forceinline__ void group_copy(uint32_t* dst, const uint32_t* src, i
     }
 }
 
+// Packed spins -> one byte per site (no owners) and back, a 32-site word per lane
+// and round, four sites at a time: the products spread a nibble's bits over the
+// bytes of a word and gather them again (no two partial products meet).
+template <int S>
+__device__ __forceinline__ void sites_load(uint8_t* own, const uint32_t* sp, int N, int m)
+{
+    uint32_t* o = reinterpret_cast<uint32_t*>(own);
+#pragma unroll 2
+    for (int w = m; w * 32 < N; w += S) {
+        const uint32_t v = sp[w];
+#pragma unroll
+        for (int b = 0; b < 8; ++b)
+            o[w * 8 + b] = (((((v >> (4 * b)) & 0xFu) * 0x00204081u) & 0x01010101u) << 7) | (kNoOwner * 0x01010101u);
+    }
+}
+
+template <int S>
+__device__ __forceinline__ void sites_store(uint32_t* sp, const uint8_t* own, int N, int m)
+{
+    const uint32_t* o = reinterpret_cast<const uint32_t*>(own);
+    for (int w = m; w * 32 < N; w += S) {
+        uint32_t v = 0u;
+#pragma unroll
+        for (int b = 0; b < 8; ++b)
+            v |= (((((o[w * 8 + b] >> 7) & 0x01010101u) * 0x01020408u) >> 24) & 0xFu) << (4 * b);
+        sp[w] = v;
+    }
+}
+
 // Persistent walker: every group pops lines from the work queue until it is
 // empty.  With one group and a one-entry queue the same kernel is the plain
-// one-launch-per-line form.
-template <int LAT, int S, bool DET, typename IDX, bool TBL>
+// one-launch-per-line form.  A group's slot of shared memory: the list (when
+// staged), the window, the sites, the step records (plan_slot in wl_api.cu).
+template <int LAT, int S, bool DET, typename IDX, bool BYTES>
 __global__ void walk_kernel(const WalkArgs A)
 {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -536,18 +727,14 @@ __global__ void walk_kernel(const WalkArgs A)
     const int gbase = lane - m;
     const unsigned gmask = group_mask<S>(gbase);
     const int gid = threadIdx.x / S;
-    // per-group slot: window, then (when staged) the list and the spins
     uint8_t* slot = smem + (size_t)gid * (size_t)A.slot_bytes;
-    uint8_t* win = slot;
-    slot += kWinBytes;
-    uint32_t* tbl = nullptr;
-    if constexpr (TBL) {
-        // the conflict filter table starts empty and is left empty by every batch
-        tbl = reinterpret_cast<uint32_t*>(slot);
-        const int words = A.tbl_mask + 1;
-        for (int x = m; x < words; x += S) tbl[x] = 0u;
+    int64_t* wl = reinterpret_cast<int64_t*>(slot + A.off_win);
+    static_assert(sizeof(Steps<S>) <= (kStepBytes * S + 15) / 16 * 16, "plan_slot");
+    Steps<S>* steps = reinterpret_cast<Steps<S>*>(slot + A.off_rec);
+    Sites<BYTES> st{slot + A.off_sites, nullptr, (uint32_t)A.owner_mask};
+    if constexpr (!BYTES) {
+        for (int x = m; x <= A.owner_mask; x += S) st.own[x] = (uint8_t)kNoOwner;
         __syncwarp(gmask);
-        slot += (size_t)words * 4;
     }
     // per-line strides are padded to 16 bytes: pstride list entries, W spin words
     const int pstride = A.pstride, W = A.g.W;
@@ -562,21 +749,21 @@ __global__ void walk_kernel(const WalkArgs A)
         if (A.st[li].status != 0) continue;
         IDX* gperm = reinterpret_cast<IDX*>(A.perm) + (size_t)li * pstride;
         uint32_t* gsp = A.spins + (size_t)li * W;
-        if (A.stage_smem) {
-            IDX* sperm = reinterpret_cast<IDX*>(slot);
-            uint32_t* ssp = reinterpret_cast<uint32_t*>(slot + (size_t)perm_words * 4);
-            group_copy<S>(reinterpret_cast<uint32_t*>(sperm), reinterpret_cast<const uint32_t*>(gperm),
+        IDX* perm = gperm;
+        if (A.stage_perm) {
+            perm = reinterpret_cast<IDX*>(slot);
+            group_copy<S>(reinterpret_cast<uint32_t*>(perm), reinterpret_cast<const uint32_t*>(gperm),
                           perm_words, m);
-            group_copy<S>(ssp, gsp, W, m);
-            __syncwarp(gmask);
-            walk_line<LAT, S, DET, IDX, TBL>(A, li, m, gbase, gmask, sperm, ssp, win, tbl);
-            group_copy<S>(reinterpret_cast<uint32_t*>(gperm), reinterpret_cast<const uint32_t*>(sperm),
-                          perm_words, m);
-            group_copy<S>(gsp, ssp, W, m);
-            __syncwarp(gmask);
-        } else {
-            walk_line<LAT, S, DET, IDX, TBL>(A, li, m, gbase, gmask, gperm, gsp, win, tbl);
         }
+        if constexpr (BYTES) sites_load<S>(st.own, gsp, A.g.N, m);
+        else st.sp = gsp;
+        __syncwarp(gmask);
+        walk_line<LAT, S, DET, IDX, BYTES>(A, li, m, gbase, gmask, perm, st, wl, steps);
+        if (A.stage_perm)
+            group_copy<S>(reinterpret_cast<uint32_t*>(gperm), reinterpret_cast<const uint32_t*>(perm),
+                          perm_words, m);
+        if constexpr (BYTES) sites_store<S>(gsp, st.own, A.g.N, m);
+        __syncwarp(gmask);
     }
 }
 

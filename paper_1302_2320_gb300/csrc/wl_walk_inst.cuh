@@ -5,15 +5,13 @@
 #pragma once
 
 #include "wl_kernels.cuh"
-#include "wl_walk.cuh"
+#include "wl_lone.cuh"
 
 namespace wl {
 
-template <int LAT, int S, bool DET, typename IDX, bool TBL>
-cudaError_t walk_one(dim3 grid, dim3 block, size_t smem, cudaStream_t s, const WalkArgs& a,
-                     int* bps)
+inline cudaError_t launch_or_query(void (*fn)(const WalkArgs), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                   const WalkArgs& a, int* bps)
 {
-    auto* fn = walk_kernel<LAT, S, DET, IDX, TBL>;
     // The dynamic shared-memory limit is a property of the kernel function,
     // shared by every handle: raise it to the device maximum (outside stream
     // capture) and never lower it, so a captured launch of one handle stays
@@ -38,20 +36,23 @@ cudaError_t walk_one(dim3 grid, dim3 block, size_t smem, cudaStream_t s, const W
     return cudaGetLastError();
 }
 
-// The conflict-filter form (a.tbl_mask != 0) exists for 32 lanes per walker.
+template <int LAT, int S, bool DET, typename IDX, bool BYTES>
+cudaError_t walk_one(dim3 grid, dim3 block, size_t smem, cudaStream_t s, const WalkArgs& a, int* bps)
+{
+    return launch_or_query(walk_kernel<LAT, S, DET, IDX, BYTES>, grid, block, smem, s, a, bps);
+}
+
+// Sites staged as bytes (a.stage_sites) or left packed in global memory; a list
+// of 32-bit entries belongs to a lattice whose bytes do not fit anyway.
 template <int LAT, int S>
 cudaError_t walk_s(bool det, bool idx16, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                    const WalkArgs& a, int* bps)
 {
-    if (S == 32 && a.tbl_mask != 0) {
-        if (det) {
-            if (idx16) return walk_one<LAT, S, true, uint16_t, true>(grid, block, smem, s, a, bps);
-            return walk_one<LAT, S, true, uint32_t, true>(grid, block, smem, s, a, bps);
-        }
-        if (idx16) return walk_one<LAT, S, false, uint16_t, true>(grid, block, smem, s, a, bps);
-        return walk_one<LAT, S, false, uint32_t, true>(grid, block, smem, s, a, bps);
+    if (a.stage_sites) {
+        if (!idx16) return cudaErrorInvalidValue;
+        if (det) return walk_one<LAT, S, true, uint16_t, true>(grid, block, smem, s, a, bps);
+        return walk_one<LAT, S, false, uint16_t, true>(grid, block, smem, s, a, bps);
     }
-    if (a.tbl_mask != 0) return cudaErrorInvalidValue;
     if (det) {
         if (idx16) return walk_one<LAT, S, true, uint16_t, false>(grid, block, smem, s, a, bps);
         return walk_one<LAT, S, true, uint32_t, false>(grid, block, smem, s, a, bps);
@@ -64,6 +65,10 @@ template <int LAT>
 cudaError_t walk_dispatch(int S, bool det, bool idx16, dim3 grid, dim3 block, size_t smem,
                           cudaStream_t s, const WalkArgs& a, int* bps)
 {
+    if (a.lone) {
+        if (!idx16 || S != 32) return cudaErrorInvalidValue;
+        return launch_or_query(det ? lone_kernel<LAT, true> : lone_kernel<LAT, false>, grid, block, smem, s, a, bps);
+    }
     switch (S) {
     case 1: return walk_s<LAT, 1>(det, idx16, grid, block, smem, s, a, bps);
     case 2: return walk_s<LAT, 2>(det, idx16, grid, block, smem, s, a, bps);
