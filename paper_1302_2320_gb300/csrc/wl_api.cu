@@ -148,8 +148,6 @@ struct TuneRec {
     int best = 0;                          // 0 until every candidate has a rate
 };
 constexpr int kTuneS[3] = {32, 16, 8};
-// Lines per SM up to which each gets a block of its own (plan_shape).
-constexpr int kLonePerSM = 5;
 std::mutex g_tune_mu;
 std::map<TuneKey, TuneRec> g_tune_cache;
 
@@ -241,15 +239,14 @@ wl_status allocate(wl_ctx* h)
 
 Geo make_geo(const wl_ctx* h) { return wl::make_geo(h->g.type, h->g.L, h->g.N, h->g.NB, h->lo.W); }
 
-// The work queue: selected lines by estimated cost (bins^2), largest first.
+// The work queue: selected lines, slowest first.  A slice takes every line the same
+// number of moves further, and a move takes longest where few up spins make
+// neighbouring steps draw the same list slot.
 wl_status upload_queue(wl_ctx* h)
 {
     std::vector<int32_t> order;
     for (int l = h->ell_min; l <= h->ell_max; ++l)
         if (line_selected(h, l)) order.push_back(l);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        return h->lo.desc[a].nbins > h->lo.desc[b].nbins;
-    });
     h->nqueue = (int)order.size();
     CU(cudaMemcpyAsync(h->d_order, order.data(), order.size() * 4, cudaMemcpyHostToDevice, h->s));
     return WL_OK;
@@ -471,8 +468,16 @@ wl_status run_persistent(wl_ctx* h, std::chrono::steady_clock::time_point t_star
         int curS = h->mapping;
         tried = -1;
         const int active = prev_moves < 0 ? h->nqueue : h->h_summary->active;
-        const bool tail = h->tail && (h->mapping == 0 || h->mapping == 32) && active <= kLonePerSM * h->num_sms;
-        if (tail) {
+        // a block per line, where that is the faster shape, needs no tuning
+        Shape sh;
+        wl_status st = WL_OK;
+        bool lone = false;
+        if (h->tail && (h->mapping == 0 || h->mapping == 32)) {
+            st = persistent_shape(h, 32, active, &sh);
+            if (st) return st;
+            lone = sh.slot.lone;
+        }
+        if (lone) {
             curS = 32;
         } else if (curS == 0) {
             std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -483,8 +488,7 @@ wl_status run_persistent(wl_ctx* h, std::chrono::steady_clock::time_point t_star
                 if (tr.rate[c] < 0.0) tried = c;
             curS = tried >= 0 ? kTuneS[tried] : tr.best;
         }
-        Shape sh;
-        wl_status st = persistent_shape(h, curS, h->tail ? active : h->nqueue, &sh);
+        if (!lone) st = persistent_shape(h, curS, h->tail ? active : h->nqueue, &sh);
         if (st) return st;
         if (prev_moves < 0) {
             // moves before this run, for the tuning rates
@@ -688,7 +692,9 @@ static bool plan_lone(const ShapeKey& k, size_t room, Slot* o)
     // the words start at a whole row (cubic: plane), and a list entry holds an address
     const size_t row = 4 * stride * (k.lattice == kCubic ? stride : 1);
     if (4 * (codes + 1) + row > 65536 - 2048) return false;
-    const int min_win = std::min(k.max_bins, 1024);   // two margins of 32 steps and a walk between them
+    // two margins of 32 steps of the largest bin step, and 64 bins to walk between them
+    const int zb = k.lattice == kSquareOpen ? 8 : k.lattice == kTriangular || k.lattice == kCubic ? 6 : 4;
+    const int min_win = std::min(k.max_bins, 64 * zb + 64);
     Slot s;
     s.lone = true;
     size_t at = align16(4 * (codes + 1) + row);
@@ -705,7 +711,14 @@ static bool plan_lone(const ShapeKey& k, size_t room, Slot* o)
     return true;
 }
 
-// One warp per block, 32 / S walkers each.  The shape spreads the walkers over
+// Cycles a move takes its walker (GB300, 64x64): alone, and per walker on the SM where
+// the SM's issue rate is the limit.  A block per line (wl_lone.cuh): 118 alone, ~55
+// instructions on four schedulers; batches (wl_walk.cuh): 150 alone, 269 with 11.8
+// walkers on an SM.
+constexpr double kLoneCycles = 120.0, kLoneIssue = 15.0, kBatchIssue = 23.0;
+
+// Either a block of two warps per line, or one warp per block with 32 / S walkers,
+// whichever takes its walkers less time for a move of all of them.  The shape spreads the walkers over
 // the SMs and gives each the shared memory its share of an SM leaves.  When the
 // walkers do not all fit at once with their lists staged, the lists stay in
 // global memory if that takes fewer rounds: they are read once per batch, so
@@ -725,17 +738,24 @@ wl_status plan_shape(const ShapeKey& k, Shape* sh)
         const int b = std::min(per_block, per_sm / blocks - reserved - 128) / 128 * 128;
         return b > 0 ? (size_t)b : (size_t)0;
     };
-    // few lines: a block each (~45 cycles of issue and ~90 of latency a step, so
-    // several share an SM before the batches of the other kernel are cheaper)
-    const int per = (k.lines + sms - 1) / sms;
-    if (k.lone && per <= kLonePerSM && plan_lone(k, room_of(per), &sh->slot)) {
-        int bps = 0;
-        CU(walk_attrs(k, sh->slot, sh->slot.bytes, 64, &bps));
-        if (bps < 1) return fail(WL_ECUDA, "walker kernel cannot be resident");
-        sh->grid = dim3(k.lines);
-        sh->block = dim3(64);
-        sh->smem = sh->slot.bytes;
-        return WL_OK;
+    double best = 0.0;
+    int best_blocks = 0;
+    // a block per line: as many as fit, each with its share of the shared memory
+    if (k.lone) {
+        int b = std::min((k.lines + sms - 1) / sms, 32), bps = 0;
+        Slot slot;
+        while (b > 0 && !plan_lone(k, room_of(b), &slot)) --b;
+        if (b > 0) CU(walk_attrs(k, slot, slot.bytes, 64, &bps));
+        b = std::min(b, bps);
+        if (b > 0) {
+            const double rounds = (double)((k.lines + sms * b - 1) / (sms * b));
+            best = rounds * std::max(kLoneCycles, kLoneIssue * b);
+            best_blocks = b;
+            plan_lone(k, room_of(b), &sh->slot);
+            sh->grid = dim3(std::min(k.lines, sms * b));
+            sh->block = dim3(64);
+            sh->smem = sh->slot.bytes;
+        }
     }
     auto room = [&](int blocks) {      // bytes per walker with this many blocks on an SM
         const int b = std::min(per_block, per_sm / blocks - reserved) / 128 * 128;
@@ -745,9 +765,7 @@ wl_status plan_shape(const ShapeKey& k, Shape* sh)
         bool sites, perm;
         double cycles;                 // a lone walker's cycles per move, to weigh rounds
     };
-    const Mode modes[3] = {{true, true, 72.0}, {true, false, 84.0}, {false, false, 110.0}};
-    double best = 0.0;
-    int best_blocks = 0;
+    const Mode modes[3] = {{true, true, 150.0}, {true, false, 165.0}, {false, false, 200.0}};
     for (const Mode& m : modes) {
         if (m.sites && !k.idx16) continue;
         int b = want;
@@ -759,18 +777,18 @@ wl_status plan_shape(const ShapeKey& k, Shape* sh)
         b = std::min(b, bps);
         if (b < 1) continue;
         const double rounds = (double)((need + sms * b - 1) / (sms * b));
-        // ~28 warp instructions a move, four schedulers
-        const double cost = rounds * std::max(m.cycles, 7.0 * b);
+        const double cost = rounds * std::max(m.cycles, kBatchIssue * b * groups);
         if (best_blocks == 0 || cost < best) {
-            if (!plan_slot(k, m.sites, m.perm, room(b), &sh->slot)) continue;
+            if (!plan_slot(k, m.sites, m.perm, room(b), &slot)) continue;
             best = cost;
             best_blocks = b;
+            sh->slot = slot;
+            sh->grid = dim3(std::max(1, std::min(need, sms * b)));
+            sh->block = dim3(32);
+            sh->smem = (size_t)groups * slot.bytes;
         }
     }
     if (best_blocks == 0) return fail(WL_ECUDA, "no walker shape fits shared memory (S=%d)", k.S);
-    sh->grid = dim3(std::max(1, std::min(need, sms * best_blocks)));
-    sh->block = dim3(32);
-    sh->smem = (size_t)groups * sh->slot.bytes;
     return WL_OK;
 }
 

@@ -236,13 +236,15 @@ __device__ __forceinline__ void lone_step(Lone& w, const LoneLane<LAT>& L, uint3
         w.u = (p ? gt : w.u) + F;
     };
     if constexpr (WAIT) {
+        // what the next step finds in a slot it shares is known with the decision
         decide();
-        sts64(w.xa, w.u);
-        sts16(r.z, p ? w.oth : w.own);
+        const uint32_t no = p ? w.oth : w.own, nt = p ? w.own : w.oth;
+        w.own1 = s1.x == r.z ? no : w.own1;
+        w.oth1 = s1.y == r.w ? nt : w.oth1;
         reds(w.nb, (p ? L.accept : L.reject) & ~L.ahead);
+        sts16(r.z, no);
+        sts64(w.xa, w.u);
         __syncwarp();
-        w.own1 = lds16(s1.x);
-        w.oth1 = lds16(s1.y);
     }
     const uint32_t wo = lds32(w.own1), wt = lds32(w.oth1);
     const uint32_t own2 = lds16(w.slots.x), oth2 = lds16(w.slots.y);
@@ -276,35 +278,45 @@ __device__ __forceinline__ void lone_step(Lone& w, const LoneLane<LAT>& L, uint3
     __syncwarp();
 }
 
-// K steps without a wait flag.
-template <int LAT, int K>
+template <int LAT, int K, bool WAIT>
 __device__ __forceinline__ void lone_block(Lone& w, const LoneLane<LAT>& L, uint32_t& at, int64_t F)
 {
 #pragma unroll
-    for (int q = 0; q < K; ++q) lone_step<LAT, false>(w, L, at + 32u * q, F);
+    for (int q = 0; q < K; ++q) lone_step<LAT, WAIT>(w, L, at + 32u * q, F);
     at += 32u * K;
 }
 
-// Take n <= 32 steps, from the record at `at` on; waits: their wait flags.  Steps
-// without one go eight at a time: the end of a loop's body costs ~75 cycles here (a
-// step 97), so a body of one step takes 182 cycles a step, of two 143, of four 115,
-// of eight 106 (64x64, l = 2048).
+// Take n <= 32 steps, from the record at `at` on; waits: their wait flags (any step
+// may wait).  The end of a loop's body costs ~75 cycles here (the compiler lets the
+// loops of a kernel yield whose warps part before a barrier), and so do the turns
+// between the two kinds of step.  So steps without a flag go eight at a time
+// (64x64, l = 2048: 182 cycles a step one at a time, 143 two, 115 four, 106 eight),
+// and where flags are many (few up spins, a tiny lattice) all steps wait, four at a
+// time.
+constexpr int kManyWaits = 6;
+
 template <int LAT>
 __device__ __forceinline__ void lone_run(Lone& w, const LoneLane<LAT>& L, uint32_t at, int n, uint32_t waits, int64_t F)
 {
+    if (__popc(waits) >= kManyWaits) {
+#pragma unroll 1
+        for (; n >= 4; n -= 4) lone_block<LAT, 4, true>(w, L, at, F);
+#pragma unroll 1
+        for (; n > 0; --n) lone_block<LAT, 1, true>(w, L, at, F);
+        return;
+    }
     for (;;) {
         const int clear = waits ? __ffs((int)waits) - 1 : 32;      // steps before the next flag
         int k = clear < n ? clear : n;
         n -= k;
         waits = clear < 31 ? waits >> (clear + 1) : 0u;
 #pragma unroll 1
-        for (; k >= 8; k -= 8) lone_block<LAT, 8>(w, L, at, F);
-        if (k & 4) lone_block<LAT, 4>(w, L, at, F);
-        if (k & 2) lone_block<LAT, 2>(w, L, at, F);
-        if (k & 1) lone_block<LAT, 1>(w, L, at, F);
+        for (; k >= 8; k -= 8) lone_block<LAT, 8, false>(w, L, at, F);
+        if (k & 4) lone_block<LAT, 4, false>(w, L, at, F);
+        if (k & 2) lone_block<LAT, 2, false>(w, L, at, F);
+        if (k & 1) lone_block<LAT, 1, false>(w, L, at, F);
         if (n == 0) break;
-        lone_step<LAT, true>(w, L, at, F);
-        at += 32u;
+        lone_block<LAT, 1, true>(w, L, at, F);
         n -= 1;
         if (n == 0) break;
     }
@@ -545,7 +557,15 @@ __global__ void __launch_bounds__(kLoneThreads) lone_kernel(const WalkArgs A)
     uint16_t* perm = reinterpret_cast<uint16_t*>(smem + A.off_perm);
     uint4* ring = reinterpret_cast<uint4*>(smem + A.off_rec);
     uint32_t* waits = reinterpret_cast<uint32_t*>(ring + 2 * (kRing + kRingMore));
-    int32_t* ctl = reinterpret_cast<int32_t*>(waits + 4);         // the line; the walker is done
+    int32_t* ctl = reinterpret_cast<int32_t*>(waits + 4);         // the line; the walker is done; who walks
+    if (th == 0) {
+        // The SM deals its warps out to four schedulers in order of their slots: were
+        // it always the first warp of a block that walks, all walkers would share two
+        // of them.  Any choice is right; this one spreads them over all four.
+        uint32_t slot;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
+        ctl[2] = (int32_t)((slot >> 2) & 1u);
+    }
     const int N = A.g.N, pstride = A.pstride;
     for (;;) {
         if (th == 0) {
@@ -578,7 +598,7 @@ __global__ void __launch_bounds__(kLoneThreads) lone_kernel(const WalkArgs A)
             const int64_t t = A.st[li].t;
             const int ell = A.desc[li].ell;
             __syncthreads();
-            if (warp == 0)
+            if (warp == ctl[2])
                 lone_walk<LAT>(A, li, lane, smem, ring, waits, words_at, words_at + 4u * codes, ctl + 1);
             else
                 lone_draw<DET>(A, t, ell, ring, waits, (uint32_t)__cvta_generic_to_shared(perm), ctl + 1, lane);

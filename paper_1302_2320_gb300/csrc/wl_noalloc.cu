@@ -184,8 +184,6 @@ extern "C" wl_status wl_walk_noalloc(wl_lattice lattice, int L, int ell_first, i
         max_bins = std::max(max_bins, g_desc[i].nbins);
         g_order[i] = i;
     }
-    std::stable_sort(g_order, g_order + nlines,
-                     [&](int a, int b) { return g_desc[a].nbins > g_desc[b].nbins; });
     NCU(cudaMemcpyAsync(d_desc, g_desc, nlines * sizeof(LineDesc), cudaMemcpyHostToDevice, s));
     NCU(cudaMemcpyAsync(d_order, g_order, nlines * 4, cudaMemcpyHostToDevice, s));
     // control words start at zero on every call

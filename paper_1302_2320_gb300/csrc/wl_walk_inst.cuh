@@ -28,6 +28,10 @@ inline cudaError_t launch_or_query(void (*fn)(const WalkArgs), dim3 grid, dim3 b
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      optin > (int)smem ? optin : (int)smem);
+        // one split of an SM's memory for every walker kernel: a kernel that asks for
+        // another one waits until the SM is empty, and handles no longer overlap
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
     }
     if (bps) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, fn, (int)block.x, smem);
