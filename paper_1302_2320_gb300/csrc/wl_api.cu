@@ -177,6 +177,8 @@ void free_all(wl_ctx* h)
     if (h->ev1) cudaEventDestroy(h->ev1);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->ev_t0) cudaEventDestroy(h->ev_t0);
+    if (h->ev_i0) cudaEventDestroy(h->ev_i0);
+    if (h->ev_i1) cudaEventDestroy(h->ev_i1);
     if (h->ev_t1) cudaEventDestroy(h->ev_t1);
     if (h->s) cudaStreamDestroy(h->s);
     h->allocated = false;
@@ -196,6 +198,8 @@ wl_status allocate(wl_ctx* h)
     CU(cudaEventCreate(&h->ev1));
     CU(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
     CU(cudaEventCreate(&h->ev_t0));
+    CU(cudaEventCreate(&h->ev_i0));
+    CU(cudaEventCreate(&h->ev_i1));
     CU(cudaEventCreate(&h->ev_t1));
     const Layout& lo = h->lo;
     const size_t isz = lo.idx16 ? 2 : 4;
@@ -252,73 +256,75 @@ wl_status upload_queue(wl_ctx* h)
     return WL_OK;
 }
 
-wl_status initialise(wl_ctx* h, double u, int flat_pm)
+// The exp threshold table of ln f_min = u on the device, kept while u stays the same:
+// the host's own build of it, in the long double that is software on the machines
+// this GPU comes with, takes 2 ms, as long as a small walk.
+wl_status exp_table(wl_ctx* h, double u)
 {
-    const int q = host_table_q(u);
-    if (q < 0) return fail(WL_EINVAL, "ln_f_min %g out of range", u);
-    CU(launch_exp_table(u, q, h->d_table64, h->s));
-    h->table64.assign(kTableN, 0);
-    CU(cudaMemcpyAsync(h->table64.data(), h->d_table64, kTableN * 8, cudaMemcpyDeviceToHost, h->s));
-    CU(cudaStreamSynchronize(h->s));
-    std::vector<uint64_t> ref;
-    host_table(u, q, ref);
-    if (h->det) {
+    if (h->table_u != u) {
+        const int q = host_table_q(u);
+        if (q < 0) return fail(WL_EINVAL, "ln_f_min %g out of range", u);
+        h->table_u = 0.0;
+        h->table_checked = false;
+        CU(launch_exp_table(u, q, h->d_table64, h->s));
+        h->table64.assign(kTableN, 0);
+        CU(cudaMemcpyAsync(h->table64.data(), h->d_table64, kTableN * 8, cudaMemcpyDeviceToHost, h->s));
+        CU(cudaStreamSynchronize(h->s));
+        std::vector<uint32_t> t32(kTableN);
+        t32[0] = 0xFFFFFFFFu;   // entry 0 (2^32) is implicit in the kernel
+        for (int i = 1; i < kTableN; ++i) t32[i] = (uint32_t)h->table64[i];
+        CU(cudaMemcpyAsync(h->d_table, t32.data(), kTableN * 4, cudaMemcpyHostToDevice, h->s));
+        h->table_u = u;
+        h->q = q;
+    }
+    if (h->det && !h->table_checked) {
+        std::vector<uint64_t> ref;
+        host_table(u, h->q, ref);
         for (int i = 0; i < kTableN; ++i)
             if (ref[i] != h->table64[i])
                 return fail(WL_EMISMATCH, "exp table entry %d: device %llu host %llu", i,
                             (unsigned long long)h->table64[i], (unsigned long long)ref[i]);
+        h->table_checked = true;
     }
-    std::vector<uint32_t> t32(kTableN);
-    t32[0] = 0xFFFFFFFFu;   // entry 0 (2^32) is implicit in the kernel
-    for (int i = 1; i < kTableN; ++i) t32[i] = (uint32_t)h->table64[i];
-    CU(cudaMemcpyAsync(h->d_table, t32.data(), kTableN * 4, cudaMemcpyHostToDevice, h->s));
-    wl_status st = upload_queue(h);
-    if (st) return st;
-    CU(cudaMemsetAsync(h->d_flags, 0, 16, h->s));
-    CU(cudaMemsetAsync(h->d_st, 0, h->lo.nlines * sizeof(LineState), h->s));
-    // lines outside [ell_min, ell_max], or not in a selected set, are marked
-    // converged with t = 0 so that no launch touches them
+    return WL_OK;
+}
+
+InitArgs init_args(const wl_ctx* h, double u)
+{
     InitArgs a;
     a.g = make_geo(h);
-    a.desc = h->d_desc + h->ell_min;
-    a.st = h->d_st + h->ell_min;
-    a.perm = (uint8_t*)h->d_perm + (size_t)h->ell_min * h->lo.pstride * (h->lo.idx16 ? 2 : 4);
-    a.spins = h->d_spins + (size_t)h->ell_min * h->lo.W;
+    a.desc = h->d_desc;
+    a.st = h->d_st;
+    a.perm = h->d_perm;
+    a.spins = h->d_spins;
     a.lng = h->d_lng;
     a.hist = h->d_hist;
     a.pstride = h->lo.pstride;
-    a.nlines = h->ell_max - h->ell_min + 1;
+    a.nlines = h->nqueue;
     a.seed = h->seed;
     a.F0 = std::llround(1.0 / u);
-    CU(cudaEventRecord(h->ev0, h->s));
-    CU(launch_init(h->g.type == WL_SQUARE_OPEN ? (int)kSquareOpen : h->g.type, h->lo.idx16, a, h->s));
-    CU(cudaEventRecord(h->ev1, h->s));
-    {
-        std::vector<LineState> out(h->lo.nlines);
-        for (auto& s : out) {
-            memset(&s, 0, sizeof s);
-            s.status = 1;
-        }
-        // runs of lines that are not walked
-        for (int l = 0; l < h->lo.nlines;) {
-            if (line_selected(h, l)) {
-                ++l;
-                continue;
-            }
-            int e = l;
-            while (e < h->lo.nlines && !line_selected(h, e)) ++e;
-            CU(cudaMemcpyAsync(h->d_st + l, out.data(), (size_t)(e - l) * sizeof(LineState),
-                               cudaMemcpyHostToDevice, h->s));
-            l = e;
-        }
-    }
-    CU(cudaStreamSynchronize(h->s));
-    float ms = 0;
-    CU(cudaEventElapsedTime(&ms, h->ev0, h->ev1));
-    h->init_ms = ms;
+    a.order = h->d_order;
+    return a;
+}
+
+int init_lattice(const wl_ctx* h) { return h->g.type == WL_SQUARE_OPEN ? (int)kSquareOpen : h->g.type; }
+
+wl_status initialise(wl_ctx* h, double u, int flat_pm)
+{
+    wl_status st = exp_table(h, u);
+    if (st) return st;
+    st = upload_queue(h);
+    if (st) return st;
+    CU(cudaMemsetAsync(h->d_flags, 0, 16, h->s));
+    // lines outside [ell_min, ell_max], or not in a selected set, are marked
+    // converged with t = 0 so that no launch touches them
+    CU(launch_blank_states(h->d_st, h->lo.nlines, h->s));
+    const InitArgs a = init_args(h, u);
+    CU(cudaEventRecord(h->ev_i0, h->s));
+    CU(launch_init(init_lattice(h), h->lo.idx16, a, h->s));
+    CU(cudaEventRecord(h->ev_i1, h->s));
     h->u = u;
     h->flat_pm = flat_pm;
-    h->q = q;
     h->initialized = true;
     h->assembled = false;
     return WL_OK;
@@ -490,7 +496,9 @@ wl_status run_persistent(wl_ctx* h, std::chrono::steady_clock::time_point t_star
         }
         if (!lone) st = persistent_shape(h, curS, h->tail ? active : h->nqueue, &sh);
         if (st) return st;
-        if (prev_moves < 0) {
+        if (prev_moves < 0 && (lone || h->mapping != 0)) {
+            prev_moves = 0;           // nothing is tuned
+        } else if (prev_moves < 0) {
             // moves before this run, for the tuning rates
             CU(launch_summary(h->d_st, h->lo.nlines, h->budget, h->d_flags, h->d_summary, h->s));
             CU(cudaMemcpyAsync(h->h_summary, h->d_summary, sizeof(Summary), cudaMemcpyDeviceToHost, h->s));
@@ -819,8 +827,7 @@ wl_status assemble_copy_async(wl_ctx* h, double* dst, size_t cap, size_t* n_out)
     const size_t n = (size_t)(b.bin_off + b.nbins - a.bin_off);
     if (n_out) *n_out = n;
     if (!dst || cap < n) return fail(WL_EINVAL, "output capacity %zu < %zu bins", cap, n);
-    CU(launch_assemble(h->d_desc + h->ell_min, h->d_lng, h->d_hist, h->g.N,
-                       h->ell_max - h->ell_min + 1, h->u, h->d_out, h->s));
+    CU(launch_assemble(h->d_desc, h->d_order, h->d_lng, h->d_hist, h->g.N, h->nqueue, h->u, h->d_out, h->s));
     CU(cudaMemcpyAsync(dst, h->d_out + a.bin_off, n * 8, cudaMemcpyDeviceToHost, h->s));
     h->assembled = true;
     return WL_OK;
@@ -1061,8 +1068,7 @@ wl_status wl_assemble(wl_handle h)
         CU(cudaStreamWaitEvent(h->s, h->ev_join, 0));
     }
     CU(cudaEventRecord(h->ev0, h->s));
-    CU(launch_assemble(h->d_desc + h->ell_min, h->d_lng, h->d_hist, h->g.N,
-                       h->ell_max - h->ell_min + 1, h->u, h->d_out, h->s));
+    CU(launch_assemble(h->d_desc, h->d_order, h->d_lng, h->d_hist, h->g.N, h->nqueue, h->u, h->d_out, h->s));
     CU(cudaEventRecord(h->ev1, h->s));
     if (h->has_user_stream) {
         CU(cudaEventRecord(h->ev_join, h->s));
@@ -1110,6 +1116,11 @@ wl_status wl_get_surface(wl_handle h, double* out, size_t cap, int64_t* offsets,
         for (int l = 0; l < lines; ++l) offsets[l] = h->lo.desc[h->ell_min + l].bin_off - a.bin_off;
         offsets[lines] = n;
     }
+    if (!h->sel.empty()) {
+        // the lines between those of the set
+        CU(launch_fill_unvisited(h->d_out + a.bin_off, (size_t)n, h->s));
+        CU(launch_assemble(h->d_desc, h->d_order, h->d_lng, h->d_hist, h->g.N, h->nqueue, h->u, h->d_out, h->s));
+    }
     CU(cudaMemcpyAsync(out, h->d_out + a.bin_off, (size_t)n * 8, cudaMemcpyDeviceToHost, h->s));
     CU(cudaStreamSynchronize(h->s));
     return WL_OK;
@@ -1124,8 +1135,12 @@ wl_status wl_get_stats(wl_handle h, wl_stats* out)
     out->form = h->form;
     out->launches = h->launches;
     out->walk_ms = h->walk_ms;
-    out->init_ms = h->init_ms;
     out->assemble_ms = h->assemble_ms;
+    if (h->allocated && cudaEventSynchronize(h->ev_i1) == cudaSuccess) {
+        float ms = 0;
+        if (cudaEventElapsedTime(&ms, h->ev_i0, h->ev_i1) == cudaSuccess) out->init_ms = ms;
+        clear_stale_error();          // events not recorded yet
+    }
     if (!h->initialized) return WL_OK;
     std::vector<LineState> st(h->lo.nlines);
     CU(cudaMemcpyAsync(st.data(), h->d_st, st.size() * sizeof(LineState), cudaMemcpyDeviceToHost, h->s));
@@ -1153,6 +1168,14 @@ wl_status wl_get_line_state(wl_handle h, int ell, int64_t* scal, int32_t* perm, 
     if (ell < 0 || ell >= h->lo.nlines) return fail(WL_EINVAL, "ell must be in [0, N/2]");
     const LineDesc& d = h->lo.desc[ell];
     const int N = h->g.N;
+    if (ell >= h->ell_min && ell <= h->ell_max && !line_selected(h, ell)) {
+        // between the lines of a set: not walked, and initialised only when asked for
+        InitArgs a = init_args(h, h->u);
+        a.st = nullptr;
+        a.order = h->d_ident + ell;
+        a.nlines = 1;
+        CU(launch_init(init_lattice(h), h->lo.idx16, a, h->s));
+    }
     if (scal) {
         LineState s;
         CU(cudaMemcpyAsync(&s, h->d_st + ell, sizeof s, cudaMemcpyDeviceToHost, h->s));

@@ -14,17 +14,20 @@ namespace wl {
 // counter (t, 0, 1, 0), key (l, seed)); U = perm[0, l), D = perm[l, N); ln g = 0,
 // h = 0, ln f = 1 (F0 = round(1/u)); k0 counted from the spins.  The line l = 0
 // has no exchange move: its single bin k = 0 is marked visited and it is done.
+// The shuffle is a chain of l dependent swaps: it runs in shared memory where the
+// list fits (A.stage; ~45 cycles a swap against ~600 from global memory: the four
+// lines of the 256x256 lattice take 1.1 ms), one line per block of one warp.
 // ---------------------------------------------------------------------------
 template <int LAT, typename IDX>
-__global__ void init_kernel(const InitArgs A)
+__global__ void __launch_bounds__(32) init_kernel(const InitArgs A)
 {
-    const int warps = blockDim.x >> 5;
-    const int li = blockIdx.x * warps + (threadIdx.x >> 5);
+    extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31;
-    if (li >= A.nlines) return;
+    const int li = A.order ? A.order[blockIdx.x] : (int)blockIdx.x;
     const LineDesc D = A.desc[li];
     const int N = A.g.N, W = A.g.W, ell = D.ell;
-    IDX* perm = reinterpret_cast<IDX*>(A.perm) + (size_t)li * A.pstride;
+    IDX* gperm = reinterpret_cast<IDX*>(A.perm) + (size_t)li * A.pstride;
+    IDX* perm = A.stage ? reinterpret_cast<IDX*>(smem) : gperm;
     uint32_t* sp = A.spins + (size_t)li * W;
     int64_t* lng = A.lng + D.bin_off;
     hist_t* hist = A.hist + D.bin_off;
@@ -55,6 +58,8 @@ __global__ void init_kernel(const InitArgs A)
         }
         __syncwarp();
     }
+    if (A.stage)
+        for (int n = lane; n < A.pstride; n += 32) gperm[n] = perm[n];
     for (int a = lane; a < ell; a += 32) {
         const uint32_t n = (uint32_t)perm[a];
         atomicOr(&sp[n >> 5], 1u << (n & 31u));
@@ -73,7 +78,7 @@ __global__ void init_kernel(const InitArgs A)
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) twice += __shfl_xor_sync(0xffffffffu, twice, off);
-    if (lane == 0) {
+    if (lane == 0 && A.st) {
         LineState s;
         s.k = twice / 2;
         s.t = 0;
@@ -159,24 +164,46 @@ cudaError_t launch_check_state(int lattice, bool idx16, const InitArgs& a, int32
     return cudaGetLastError();
 }
 
+template <int LAT, typename IDX>
+static cudaError_t init_one(InitArgs a, cudaStream_t s)
+{
+    // up to 64 KB of list per block, or the whole of an SM's shared memory for a line
+    const size_t list = (size_t)a.pstride * sizeof(IDX);
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    a.stage = list <= (size_t)optin;
+    if (a.stage && list > 48 * 1024) {
+        e = cudaFuncSetAttribute(init_kernel<LAT, IDX>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+        if (e != cudaSuccess) return e;
+    }
+    init_kernel<LAT, IDX><<<a.nlines, 32, a.stage ? list : 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_init(int lattice, bool idx16, const InitArgs& a, cudaStream_t s)
 {
     clear_stale_error();
-    const int warps = 4;
-    const dim3 grid((a.nlines + warps - 1) / warps), block(32 * warps);
-    if (lattice == kSquare) {
-        if (idx16) init_kernel<kSquare, uint16_t><<<grid, block, 0, s>>>(a);
-        else init_kernel<kSquare, uint32_t><<<grid, block, 0, s>>>(a);
-    } else if (lattice == kTriangular) {
-        if (idx16) init_kernel<kTriangular, uint16_t><<<grid, block, 0, s>>>(a);
-        else init_kernel<kTriangular, uint32_t><<<grid, block, 0, s>>>(a);
-    } else if (lattice == kCubic) {
-        if (idx16) init_kernel<kCubic, uint16_t><<<grid, block, 0, s>>>(a);
-        else init_kernel<kCubic, uint32_t><<<grid, block, 0, s>>>(a);
-    } else {
-        if (idx16) init_kernel<kSquareOpen, uint16_t><<<grid, block, 0, s>>>(a);
-        else init_kernel<kSquareOpen, uint32_t><<<grid, block, 0, s>>>(a);
-    }
+    if (a.nlines < 1) return cudaSuccess;
+    if (lattice == kSquare) return idx16 ? init_one<kSquare, uint16_t>(a, s) : init_one<kSquare, uint32_t>(a, s);
+    if (lattice == kTriangular)
+        return idx16 ? init_one<kTriangular, uint16_t>(a, s) : init_one<kTriangular, uint32_t>(a, s);
+    if (lattice == kCubic) return idx16 ? init_one<kCubic, uint16_t>(a, s) : init_one<kCubic, uint32_t>(a, s);
+    return idx16 ? init_one<kSquareOpen, uint16_t>(a, s) : init_one<kSquareOpen, uint32_t>(a, s);
+}
+
+// Line states of lines that are not walked: converged, with no move made.
+__global__ void blank_states_kernel(LineState* st, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) st[i] = LineState{0, 0, 0, 0, 0, 0, 1, 0, 0};
+}
+
+cudaError_t launch_blank_states(LineState* st, int n, cudaStream_t s)
+{
+    clear_stale_error();
+    blank_states_kernel<<<(n + 255) / 256, 256, 0, s>>>(st, n);
     return cudaGetLastError();
 }
 
@@ -185,13 +212,14 @@ cudaError_t launch_init(int lattice, bool idx16, const InitArgs& a, cudaStream_t
 //   ln g_kl = ln C(N,l) + u lng[b] - (M + ln sum_visited exp(u lng[b] - M)),
 // M the visited maximum; unvisited bins get -inf.  FP64.
 // ---------------------------------------------------------------------------
-__global__ void assemble_kernel(const LineDesc* desc, const int64_t* lng, const hist_t* hist,
+__global__ void assemble_kernel(const LineDesc* desc, const int32_t* order, const int64_t* lng, const hist_t* hist,
                                 int N, int nlines, double u, double* out)
 {
     const int warps = blockDim.x >> 5;
-    const int li = blockIdx.x * warps + (threadIdx.x >> 5);
+    const int x = blockIdx.x * warps + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    if (li >= nlines) return;
+    if (x >= nlines) return;
+    const int li = order[x];
     const LineDesc D = desc[li];
     const int64_t* lg = lng + D.bin_off;
     const hist_t* h = hist + D.bin_off;
@@ -213,13 +241,25 @@ __global__ void assemble_kernel(const LineDesc* desc, const int64_t* lng, const 
         o[b] = (h[b] & kVisited) ? lnC + u * (double)lg[b] - lse : -INFINITY;
 }
 
-cudaError_t launch_assemble(const LineDesc* desc, const int64_t* lng, const hist_t* hist, int N,
+cudaError_t launch_assemble(const LineDesc* desc, const int32_t* order, const int64_t* lng, const hist_t* hist, int N,
                             int nlines, double u, double* out, cudaStream_t s)
 {
     clear_stale_error();
     const int warps = 8;
-    assemble_kernel<<<(nlines + warps - 1) / warps, 32 * warps, 0, s>>>(desc, lng, hist, N, nlines,
-                                                                       u, out);
+    assemble_kernel<<<(nlines + warps - 1) / warps, 32 * warps, 0, s>>>(desc, order, lng, hist, N, nlines, u, out);
+    return cudaGetLastError();
+}
+
+__global__ void fill_unvisited_kernel(double* out, size_t n)
+{
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        out[i] = -INFINITY;
+}
+
+cudaError_t launch_fill_unvisited(double* out, size_t n, cudaStream_t s)
+{
+    clear_stale_error();
+    fill_unvisited_kernel<<<1216, 256, 0, s>>>(out, n);
     return cudaGetLastError();
 }
 

@@ -21,6 +21,8 @@ struct InitArgs {
     int32_t nlines;
     uint32_t seed;
     int64_t F0;
+    const int32_t* order = nullptr;   // the lines to initialise (null: 0 .. nlines - 1)
+    int32_t stage = 0;                // set by launch_init: the list fits shared memory
 };
 
 struct Summary {
@@ -55,8 +57,11 @@ cudaError_t launch_walk_square_open(int S, bool det, bool idx16, dim3 grid, dim3
 
 cudaError_t launch_init(int lattice, bool idx16, const InitArgs& a, cudaStream_t s);
 cudaError_t launch_check_state(int lattice, bool idx16, const InitArgs& a, int32_t* flags, cudaStream_t s);
-cudaError_t launch_assemble(const LineDesc* desc, const int64_t* lng, const hist_t* hist, int N,
+cudaError_t launch_blank_states(LineState* st, int n, cudaStream_t s);
+// Assemble the lines order[0 .. nlines); fill n entries with -inf (no bin visited).
+cudaError_t launch_assemble(const LineDesc* desc, const int32_t* order, const int64_t* lng, const hist_t* hist, int N,
                             int nlines, double u, double* out, cudaStream_t s);
+cudaError_t launch_fill_unvisited(double* out, size_t n, cudaStream_t s);
 cudaError_t launch_exp_table(double u, int q, uint64_t* out, cudaStream_t s);
 cudaError_t launch_philox(size_t n, const uint32_t* ctr, const uint32_t* key, uint32_t* out,
                           cudaStream_t s);

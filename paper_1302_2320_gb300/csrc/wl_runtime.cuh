@@ -83,13 +83,14 @@ struct wl_ctx {
     int q = 0;
     int last_mapping = 0;
     int64_t launches = 0;
-    double walk_ms = 0, init_ms = 0, assemble_ms = 0;
+    double walk_ms = 0, assemble_ms = 0;
     int64_t init_moves = 0;
     // device
     int device = 0, num_sms = 0;
     cudaStream_t s = nullptr;
     std::vector<cudaStream_t> pool;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_join = nullptr;
+    cudaEvent_t ev_i0 = nullptr, ev_i1 = nullptr;   // around the initialisation
     cudaEvent_t ev_t0 = nullptr, ev_t1 = nullptr;   // one slice, for the lane-count tuner
     wl::LineDesc* d_desc = nullptr;
     wl::LineState* d_st = nullptr;
@@ -110,6 +111,8 @@ struct wl_ctx {
     int32_t* h_abort = nullptr;           // pinned, mapped
     int32_t* d_abort = nullptr;
     std::vector<uint64_t> table64;        // device-built table, copied back
+    double table_u = 0.0;                 // the ln f_min it is for (0: none)
+    bool table_checked = false;           // equal to the host's own build of it
     int nqueue = 0;
     // captured slice graph
     cudaGraphExec_t graph = nullptr;
