@@ -18,7 +18,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libwl.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
-SOURCES = ["wl_api.cu", "wl_kernels.cu", "wl_walk_square.cu", "wl_walk_square_p2.cu",
+SOURCES = ["wl_api.cu", "wl_lone.cu", "wl_kernels.cu", "wl_walk_square.cu", "wl_walk_square_p2.cu",
            "wl_walk_triangular.cu", "wl_walk_cubic.cu", "wl_noalloc.cu",
            "wl_server.cu", "wl_walk_square_open.cu", "wl_probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -241,7 +241,7 @@ wl_status allocate(wl_ctx* h)
     return WL_OK;
 }
 
-Geo make_geo(const wl_ctx* h) { return wl::make_geo(h->g.type, h->g.L, h->g.N, h->g.NB, h->lo.W); }
+Geo make_geo(const wl_ctx* h) { return wl::make_geo(h->g.type, (LatticeShape)h->g.type, h->g.L, h->g.N, h->g.NB, h->lo.W); }
 
 // The work queue: selected lines, slowest first.  A slice takes every line the same
 // number of moves further, and a move takes longest where few up spins make
@@ -686,26 +686,28 @@ static cudaError_t walk_attrs(const ShapeKey& k, const Slot& slot, size_t smem, 
 {
     WalkArgs a{};
     set_slot(slot, &a);
+    a.g.shape = k.lattice == kTriangular ? kShapeTriangular : kShapeSquare;      // picks the kernel
     return walk_kernel_attrs(k.lattice, k.S, k.det, k.idx16, smem, threads, a, bps);
 }
 
 // The slot of a line with a block of its own (wl_lone.cuh): the words of the sites
-// by code and one more, the list, the window, the ring.
+// by code, the list, the window, the ring.
 static bool plan_lone(const ShapeKey& k, size_t room, Slot* o)
 {
     if (!k.idx16) return false;
+    const bool open = k.lattice == kSquareOpen;      // with a border around it
     size_t stride = 1;
-    while (stride < (size_t)k.L) stride <<= 1;
-    const size_t codes = k.lattice == kCubic ? stride * stride * k.L : stride * k.L;
+    while (stride < (size_t)k.L + (open ? 1 : 0)) stride <<= 1;
+    const size_t codes = (k.lattice == kCubic ? stride : 1) * stride * ((size_t)k.L + (open ? 2 : 0));
     // the words start at a whole row (cubic: plane), and a list entry holds an address
     const size_t row = 4 * stride * (k.lattice == kCubic ? stride : 1);
-    if (4 * (codes + 1) + row > 65536 - 2048) return false;
+    if (4 * codes + row > 65536 - 2048) return false;
     // two margins of 32 steps of the largest bin step, and 64 bins to walk between them
     const int zb = k.lattice == kSquareOpen ? 8 : k.lattice == kTriangular || k.lattice == kCubic ? 6 : 4;
     const int min_win = std::min(k.max_bins, 64 * zb + 64);
     Slot s;
     s.lone = true;
-    size_t at = align16(4 * (codes + 1) + row);
+    size_t at = align16(4 * codes + row);
     s.off_perm = (int)at;
     at += (size_t)k.pstride * 2;
     s.off_win = (int)at;

@@ -41,20 +41,25 @@ struct LineDesc {
     int32_t nbins;     // bins k = 0, 2, ..., 2*(nbins-1)
 };
 
+// A lattice at run time, whatever its kernel specialisation.
+enum LatticeShape : int { kShapeSquare = 0, kShapeTriangular = 1, kShapeCubic = 2, kShapeOpen = 3 };
+
 struct Geo {
     int type, L, N, NB, W;   // W = 32-bit words of packed spins per line (multiple of 4)
     uint64_t magic;          // ceil(2^40 / L): x / L == (x * magic) >> 40 for x < 2^24
     int lshift;              // log2(L) when L is a power of two
     uint32_t lmask;          // L - 1 when L is a power of two
-    int cshift;              // site codes (wl_lone.cuh): L rounded up to a power of two is 1 << cshift
+    int shape;               // LatticeShape
+    int cshift;              // site codes (wl_lone.cuh): rows of 1 << cshift, L (open: L + 1) rounded up
     uint32_t cmask;          // (1 << cshift) - 1
 };
 
 // The geometry of an L lattice of N sites, W spin words per line.
-inline Geo make_geo(int type, int L, int N, int NB, int W)
+inline Geo make_geo(int type, LatticeShape shape, int L, int N, int NB, int W)
 {
     Geo g{};
     g.type = type;
+    g.shape = shape;
     g.L = L;
     g.N = N;
     g.NB = NB;
@@ -62,7 +67,7 @@ inline Geo make_geo(int type, int L, int N, int NB, int W)
     g.magic = (((uint64_t)1 << 40) + (uint64_t)L - 1) / (uint64_t)L;
     while ((1 << (g.lshift + 1)) <= L) ++g.lshift;
     g.lmask = (uint32_t)L - 1u;
-    while ((1 << g.cshift) < L) ++g.cshift;
+    while ((1 << g.cshift) < L + (shape == kShapeOpen ? 1 : 0)) ++g.cshift;
     g.cmask = (1u << g.cshift) - 1u;
     return g;
 }

@@ -602,6 +602,7 @@ cudaError_t launch_set_deadline(uint64_t* deadline, uint64_t timeout_ns, cudaStr
 cudaError_t launch_walk(int lattice, int S, bool det, bool idx16, dim3 grid, dim3 block,
                         size_t smem, cudaStream_t s, const WalkArgs& a)
 {
+    if (a.lone) return idx16 ? launch_lone(det, grid, block, smem, s, a, nullptr) : cudaErrorInvalidValue;
     if (lattice == kSquare) return launch_walk_square(S, det, idx16, grid, block, smem, s, a, nullptr);
     if (lattice == kSquareP2)
         return launch_walk_square_p2(S, det, idx16, grid, block, smem, s, a, nullptr);
@@ -616,6 +617,7 @@ cudaError_t walk_kernel_attrs(int lattice, int S, bool det, bool idx16, size_t s
                               const WalkArgs& a, int* blocks_per_sm)
 {
     const dim3 z(0), b(block_threads);
+    if (a.lone) return idx16 ? launch_lone(det, z, b, smem, 0, a, blocks_per_sm) : cudaErrorInvalidValue;
     if (lattice == kSquare) return launch_walk_square(S, det, idx16, z, b, smem, 0, a, blocks_per_sm);
     if (lattice == kSquareP2)
         return launch_walk_square_p2(S, det, idx16, z, b, smem, 0, a, blocks_per_sm);

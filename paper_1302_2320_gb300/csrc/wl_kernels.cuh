@@ -44,6 +44,9 @@ cudaError_t launch_walk(int lattice, int S, bool det, bool idx16, dim3 grid, dim
 cudaError_t walk_kernel_attrs(int lattice, int S, bool det, bool idx16, size_t smem, int block_threads,
                               const WalkArgs& a, int* blocks_per_sm);
 
+// The block-per-line walker (a.lone): one code for all lattices with 16-bit lists.
+cudaError_t launch_lone(bool det, dim3 grid, dim3 block, size_t smem, cudaStream_t s, const WalkArgs& a, int* bps);
+
 cudaError_t launch_walk_square(int S, bool det, bool idx16, dim3 grid, dim3 block, size_t smem,
                                cudaStream_t s, const WalkArgs& a, int* bps);
 cudaError_t launch_walk_triangular(int S, bool det, bool idx16, dim3 grid, dim3 block, size_t smem,

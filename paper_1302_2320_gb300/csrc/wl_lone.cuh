@@ -41,36 +41,48 @@ constexpr int kRing = 128;                 // steps (4 batches of 32)
 constexpr int kRingMore = 3;               // the first records again past the end: a step reads up to 3 ahead
 constexpr int kLoneThreads = 64;           // one warp walks, one draws
 
-template <int LAT>
+// The lattice is a run-time matter but for the second axis of the triangular one's
+// diagonals (TRI): requests for different lattices that share an SM then run the same
+// code, and do not drive each other's out of its instruction cache (eight requests of
+// five lattices: 121 ms with a kernel for each lattice, each 26 ms alone).
 __device__ __forceinline__ uint32_t site_code(const Geo& g, uint32_t n)
 {
-    if constexpr (LAT == kSquareP2) {
-        return n;
-    } else {
-        const uint32_t L = (uint32_t)g.L, r = divL(g, n), x = n - r * L;
-        if constexpr (LAT == kCubic) {
-            const uint32_t z = divL(g, r), y = r - z * L;
-            return (((z << g.cshift) | y) << g.cshift) | x;
-        } else {
-            return (r << g.cshift) | x;
-        }
+    const uint32_t L = (uint32_t)g.L, r = divL(g, n), x = n - r * L;
+    if (g.shape == kShapeCubic) {
+        const uint32_t z = divL(g, r), y = r - z * L;
+        return (((z << g.cshift) | y) << g.cshift) | x;
     }
+    return ((r + (g.shape == kShapeOpen ? 1u : 0u)) << g.cshift) | x;
 }
 
-template <int LAT>
 __device__ __forceinline__ uint32_t code_site(const Geo& g, uint32_t c)
 {
-    if constexpr (LAT == kSquareP2) {
-        return c;
-    } else {
-        const uint32_t L = (uint32_t)g.L, x = c & g.cmask;
-        if constexpr (LAT == kCubic) {
-            const uint32_t y = (c >> g.cshift) & g.cmask, z = c >> (2 * g.cshift);
-            return (z * L + y) * L + x;
-        } else {
-            return (c >> g.cshift) * L + x;
-        }
+    const uint32_t L = (uint32_t)g.L, x = c & g.cmask;
+    if (g.shape == kShapeCubic) {
+        const uint32_t y = (c >> g.cshift) & g.cmask, z = c >> (2 * g.cshift);
+        return (z * L + y) * L + x;
     }
+    return ((c >> g.cshift) - (g.shape == kShapeOpen ? 1u : 0u)) * L + x;
+}
+
+// 8 for every up neighbour of site n (open boundaries: 16, less 8 for every neighbour).
+template <int LAT>
+__device__ __forceinline__ uint32_t site_word(const Geo& g, const uint32_t* sp, uint32_t n)
+{
+    constexpr int z = Coord<LAT>::z;
+    uint32_t nb[z];
+    int u = 0;
+    if constexpr (LAT == kSquareOpen) {
+        const unsigned v = open_neighbours(g, n, nb);
+#pragma unroll
+        for (int q = 0; q < z; ++q) u += (int)((v >> q) & 1u & spin_at(sp, nb[q]));
+        u = 2 * u - __popc(v);
+    } else {
+        neighbours<LAT>(g, n, nb);
+#pragma unroll
+        for (int q = 0; q < z; ++q) u += (int)spin_at(sp, nb[q]);
+    }
+    return (uint32_t)(8 * u);
 }
 
 // Shared memory by 32-bit address (generic pointers cost 64-bit address arithmetic).
@@ -120,6 +132,9 @@ __device__ __forceinline__ void reds(uint32_t a, uint32_t v)
 
 __device__ __forceinline__ void lone_barrier() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
 
+constexpr uint32_t kBias = 128u;            // keeps the two halves of a difference of words apart
+constexpr uint32_t kBoth = 0x10001u;        // a number in both halves
+
 // The lanes of the walking warp.  Lane q < z stands for neighbour q of the pending
 // step's up site, lane z + q for neighbour q of its down site; the next 2z lanes
 // stand for the neighbours of the step after it in the same way, so that one
@@ -127,30 +142,35 @@ __device__ __forceinline__ void lone_barrier() { asm volatile("bar.sync 1, 64;" 
 // lanes past those go along, so that no step branches: they load and store the
 // same, and each has a word of its own in the place of a neighbour's; the first of
 // them counts the accepted steps in its.
-template <int LAT>
+//
+// A word holds 8 for every up neighbour, the bytes of one bin of ln g: half the change
+// of k.  With open boundaries bins are half as wide, and a word holds 16 for every up
+// neighbour less 8 for every neighbour; a missing neighbour is a word of the border
+// around the lattice, which nobody reads.
+template <bool TRI>
 struct LoneLane {
-    static constexpr int z = Coord<LAT>::z;
-    // A word holds 8 for every up neighbour, the bytes of one bin of ln g: half the
-    // change of k.  With open boundaries bins are half as wide, and a word holds 16 for
-    // every up neighbour less 8 for every neighbour.
-    static constexpr uint32_t kUnit = LAT == kSquareOpen ? 16u : 8u;
-    static constexpr int kCounter = 4 * z;   // the lane that counts
     uint32_t swap;                   // 16 for the lanes of the down site: their order in a ring record
     int32_t sign;                    // own word less the other's, as up less down
     uint32_t ahead;                  // all ones in the lanes of the step after the pending one
     uint32_t accept, reject;         // what the decision adds to this lane's word
     uint32_t next;                   // what becoming the pending step adds to it
     uint32_t scale;                  // 0 for a lane without a neighbour
+    uint32_t apart, touching;        // bias of a difference whose sites are not, are neighbours
     uint32_t s0, m0, e0, d0, w0;     // along one axis: shift, mask, coordinate at the edge, step, step at the edge
     uint32_t s1, m1, e1, d1, w1;     // along the other (triangular diagonals)
 
-    __device__ __forceinline__ void setup(const Geo& g, int lane, uint32_t words, uint32_t none, uint32_t spare)
+    __device__ __forceinline__ void setup(const Geo& g, int lane, uint32_t words, uint32_t spare)
     {
+        const int z = g.shape == kShapeTriangular || g.shape == kShapeCubic ? 6 : 4;
+        const bool open = g.shape == kShapeOpen;
+        const uint32_t unit = open ? 16u : 8u;
         const int q = lane % z;
         const bool down = ((lane / z) & 1) != 0;
         swap = down ? 16u : 0u;
         sign = down ? -1 : 1;
-        const uint32_t delta = down ? kUnit : 0u - kUnit;    // the up site goes, the down site comes
+        apart = kBias * kBoth;
+        touching = (kBias + unit) * kBoth;
+        const uint32_t delta = down ? unit : 0u - unit;    // the up site goes, the down site comes
         ahead = lane >= 2 * z && lane < 4 * z ? 0xFFFFFFFFu : 0u;
         next = ahead & (delta << 16);
         accept = ahead ? next : delta;
@@ -160,26 +180,25 @@ struct LoneLane {
             s = (uint32_t)(ax * g.cshift) + 2u;
             const uint32_t u = 1u << s;
             // the outermost coordinate is what is left of the address, base and all
-            const bool outer = ax == (LAT == kCubic ? 2 : 1);
+            const bool outer = ax == (g.shape == kShapeCubic ? 2 : 1);
             mk = outer ? 0xFFFFFFFFu : g.cmask;
             ed = (plus ? e : 0u) + (outer ? words >> s : 0u);
             d = plus ? u : 0u - u;
-            w = plus ? 0u - e * u : e * u;
+            w = open ? d : plus ? 0u - e * u : e * u;
         };
         // neighbours in the order of neighbours<LAT>: +-x, +-y, (+-z | the diagonals)
         s1 = m1 = d1 = w1 = 0u;
         e1 = 1u;
-        if (LAT == kTriangular && q >= 4) {
+        if (TRI && q >= 4) {
             axis(0, q == 4, s0, m0, e0, d0, w0);
             axis(1, q == 5, s1, m1, e1, d1, w1);
         } else {
             axis(q >> 1, (q & 1) == 0, s0, m0, e0, d0, w0);
         }
-        if (LAT == kSquareOpen) w0 = none;       // an address, not a step
         scale = 1u;
         if (lane >= 4 * z) {
             scale = d1 = w1 = reject = 0u;
-            accept = lane == kCounter ? 1u : 0u;
+            accept = lane == 4 * z ? 1u : 0u;
             d0 = w0 = spare + 4u * (uint32_t)lane;
         }
     }
@@ -187,11 +206,11 @@ struct LoneLane {
     // Address of the word of this lane's neighbour of the site at c.
     __device__ __forceinline__ uint32_t neighbour(uint32_t c) const
     {
-        const bool w = ((c >> s0) & m0) == e0;
-        uint32_t n = (w ? w0 : d0) + c * (LAT == kSquareOpen && w ? 0u : scale);
-        if constexpr (LAT == kTriangular) n += ((c >> s1) & m1) == e1 ? w1 : d1;
+        uint32_t n = (((c >> s0) & m0) == e0 ? w0 : d0) + c * scale;
+        if constexpr (TRI) n += ((c >> s1) & m1) == e1 ? w1 : d1;
         return n;
     }
+    __device__ __forceinline__ uint32_t bias(bool adjacent) const { return adjacent ? touching : apart; }
 };
 
 // A walker's state: the pending step (this lane's own site and the other one, the
@@ -208,22 +227,13 @@ struct Lone {
     uint2 slots;            // of the step after next: own, other
 };
 
-constexpr uint32_t kBias = 128u;            // keeps the two halves of a difference of words apart
-constexpr uint32_t kBoth = 0x10001u;        // a number in both halves
-
-template <int LAT>
-__device__ __forceinline__ uint32_t lone_bias(bool adjacent)
-{
-    return adjacent ? (kBias + LoneLane<LAT>::kUnit) * kBoth : kBias * kBoth;
-}
-
 // One step: decide the pending one, evaluate the next, load the one after.
 // `at`: the pending step's record in the ring, in this lane's order.  WAIT: the next
 // step or the one after it shares a list slot with the pending one.  The loads come
 // before the stores as far as they may: the compiler keeps their order, and a load
 // that waits behind a store waits for the decision.
-template <int LAT, bool WAIT>
-__device__ __forceinline__ void lone_step(Lone& w, const LoneLane<LAT>& L, uint32_t at, int64_t F)
+template <bool TRI, bool WAIT>
+__device__ __forceinline__ void lone_step(Lone& w, const LoneLane<TRI>& L, uint32_t at, int64_t F)
 {
     const int64_t gt = lds64(w.ta);
     const uint4 r = lds128(at);
@@ -252,7 +262,7 @@ __device__ __forceinline__ void lone_step(Lone& w, const LoneLane<LAT>& L, uint3
     __syncwarp();
     if constexpr (WAIT) {
         const uint32_t n1 = L.neighbour(w.own1);
-        w.bias = lone_bias<LAT>(__any_sync(0xffffffffu, n1 == w.oth1));
+        w.bias = L.bias(__any_sync(0xffffffffu, n1 == w.oth1));
         reds(n1, L.next);
     }
     // the change of k as bytes of ln g, in both halves
@@ -260,7 +270,7 @@ __device__ __forceinline__ void lone_step(Lone& w, const LoneLane<LAT>& L, uint3
     // the lanes ahead take the step after next, the others the next; only the
     // former see whether its sites are neighbours
     const uint32_t nb = L.neighbour(L.ahead ? own2 : w.own1);
-    const uint32_t bias = lone_bias<LAT>(__any_sync(0xffffffffu, nb == (oth2 & L.ahead)));
+    const uint32_t bias = L.bias(__any_sync(0xffffffffu, nb == (oth2 & L.ahead)));
     if constexpr (!WAIT) {
         decide();
         sts64(w.xa, w.u);
@@ -278,11 +288,11 @@ __device__ __forceinline__ void lone_step(Lone& w, const LoneLane<LAT>& L, uint3
     __syncwarp();
 }
 
-template <int LAT, int K, bool WAIT>
-__device__ __forceinline__ void lone_block(Lone& w, const LoneLane<LAT>& L, uint32_t& at, int64_t F)
+template <bool TRI, int K, bool WAIT>
+__device__ __forceinline__ void lone_block(Lone& w, const LoneLane<TRI>& L, uint32_t& at, int64_t F)
 {
 #pragma unroll
-    for (int q = 0; q < K; ++q) lone_step<LAT, WAIT>(w, L, at + 32u * q, F);
+    for (int q = 0; q < K; ++q) lone_step<TRI, WAIT>(w, L, at + 32u * q, F);
     at += 32u * K;
 }
 
@@ -295,14 +305,14 @@ __device__ __forceinline__ void lone_block(Lone& w, const LoneLane<LAT>& L, uint
 // time.
 constexpr int kManyWaits = 6;
 
-template <int LAT>
-__device__ __forceinline__ void lone_run(Lone& w, const LoneLane<LAT>& L, uint32_t at, int n, uint32_t waits, int64_t F)
+template <bool TRI>
+__device__ __forceinline__ void lone_run(Lone& w, const LoneLane<TRI>& L, uint32_t at, int n, uint32_t waits, int64_t F)
 {
     if (__popc(waits) >= kManyWaits) {
 #pragma unroll 1
-        for (; n >= 4; n -= 4) lone_block<LAT, 4, true>(w, L, at, F);
+        for (; n >= 4; n -= 4) lone_block<TRI, 4, true>(w, L, at, F);
 #pragma unroll 1
-        for (; n > 0; --n) lone_block<LAT, 1, true>(w, L, at, F);
+        for (; n > 0; --n) lone_block<TRI, 1, true>(w, L, at, F);
         return;
     }
     for (;;) {
@@ -311,12 +321,12 @@ __device__ __forceinline__ void lone_run(Lone& w, const LoneLane<LAT>& L, uint32
         n -= k;
         waits = clear < 31 ? waits >> (clear + 1) : 0u;
 #pragma unroll 1
-        for (; k >= 8; k -= 8) lone_block<LAT, 8, false>(w, L, at, F);
-        if (k & 4) lone_block<LAT, 4, false>(w, L, at, F);
-        if (k & 2) lone_block<LAT, 2, false>(w, L, at, F);
-        if (k & 1) lone_block<LAT, 1, false>(w, L, at, F);
+        for (; k >= 8; k -= 8) lone_block<TRI, 8, false>(w, L, at, F);
+        if (k & 4) lone_block<TRI, 4, false>(w, L, at, F);
+        if (k & 2) lone_block<TRI, 2, false>(w, L, at, F);
+        if (k & 1) lone_block<TRI, 1, false>(w, L, at, F);
         if (n == 0) break;
-        lone_block<LAT, 1, true>(w, L, at, F);
+        lone_block<TRI, 1, true>(w, L, at, F);
         n -= 1;
         if (n == 0) break;
     }
@@ -373,13 +383,14 @@ __device__ __forceinline__ void lone_draw(const WalkArgs& A, int64_t t, int ell,
 
 // The walking warp: line `li` for up to A.slice_moves moves (or to its budget, or
 // to convergence); the bookkeeping between steps as in walk_line.
-template <int LAT>
+template <bool TRI>
 __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint8_t* sm, const uint4* ring, const uint32_t* waits,
-                                          uint32_t words, uint32_t none, volatile int32_t* done)
+                                          uint32_t words, uint32_t* spare, volatile int32_t* done)
 {
-    constexpr int zb = Coord<LAT>::zbin;
-    constexpr int ks = Coord<LAT>::kshift;
-    constexpr int kMargin = 32 * zb;         // a run of steps stays inside the window
+    const bool open = A.g.shape == kShapeOpen;
+    const int ks = open ? 0 : 1;
+    const int zb = open ? 8 : A.g.shape == kShapeTriangular || A.g.shape == kShapeCubic ? 6 : 4;    // Coord::zbin
+    const int kMargin = 32 * zb;         // a run of steps stays inside the window
     constexpr unsigned all = 0xffffffffu;
     const LineDesc D = A.desc[li];
     LineState* P = A.st + li;
@@ -406,10 +417,10 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
     window_load<32>(wl, lng, wb, wn, m);
     __syncwarp(all);
     const uint32_t wa = (uint32_t)__cvta_generic_to_shared(wl);
-    LoneLane<LAT> L;
-    L.setup(A.g, m, words, none, (uint32_t)__cvta_generic_to_shared((void*)(done + 3)));
+    LoneLane<TRI> L;
+    L.setup(A.g, m, words, (uint32_t)__cvta_generic_to_shared(spare));
     const uint32_t ring_at = (uint32_t)__cvta_generic_to_shared(ring) + L.swap;
-    uint32_t* counter = reinterpret_cast<uint32_t*>(const_cast<int32_t*>(done + 3)) + LoneLane<LAT>::kCounter;
+    uint32_t* counter = spare + (zb == 6 ? 24 : 16);      // the first lane past the neighbours
     Lone w{};
     w.xa = wa + 8u * (uint32_t)(bc - wb);
     w.u = wl[bc - wb];
@@ -426,9 +437,9 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
         w.slots = lds64u(ring_at + 72u);
         const uint32_t n0 = L.neighbour(w.own), n1 = L.neighbour(w.own1);
         const uint32_t d = (uint32_t)((int32_t)(lds32(w.own) - lds32(w.oth)) * L.sign) +
-                           lone_bias<LAT>(__any_sync(all, n0 == w.oth));
+                           L.bias(__any_sync(all, n0 == w.oth));
         w.ta = w.xa + (d & 0xFFFFu) - kBias;
-        w.bias = lone_bias<LAT>(__any_sync(all, n1 == w.oth1));
+        w.bias = L.bias(__any_sync(all, n1 == w.oth1));
         w.nb = L.ahead ? n1 : n0;
         __syncwarp(all);
         reds(n0, L.next);
@@ -445,7 +456,7 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
             const uint32_t lo = wb > 0 ? wa + 8u * kMargin : wa;
             const uint32_t hi = wa + 8u * (uint32_t)(wn - 1 - (wb + wn < nbins ? kMargin : 0));
             const uint32_t wm = (waits[k & 3u] >> 2) | (waits[(k + 1u) & 3u] << 30);
-            lone_run<LAT>(w, L, ring_at + 32u * (pos & (kRing - 1)), n, wm >> (pos & 31u), F);
+            lone_run<TRI>(w, L, ring_at + 32u * (pos & (kRing - 1)), n, wm >> (pos & 31u), F);
             __syncwarp(all);
             const uint32_t xa = w.xa;
             bc = wb + ((int)(xa - wa) >> 3);
@@ -542,17 +553,15 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
 
 // One block per line: shared memory holds the words of the sites (and one more), the
 // list, the window, the ring of draws.
-template <int LAT, bool DET>
+template <bool TRI, bool DET>
 __global__ void __launch_bounds__(kLoneThreads) lone_kernel(const WalkArgs A)
 {
     extern __shared__ __align__(16) uint8_t smem[];
-    constexpr int z = Coord<LAT>::z;
     const int th = threadIdx.x, warp = th >> 5, lane = th & 31;
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
     // the words start at a whole row (cubic: plane) of addresses
-    const uint32_t row = 4u << (LAT == kCubic ? 2 * A.g.cshift : A.g.cshift);
+    const uint32_t row = 4u << (A.g.shape == kShapeCubic ? 2 * A.g.cshift : A.g.cshift);
     const uint32_t words_at = (base + row - 1u) / row * row;
-    const uint32_t codes = (uint32_t)A.g.L << (LAT == kCubic ? 2 * A.g.cshift : A.g.cshift);
     uint32_t* words = reinterpret_cast<uint32_t*>(smem + (words_at - base));
     uint16_t* perm = reinterpret_cast<uint16_t*>(smem + A.off_perm);
     uint4* ring = reinterpret_cast<uint4*>(smem + A.off_rec);
@@ -566,6 +575,7 @@ __global__ void __launch_bounds__(kLoneThreads) lone_kernel(const WalkArgs A)
         asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
         ctl[2] = (int32_t)((slot >> 2) & 1u);
     }
+    uint32_t* spare = reinterpret_cast<uint32_t*>(ctl + 4);
     const int N = A.g.N, pstride = A.pstride;
     for (;;) {
         if (th == 0) {
@@ -580,26 +590,18 @@ __global__ void __launch_bounds__(kLoneThreads) lone_kernel(const WalkArgs A)
             uint16_t* gperm = reinterpret_cast<uint16_t*>(A.perm) + (size_t)li * pstride;
             uint32_t* gsp = A.spins + (size_t)li * A.g.W;
             for (int n = th; n < N; n += kLoneThreads) {
-                perm[n] = (uint16_t)(words_at + 4u * site_code<LAT>(A.g, gperm[n]));
-                uint32_t nb[z];
-                int u = 0;
-                if constexpr (LAT == kSquareOpen) {
-                    const unsigned v = open_neighbours(A.g, (uint32_t)n, nb);
-#pragma unroll
-                    for (int q = 0; q < z; ++q) u += (int)((v >> q) & 1u & spin_at(gsp, nb[q]));
-                    u = 2 * u - __popc(v);
-                } else {
-                    neighbours<LAT>(A.g, (uint32_t)n, nb);
-#pragma unroll
-                    for (int q = 0; q < z; ++q) u += (int)spin_at(gsp, nb[q]);
-                }
-                words[site_code<LAT>(A.g, (uint32_t)n)] = (uint32_t)(8 * u) * kBoth;
+                perm[n] = (uint16_t)(words_at + 4u * site_code(A.g, gperm[n]));
+                const uint32_t u = A.g.shape == kShapeTriangular ? site_word<kTriangular>(A.g, gsp, (uint32_t)n)
+                                   : A.g.shape == kShapeCubic    ? site_word<kCubic>(A.g, gsp, (uint32_t)n)
+                                   : A.g.shape == kShapeOpen     ? site_word<kSquareOpen>(A.g, gsp, (uint32_t)n)
+                                                                 : site_word<kSquare>(A.g, gsp, (uint32_t)n);
+                words[site_code(A.g, (uint32_t)n)] = u * kBoth;
             }
             const int64_t t = A.st[li].t;
             const int ell = A.desc[li].ell;
             __syncthreads();
             if (warp == ctl[2])
-                lone_walk<LAT>(A, li, lane, smem, ring, waits, words_at, words_at + 4u * codes, ctl + 1);
+                lone_walk<TRI>(A, li, lane, smem, ring, waits, words_at, spare, ctl + 1);
             else
                 lone_draw<DET>(A, t, ell, ring, waits, (uint32_t)__cvta_generic_to_shared(perm), ctl + 1, lane);
             __syncthreads();
@@ -607,7 +609,7 @@ __global__ void __launch_bounds__(kLoneThreads) lone_kernel(const WalkArgs A)
             for (int x = th; x * 32 < N; x += kLoneThreads) words[x] = 0u;
             __syncthreads();
             for (int n = th; n < N; n += kLoneThreads) {
-                const uint32_t s = code_site<LAT>(A.g, (perm[n] - words_at) >> 2);
+                const uint32_t s = code_site(A.g, (perm[n] - words_at) >> 2);
                 gperm[n] = (uint16_t)s;
                 if (n < ell) atomicOr(&words[s >> 5], 1u << (s & 31u));
             }

@@ -204,7 +204,7 @@ extern "C" wl_status wl_walk_noalloc(wl_lattice lattice, int L, int ell_first, i
     // pageable host -> device copies have taken the data once they return
     stage_lock.unlock();
 
-    const Geo g = make_geo((int)lattice, L, N, NB, W);
+    const Geo g = make_geo((int)lattice, (LatticeShape)(int)lattice, L, N, NB, W);
     const int klat = (lattice == WL_SQUARE && (L & (L - 1)) == 0) ? (int)kSquareP2 : (int)lattice;
     LineState* d_st = reinterpret_cast<LineState*>(state);
 
