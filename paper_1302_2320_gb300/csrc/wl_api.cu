@@ -166,7 +166,7 @@ void free_all(wl_ctx* h)
     h->graph = nullptr;
     void* ptrs[] = {h->d_desc, h->d_st, h->d_perm, h->d_spins, h->d_lng, h->d_hist, h->d_out,
                     h->d_table, h->d_table64, h->d_order, h->d_ident, h->d_qheads, h->d_flags,
-                    h->d_deadline, h->d_summary};
+                    h->d_deadline, h->d_summary, h->d_thermo};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (h->h_summary) cudaFreeHost(h->h_summary);
@@ -1227,15 +1227,23 @@ wl_status wl_thermo(wl_handle h, const double* T, int nT, const double* H, int n
     for (int a = 0; a < nT; ++a)
         if (!(T[a] > 0.0)) return fail(WL_EINVAL, "temperatures must be > 0");
     const size_t nd = (size_t)nT + (size_t)nH + 6 * (size_t)nT * (size_t)nH;
-    double* d = nullptr;
-    CU(cudaMallocAsync(&d, nd * sizeof(double), h->s));
+    const size_t need = nd * sizeof(double) + thermo_scratch_bytes(h->lo.nlines, nT);
+    // the workspace is kept with the handle: to map and unmap it on every call takes
+    // longer than a scan of a small surface
+    if (h->thermo_bytes < need) {
+        if (h->d_thermo) CU(cudaFree(h->d_thermo));
+        h->d_thermo = nullptr;
+        h->thermo_bytes = 0;
+        CU(cudaMalloc(&h->d_thermo, need));
+        h->thermo_bytes = need;
+    }
+    double* d = static_cast<double*>(h->d_thermo);
     cudaError_t e = cudaMemcpyAsync(d, T, nT * sizeof(double), cudaMemcpyHostToDevice, h->s);
     if (!e) e = cudaMemcpyAsync(d + nT, H, nH * sizeof(double), cudaMemcpyHostToDevice, h->s);
     if (!e) e = launch_thermo(h->d_desc, h->lo.nlines, h->d_out, h->g.N, h->g.NB, h->g.kstep, d, nT,
-                              d + nT, nH, d + nT + nH, h->s);
+                              d + nT, nH, d + nT + nH, d + nd, h->s);
     if (!e) e = cudaMemcpyAsync(out, d + nT + nH, 6 * (size_t)nT * nH * sizeof(double),
                                 cudaMemcpyDeviceToHost, h->s);
-    cudaFreeAsync(d, h->s);
     if (!e) e = cudaStreamSynchronize(h->s);
     if (e) return fail(WL_ECUDA, "wl_thermo: %s", cudaGetErrorString(e));
     return WL_OK;

@@ -75,6 +75,7 @@ cudaError_t launch_summary(const LineState* st, int nlines, int64_t budget, cons
 cudaError_t launch_set_deadline(uint64_t* deadline, uint64_t timeout_ns, cudaStream_t s);
 cudaError_t launch_thermo(const LineDesc* desc, int nlines, const double* lng, int N, int NB,
                           int kstep, const double* T, int nT, const double* H, int nH, double* out,
-                          cudaStream_t s);
+                          void* scratch, cudaStream_t s);
+size_t thermo_scratch_bytes(int nlines, int nT);
 
 }  // namespace wl

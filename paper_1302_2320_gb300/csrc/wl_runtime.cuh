@@ -107,6 +107,8 @@ struct wl_ctx {
     int32_t* d_flags = nullptr;
     uint64_t* d_deadline = nullptr;
     wl::Summary* d_summary = nullptr;
+    void* d_thermo = nullptr;             // workspace of wl_thermo, from its first call on
+    size_t thermo_bytes = 0;
     wl::Summary* h_summary = nullptr;         // pinned
     int32_t* h_abort = nullptr;           // pinned, mapped
     int32_t* d_abort = nullptr;
