@@ -721,11 +721,12 @@ static bool plan_lone(const ShapeKey& k, size_t room, Slot* o)
     return true;
 }
 
-// Cycles a move takes its walker (GB300, 64x64): alone, and per walker on the SM where
-// the SM's issue rate is the limit.  A block per line (wl_lone.cuh): 118 alone, ~55
-// instructions on four schedulers; batches (wl_walk.cuh): 150 alone, 269 with 11.8
-// walkers on an SM.
-constexpr double kLoneCycles = 120.0, kLoneIssue = 15.0, kBatchIssue = 23.0;
+// Cycles a move takes its walker, alone, and per walker on an SM where they get in each
+// other's way (GB300).  A block per line (wl_lone.cuh): 116 alone, 155 with 7 on an SM
+// (64x64).  Batches (wl_walk.cuh): 191 with 7 on an SM and the lists staged (96x96),
+// 272 with 16 on an SM and the lists in global memory (96x96) or 12 and staged (64x64);
+// but lines of few up spins, whose batches keep running into themselves, 500.
+constexpr double kLoneCycles = 120.0, kLoneIssue = 22.0, kBatchIssue = 17.0, kBatchSlowest = 500.0;
 
 // Either a block of two warps per line, or one warp per block with 32 / S walkers,
 // whichever takes its walkers less time for a move of all of them.  The shape spreads the walkers over
@@ -775,7 +776,7 @@ wl_status plan_shape(const ShapeKey& k, Shape* sh)
         bool sites, perm;
         double cycles;                 // a lone walker's cycles per move, to weigh rounds
     };
-    const Mode modes[3] = {{true, true, 150.0}, {true, false, 165.0}, {false, false, 200.0}};
+    const Mode modes[3] = {{true, true, 190.0}, {true, false, 200.0}, {false, false, 250.0}};
     for (const Mode& m : modes) {
         if (m.sites && !k.idx16) continue;
         int b = want;
@@ -787,7 +788,7 @@ wl_status plan_shape(const ShapeKey& k, Shape* sh)
         b = std::min(b, bps);
         if (b < 1) continue;
         const double rounds = (double)((need + sms * b - 1) / (sms * b));
-        const double cost = rounds * std::max(m.cycles, kBatchIssue * b * groups);
+        const double cost = std::max(rounds * std::max(m.cycles, kBatchIssue * b * groups), kBatchSlowest);
         if (best_blocks == 0 || cost < best) {
             if (!plan_slot(k, m.sites, m.perm, room(b), &slot)) continue;
             best = cost;

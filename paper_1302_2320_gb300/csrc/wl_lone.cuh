@@ -154,6 +154,7 @@ struct LoneLane {
     uint32_t ahead;                  // all ones in the lanes of the step after the pending one
     uint32_t accept, reject;         // what the decision adds to this lane's word
     uint32_t next;                   // what becoming the pending step adds to it
+    uint32_t both;                   // what an accepted step adds where nothing is pending
     uint32_t scale;                  // 0 for a lane without a neighbour
     uint32_t apart, touching;        // bias of a difference whose sites are not, are neighbours
     uint32_t s0, m0, e0, d0, w0;     // along one axis: shift, mask, coordinate at the edge, step, step at the edge
@@ -175,6 +176,7 @@ struct LoneLane {
         next = ahead & (delta << 16);
         accept = ahead ? next : delta;
         reject = ahead ? next : 0u - (delta << 16);
+        both = ahead ? 0u : delta * kBoth;
         const uint32_t e = (uint32_t)g.L - 1u;
         auto axis = [&](int ax, bool plus, uint32_t& s, uint32_t& mk, uint32_t& ed, uint32_t& d, uint32_t& w) {
             s = (uint32_t)(ax * g.cshift) + 2u;
@@ -198,7 +200,7 @@ struct LoneLane {
         scale = 1u;
         if (lane >= 4 * z) {
             scale = d1 = w1 = reject = 0u;
-            accept = lane == 4 * z ? 1u : 0u;
+            accept = both = lane == 4 * z ? 1u : 0u;
             d0 = w0 = spare + 4u * (uint32_t)lane;
         }
     }
@@ -296,23 +298,85 @@ __device__ __forceinline__ void lone_block(Lone& w, const LoneLane<TRI>& L, uint
     at += 32u * K;
 }
 
-// Take n <= 32 steps, from the record at `at` on; waits: their wait flags (any step
-// may wait).  The end of a loop's body costs ~75 cycles here (the compiler lets the
-// loops of a kernel yield whose warps part before a barrier), and so do the turns
-// between the two kinds of step.  So steps without a flag go eight at a time
-// (64x64, l = 2048: 182 cycles a step one at a time, 143 two, 115 four, 106 eight),
-// and where flags are many (few up spins, a tiny lattice) all steps wait, four at a
-// time.
-constexpr int kManyWaits = 6;
+// One step where most would wait: decided, written back, and only then the next one
+// evaluated.  Nothing is pending in the words (their halves are the same), so an
+// accepted step needs one reduction and the next but one is not looked at ahead.
+template <bool TRI>
+__device__ __forceinline__ void dense_step(Lone& w, const LoneLane<TRI>& L, uint32_t at, int64_t F)
+{
+    const int64_t gt = lds64(w.ta);
+    const uint4 r = lds128(at);
+    const uint2 s1 = lds64u(at + 40u);
+    const bool p = gt <= w.u + (int64_t)(((uint64_t)r.y << 32) | r.x);
+    // what the next step finds in a slot it shares is known with the decision
+    const uint32_t no = p ? w.oth : w.own, nt = p ? w.own : w.oth;
+    w.own = s1.x == r.z ? no : w.own1;
+    w.oth = s1.y == r.w ? nt : w.oth1;
+    reds(w.nb, p ? L.both : 0u);
+    w.xa = p ? w.ta : w.xa;
+    w.u = (p ? gt : w.u) + F;
+    sts16(r.z, no);
+    sts64(w.xa, w.u);
+    __syncwarp();
+    const uint32_t wo = lds32(w.own), wt = lds32(w.oth);
+    w.own1 = lds16(w.slots.x);
+    w.oth1 = lds16(w.slots.y);
+    w.slots = lds64u(at + 104u);
+    __syncwarp();
+    w.nb = L.neighbour(w.own);
+    const uint32_t bias = L.bias(__any_sync(0xffffffffu, w.nb == w.oth));
+    const uint32_t d = (uint32_t)((int32_t)(wo - wt) * L.sign) + bias;
+    w.ta = w.xa + (d & 0xFFFFu) - kBias;
+}
+
+// Between the two ways: the pending step's changes leave the words' high halves, or
+// enter them (and the step after it is looked at).
+template <bool TRI>
+__device__ __forceinline__ void to_dense(Lone& w, const LoneLane<TRI>& L)
+{
+    reds(w.nb, L.reject & ~L.ahead);
+    __syncwarp();
+}
+template <bool TRI>
+__device__ __forceinline__ void from_dense(Lone& w, const LoneLane<TRI>& L)
+{
+    const uint32_t n1 = L.neighbour(w.own1);
+    w.bias = L.bias(__any_sync(0xffffffffu, n1 == w.oth1));
+    reds(w.nb, 0u - (L.reject & ~L.ahead));
+    w.nb = L.ahead ? n1 : w.nb;
+    __syncwarp();
+}
+
+// Take n <= 32 steps, from the record at `at` on; waits: their wait flags.  The end of
+// a loop's body costs ~75 cycles here (the compiler lets the loops of a kernel yield
+// whose warps part before a barrier), and so do the turns between two kinds of step.
+// So steps go in blocks: 64x64, l = 2048, takes 182 cycles a step one at a time, 143
+// two, 115 four, 106 eight.  A flagged step among others costs ~350 cycles; from
+// three in a batch on (few up spins, a tiny lattice) all steps go the dense way.
+constexpr int kToDense = 3, kFromDense = 1;
 
 template <bool TRI>
-__device__ __forceinline__ void lone_run(Lone& w, const LoneLane<TRI>& L, uint32_t at, int n, uint32_t waits, int64_t F)
+__device__ __forceinline__ void lone_run(Lone& w, const LoneLane<TRI>& L, bool& dense, uint32_t at, int n, uint32_t waits,
+                                         int64_t F)
 {
-    if (__popc(waits) >= kManyWaits) {
+    const int flags = __popc(waits);
+    if (dense ? flags <= kFromDense : flags >= kToDense) {
+        dense = !dense;
+        if (dense) to_dense<TRI>(w, L);
+        else from_dense<TRI>(w, L);
+    }
+    if (dense) {
 #pragma unroll 1
-        for (; n >= 4; n -= 4) lone_block<TRI, 4, true>(w, L, at, F);
+        for (; n >= 8; n -= 8) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) dense_step<TRI>(w, L, at + 32u * q, F);
+            at += 256u;
+        }
 #pragma unroll 1
-        for (; n > 0; --n) lone_block<TRI, 1, true>(w, L, at, F);
+        for (; n > 0; --n) {
+            dense_step<TRI>(w, L, at, F);
+            at += 32u;
+        }
         return;
     }
     for (;;) {
@@ -446,6 +510,7 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
     }
     __syncwarp(all);
 
+    bool dense = false;
     while (t < end && !stop) {
         const int64_t next_check = (t / C + 1) * C;
         const int64_t seg_end = next_check < end ? next_check : end;
@@ -456,7 +521,7 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
             const uint32_t lo = wb > 0 ? wa + 8u * kMargin : wa;
             const uint32_t hi = wa + 8u * (uint32_t)(wn - 1 - (wb + wn < nbins ? kMargin : 0));
             const uint32_t wm = (waits[k & 3u] >> 2) | (waits[(k + 1u) & 3u] << 30);
-            lone_run<TRI>(w, L, ring_at + 32u * (pos & (kRing - 1)), n, wm >> (pos & 31u), F);
+            lone_run<TRI>(w, L, dense, ring_at + 32u * (pos & (kRing - 1)), n, wm >> (pos & 31u), F);
             __syncwarp(all);
             const uint32_t xa = w.xa;
             bc = wb + ((int)(xa - wa) >> 3);
