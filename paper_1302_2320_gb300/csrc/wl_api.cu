@@ -711,7 +711,7 @@ static bool plan_lone(const ShapeKey& k, size_t room, Slot* o)
     s.off_perm = (int)at;
     at += (size_t)k.pstride * 2;
     s.off_win = (int)at;
-    const size_t ring = (128 + 3) * 32 + 32 + 128;   // the draws, their flags, control words, spare words
+    const size_t ring = (128 + 3) * 32 + 16 + 128;   // the draws, control words, spare words
     if (at + (size_t)min_win * 8 + 16 + ring > room) return false;
     s.win = (int)std::min<size_t>((size_t)k.max_bins, (room - 16 - at - ring) / 8);
     at += align16((size_t)s.win * 8);
@@ -722,7 +722,7 @@ static bool plan_lone(const ShapeKey& k, size_t room, Slot* o)
 }
 
 // Cycles a move takes its walker, alone, and per walker on an SM where they get in each
-// other's way (GB300).  A block per line (wl_lone.cuh): 116 alone, 155 with 7 on an SM
+// other's way (GB300).  A block per line (wl_lone.cuh): 118 alone, 155 with 7 on an SM
 // (64x64).  Batches (wl_walk.cuh): 191 with 7 on an SM and the lists staged (96x96),
 // 272 with 16 on an SM and the lists in global memory (96x96) or 12 and staged (64x64);
 // but lines of few up spins, whose batches keep running into themselves, 500.
