@@ -692,26 +692,24 @@ static cudaError_t walk_attrs(const ShapeKey& k, const Slot& slot, size_t smem, 
 
 // The slot of a line with a block of its own (wl_lone.cuh): the words of the sites
 // by code, the list, the window, the ring.
-static bool plan_lone(const ShapeKey& k, size_t room, Slot* o)
+static bool plan_lone(const ShapeKey& k, int word, size_t room, Slot* o)
 {
     if (!k.idx16) return false;
     const bool open = k.lattice == kSquareOpen;      // with a border around it
     size_t stride = 1;
     while (stride < (size_t)k.L + (open ? 1 : 0)) stride <<= 1;
     const size_t codes = (k.lattice == kCubic ? stride : 1) * stride * ((size_t)k.L + (open ? 2 : 0));
-    // the words start at a whole row (cubic: plane), and a list entry holds an address
-    const size_t row = 4 * stride * (k.lattice == kCubic ? stride : 1);
-    if (4 * codes + row > 65536 - 2048) return false;
-    // two margins of 32 steps of the largest bin step, and 64 bins to walk between them
+    if (word * codes > 65536) return false;          // a list entry holds an address
+    // two margins of 16 steps of the largest bin step, and 64 bins to walk between them
     const int zb = k.lattice == kSquareOpen ? 8 : k.lattice == kTriangular || k.lattice == kCubic ? 6 : 4;
-    const int min_win = std::min(k.max_bins, 64 * zb + 64);
+    const int min_win = std::min(k.max_bins, 32 * zb + 64);
     Slot s;
-    s.lone = true;
-    size_t at = align16(4 * codes + row);
+    s.lone = word;
+    size_t at = align16(word * codes);
     s.off_perm = (int)at;
     at += (size_t)k.pstride * 2;
     s.off_win = (int)at;
-    const size_t ring = (128 + 3) * 32 + 16 + 128;   // the draws, control words, spare words
+    const size_t ring = (96 + 3) * 32 + 16 + 128;   // the draws, control words, spare words
     if (at + (size_t)min_win * 8 + 16 + ring > room) return false;
     s.win = (int)std::min<size_t>((size_t)k.max_bins, (room - 16 - at - ring) / 8);
     at += align16((size_t)s.win * 8);
@@ -721,12 +719,17 @@ static bool plan_lone(const ShapeKey& k, size_t room, Slot* o)
     return true;
 }
 
-// Cycles a move takes its walker, alone, and per walker on an SM where they get in each
-// other's way (GB300).  A block per line (wl_lone.cuh): 118 alone, 155 with 7 on an SM
-// (64x64).  Batches (wl_walk.cuh): 191 with 7 on an SM and the lists staged (96x96),
-// 272 with 16 on an SM and the lists in global memory (96x96) or 12 and staged (64x64);
-// but lines of few up spins, whose batches keep running into themselves, 500.
-constexpr double kLoneCycles = 120.0, kLoneIssue = 22.0, kBatchIssue = 17.0, kBatchSlowest = 500.0;
+// Cycles a move takes its walker (GB300).
+// A block per line (wl_lone.cuh), words of 4 bytes or of one: 119 and 126 with up to 4 on
+// an SM, one for each scheduler; 153 .. 168 with up to 8; 217 with 10 (64x64).  So a
+// third more for every further walker on a scheduler.
+// Batches (wl_walk.cuh): 191 with 7 on an SM and the lists staged (96x96), 272 with 16
+// on an SM and the lists in global memory (96x96) or 12 and staged (64x64); and what a
+// surface's lines of few up spins take longer, whose batches keep running into
+// themselves.  Whole surfaces, cycles for a move of all lines, block per line against
+// batches: 64x64 320 and 1189, 96x96 827 and 1367, 112x112 1260 and ~1350,
+// 128x128 1920 and 1536.
+constexpr double kLoneCycles[2] = {119.0, 126.0}, kLoneCrowd = 0.33, kBatchIssue = 17.0, kBatchSlowest = 600.0;
 
 // Either a block of two warps per line, or one warp per block with 32 / S walkers,
 // whichever takes its walkers less time for a move of all of them.  The shape spreads the walkers over
@@ -751,21 +754,30 @@ wl_status plan_shape(const ShapeKey& k, Shape* sh)
     };
     double best = 0.0;
     int best_blocks = 0;
-    // a block per line: as many as fit, each with its share of the shared memory
-    if (k.lone) {
+    // a block per line: as many as fit, each with its share of the shared memory; words of
+    // a byte where that makes room for enough more of them (wl_lone.cuh)
+    for (int word : {4, 1}) {
+        if (!k.lone) break;
+        auto cycles = [&](int on_sm) {
+            return kLoneCycles[word == 1] * (1.0 + kLoneCrowd * ((on_sm + 3) / 4 - 1));
+        };
         int b = std::min((k.lines + sms - 1) / sms, 32), bps = 0;
         Slot slot;
-        while (b > 0 && !plan_lone(k, room_of(b), &slot)) --b;
+        while (b > 0 && !plan_lone(k, word, room_of(b), &slot)) --b;
         if (b > 0) CU(walk_attrs(k, slot, slot.bytes, 64, &bps));
         b = std::min(b, bps);
-        if (b > 0) {
-            const double rounds = (double)((k.lines + sms * b - 1) / (sms * b));
-            best = rounds * std::max(kLoneCycles, kLoneIssue * b);
+        if (b < 1) continue;
+        // whole rounds, and one of what is left
+        const int rest = (k.lines % (sms * b) + sms - 1) / sms;
+        const double cost = k.lines / (sms * b) * cycles(b) + (rest > 0 ? cycles(rest) : 0.0);
+        if (best_blocks == 0 || cost < best) {
+            if (!plan_lone(k, word, room_of(b), &slot)) continue;
+            best = cost;
             best_blocks = b;
-            plan_lone(k, room_of(b), &sh->slot);
+            sh->slot = slot;
             sh->grid = dim3(std::min(k.lines, sms * b));
             sh->block = dim3(64);
-            sh->smem = sh->slot.bytes;
+            sh->smem = slot.bytes;
         }
     }
     auto room = [&](int blocks) {      // bytes per walker with this many blocks on an SM
@@ -788,7 +800,7 @@ wl_status plan_shape(const ShapeKey& k, Shape* sh)
         b = std::min(b, bps);
         if (b < 1) continue;
         const double rounds = (double)((need + sms * b - 1) / (sms * b));
-        const double cost = std::max(rounds * std::max(m.cycles, kBatchIssue * b * groups), kBatchSlowest);
+        const double cost = rounds * std::max(m.cycles, kBatchIssue * b * groups) + kBatchSlowest;
         if (best_blocks == 0 || cost < best) {
             if (!plan_slot(k, m.sites, m.perm, room(b), &slot)) continue;
             best = cost;

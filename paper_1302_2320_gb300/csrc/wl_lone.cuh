@@ -25,9 +25,12 @@
 // each word (116 where slots are rarely shared, 200 where they often are, and with two
 // codes for the two the instruction cache suffers where handles share an SM).
 //
-// Sites are kept as the addresses of their words, whose rows have a power-of-two
-// stride, so that coordinates need no division and a list entry no address
-// arithmetic: 4 ((y << s) | x) past a base aligned to a row (cubic: a plane).
+// Sites are kept as the addresses of their words past the start of the shared memory;
+// rows have a power-of-two stride, (y << s) | x, so that coordinates need no division
+// and a list entry no address arithmetic.  A word is a
+// byte, so that a line takes little shared memory: on an SM with many lines the walkers
+// fill each other's gaps, and what bounds them together is the shared-memory pipe (14
+// of its cycles a step).
 #pragma once
 
 #include "wl_walk.cuh"
@@ -36,9 +39,10 @@ namespace wl {
 
 // The ring of draws: per step {dmax (two words), U slot, D slot} and the same with the
 // slots the other way round, for the lanes of the down site.
-constexpr int kRing = 128;                 // steps (4 batches of 32)
+constexpr int kRing = 96;                  // steps (3 batches of 32)
 constexpr int kRingMore = 3;               // the first records again past the end: a step reads up to 3 ahead
 constexpr int kLoneThreads = 64;           // one warp walks, one draws
+constexpr uint32_t kLow = 1024u;           // address at which the shared memory of a block starts
 
 // The lattice is a run-time matter but for the second axis of the triangular one's
 // diagonals (TRI): requests for different lattices that share an SM then run the same
@@ -64,7 +68,7 @@ __device__ __forceinline__ uint32_t code_site(const Geo& g, uint32_t c)
     return ((c >> g.cshift) - (g.shape == kShapeOpen ? 1u : 0u)) * L + x;
 }
 
-// 8 for every up neighbour of site n (open boundaries: 16, less 8 for every neighbour).
+// The word of site n (LoneLane).
 template <int LAT>
 __device__ __forceinline__ uint32_t site_word(const Geo& g, const uint32_t* sp, uint32_t n)
 {
@@ -81,7 +85,7 @@ __device__ __forceinline__ uint32_t site_word(const Geo& g, const uint32_t* sp, 
 #pragma unroll
         for (int q = 0; q < z; ++q) u += (int)spin_at(sp, nb[q]);
     }
-    return (uint32_t)(8 * u);
+    return (uint32_t)(8 * u) + (LAT == kSquareOpen ? 32u : 0u);
 }
 
 // Shared memory by 32-bit address (generic pointers cost 64-bit address arithmetic).
@@ -92,10 +96,14 @@ __device__ __forceinline__ uint32_t lds16(uint32_t a)
     asm volatile("{.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;}" : "=r"(v) : "r"(a) : "memory");
     return v;
 }
-__device__ __forceinline__ uint32_t lds32(uint32_t a)
+template <int WORD>
+__device__ __forceinline__ uint32_t lds_word(uint32_t a)      // the word of the site at a
 {
     uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    if constexpr (WORD == 4)
+        asm volatile("ld.shared.u32 %0, [%1+1024];" : "=r"(v) : "r"(a) : "memory");
+    else
+        asm volatile("ld.shared.u8 %0, [%1+1024];" : "=r"(v) : "r"(a) : "memory");
     return v;
 }
 __device__ __forceinline__ uint2 lds64u(uint32_t a)
@@ -110,12 +118,6 @@ __device__ __forceinline__ int64_t lds64(uint32_t a)
     asm volatile("ld.shared.s64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
     return v;
 }
-__device__ __forceinline__ uint4 lds128(uint32_t a)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
-    return v;
-}
 __device__ __forceinline__ void sts64(uint32_t a, int64_t v)
 {
     asm volatile("st.shared.s64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
@@ -124,12 +126,19 @@ __device__ __forceinline__ void sts16(uint32_t a, uint32_t v)
 {
     asm volatile("{.reg .u16 h;\n\tcvt.u16.u32 h, %1;\n\tst.shared.u16 [%0], h;}" ::"r"(a), "r"(v) : "memory");
 }
-__device__ __forceinline__ void reds(uint32_t a, uint32_t v)
+__device__ __forceinline__ void red_word(uint32_t a, uint32_t v)     // a: a multiple of 4
 {
-    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+    asm volatile("red.shared.add.u32 [%0+1024], %1;" ::"r"(a), "r"(v) : "memory");
 }
+static_assert(kLow == 1024u, "the offset in lds_word and red_word");
 
-__device__ __forceinline__ void lone_barrier() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+// The two warps of a block keep step at a barrier per batch of 32 steps.  The lanes of a
+// warp come to it together, and its form allows for those that do not.
+__device__ __forceinline__ void lone_barrier()
+{
+    __syncwarp();
+    asm volatile("barrier.sync 1, 64;" ::: "memory");
+}
 
 // The lanes of the walking warp.  Lane q < z stands for neighbour q of the pending
 // step's up site, lane z + q for neighbour q of its down site.  The others go along, so
@@ -138,9 +147,10 @@ __device__ __forceinline__ void lone_barrier() { asm volatile("bar.sync 1, 64;" 
 //
 // A word holds 8 for every up neighbour, the bytes of one bin of ln g: half the change
 // of k.  With open boundaries bins are half as wide, and a word holds 16 for every up
-// neighbour less 8 for every neighbour; a missing neighbour is a word of the border
-// around the lattice, which nobody reads.
-template <bool TRI>
+// neighbour less 8 for every neighbour, plus 32; a missing neighbour is a word of the
+// border around the lattice, which nobody reads.  Words stay within 0 .. 255, so that
+// what is added to one of the four in 32 bits never reaches the next.
+template <bool TRI, int WORD>
 struct LoneLane {
     uint32_t swap;                   // 16 for the lanes of the down site: their order in a ring record
     int32_t sign;                    // own word less the other's, as up less down
@@ -150,7 +160,7 @@ struct LoneLane {
     uint32_t s0, m0, e0, d0, w0;     // along one axis: shift, mask, coordinate at the edge, step, step at the edge
     uint32_t s1, m1, e1, d1, w1;     // along the other (triangular diagonals)
 
-    __device__ __forceinline__ void setup(const Geo& g, int lane, uint32_t words, uint32_t spare)
+    __device__ __forceinline__ void setup(const Geo& g, int lane, uint32_t spare)
     {
         const int z = g.shape == kShapeTriangular || g.shape == kShapeCubic ? 6 : 4;
         const bool open = g.shape == kShapeOpen;
@@ -162,12 +172,10 @@ struct LoneLane {
         accept = down ? unit : 0u - unit;            // the up site goes, the down site comes
         const uint32_t e = (uint32_t)g.L - 1u;
         auto axis = [&](int ax, bool plus, uint32_t& s, uint32_t& mk, uint32_t& ed, uint32_t& d, uint32_t& w) {
-            s = (uint32_t)(ax * g.cshift) + 2u;
+            s = (uint32_t)(ax * g.cshift) + (WORD == 4 ? 2u : 0u);
             const uint32_t u = 1u << s;
-            // the outermost coordinate is what is left of the address, base and all
-            const bool outer = ax == (g.shape == kShapeCubic ? 2 : 1);
-            mk = outer ? 0xFFFFFFFFu : g.cmask;
-            ed = (plus ? e : 0u) + (outer ? words >> s : 0u);
+            mk = g.cmask;
+            ed = plus ? e : 0u;
             d = plus ? u : 0u - u;
             w = open ? d : plus ? 0u - e * u : e * u;
         };
@@ -184,7 +192,7 @@ struct LoneLane {
         if (lane >= 2 * z) {
             scale = d1 = w1 = 0u;
             accept = lane == 2 * z ? 1u : 0u;
-            d0 = w0 = spare + 4u * (uint32_t)lane;
+            d0 = w0 = spare - kLow + 4u * (uint32_t)lane;
         }
     }
 
@@ -206,17 +214,23 @@ struct Lone {
     uint32_t ta;            // address of the bin the pending step proposes
     int64_t u;              // ln g of the current bin
     uint32_t own, oth, nb;  // pending step
+    uint32_t add;           // what it adds to the four words around nb's if accepted
     uint32_t own1, oth1;    // the step after it
     uint2 slot0, slot1, slot2;      // own, other
 };
 
 // The pending step's neighbour of this lane and the bin it proposes, from the words wo
 // and wt of its sites.
-template <bool TRI>
-__device__ __forceinline__ void lone_propose(Lone& w, const LoneLane<TRI>& L, uint32_t wo, uint32_t wt)
+template <bool TRI, int WORD>
+__device__ __forceinline__ void lone_propose(Lone& w, const LoneLane<TRI, WORD>& L, uint32_t wo, uint32_t wt)
 {
     w.nb = L.neighbour(w.own);
     const uint32_t at = w.xa + (__any_sync(0xffffffffu, w.nb == w.oth) ? L.unit : 0u);
+    w.add = L.accept;
+    if constexpr (WORD == 1) {
+        w.add = __funnelshift_l(0u, L.accept, w.nb << 3);     // by 8 (nb & 3)
+        w.nb &= ~3u;
+    }
     w.ta = at + (uint32_t)((int32_t)(wo - wt) * L.sign);
 }
 
@@ -224,8 +238,8 @@ __device__ __forceinline__ void lone_propose(Lone& w, const LoneLane<TRI>& L, ui
 // step's record in the ring, in this lane's order.  The order of the memory accesses is
 // the order they are written in here: the reduction first and the words right behind
 // it, the stores the next decision does not wait for after them.
-template <bool TRI>
-__device__ __forceinline__ void lone_step(Lone& w, const LoneLane<TRI>& L, uint32_t at, int64_t F)
+template <bool TRI, int WORD>
+__device__ __forceinline__ void lone_step(Lone& w, const LoneLane<TRI, WORD>& L, uint32_t at, int64_t F)
 {
     const int64_t gt = lds64(w.ta);
     const int64_t dmax = lds64(at);
@@ -234,9 +248,9 @@ __device__ __forceinline__ void lone_step(Lone& w, const LoneLane<TRI>& L, uint3
     const uint32_t no = p ? w.oth : w.own, nt = p ? w.own : w.oth;
     w.own = w.slot1.x == w.slot0.x ? no : w.own1;
     w.oth = w.slot1.y == w.slot0.y ? nt : w.oth1;
-    reds(w.nb, p ? L.accept : 0u);
+    red_word(w.nb, p ? w.add : 0u);
     __syncwarp();
-    const uint32_t wo = lds32(w.own), wt = lds32(w.oth);
+    const uint32_t wo = lds_word<WORD>(w.own), wt = lds_word<WORD>(w.oth);
     w.xa = p ? w.ta : w.xa;
     w.u = (p ? gt : w.u) + F;
     sts16(w.slot0.x, no);                // the lanes of either site write its slot
@@ -247,44 +261,46 @@ __device__ __forceinline__ void lone_step(Lone& w, const LoneLane<TRI>& L, uint3
     w.slot0 = w.slot1;
     w.slot1 = w.slot2;
     w.slot2 = lds64u(at + 104u);
-    lone_propose<TRI>(w, L, wo, wt);
+    lone_propose<TRI, WORD>(w, L, wo, wt);
 }
 
-template <bool TRI, int K>
-__device__ __forceinline__ void lone_block(Lone& w, const LoneLane<TRI>& L, uint32_t& at, int64_t F)
+template <bool TRI, int WORD, int K>
+__device__ __forceinline__ void lone_block(Lone& w, const LoneLane<TRI, WORD>& L, uint32_t& at, int64_t F)
 {
 #pragma unroll
-    for (int q = 0; q < K; ++q) lone_step<TRI>(w, L, at + 32u * q, F);
+    for (int q = 0; q < K; ++q) lone_step<TRI, WORD>(w, L, at + 32u * q, F);
     at += 32u * K;
 }
 
-// Take n <= 32 steps, from the record at `at` on, in blocks: the end of a loop's body
+// Take n <= 16 steps, from the record at `at` on, in blocks: the end of a loop's body
 // costs ~75 cycles (the compiler lets the loops of a kernel yield whose warps part
 // before a barrier).  16x16, l = 4: 126 cycles a step in blocks of 8, 118 of 16.
-template <bool TRI>
-__device__ __forceinline__ void lone_run(Lone& w, const LoneLane<TRI>& L, uint32_t at, int n, int64_t F)
+template <bool TRI, int WORD>
+__device__ __forceinline__ void lone_run(Lone& w, const LoneLane<TRI, WORD>& L, uint32_t at, int n, int64_t F)
 {
+    if (n == 16) {
+        lone_block<TRI, WORD, 16>(w, L, at, F);
+        return;
+    }
 #pragma unroll 1
-    for (; n >= 16; n -= 16) lone_block<TRI, 16>(w, L, at, F);
+    for (; n >= 4; n -= 4) lone_block<TRI, WORD, 4>(w, L, at, F);
 #pragma unroll 1
-    for (; n >= 4; n -= 4) lone_block<TRI, 4>(w, L, at, F);
-#pragma unroll 1
-    for (; n > 0; --n) lone_block<TRI, 1>(w, L, at, F);
+    for (; n > 0; --n) lone_block<TRI, WORD, 1>(w, L, at, F);
 }
 
 // The drawing warp: batches of 32 steps from t on, until the walker is done.
 template <bool DET>
 __device__ __forceinline__ void lone_draw(const WalkArgs& A, int64_t t, int ell, uint4* ring, uint32_t perm,
-                                          const volatile int32_t* done, int lane)
+                                          const volatile uint64_t* last, int lane)
 {
     const uint2 key = make_uint2((uint32_t)ell, A.seed);
     const uint32_t nd = (uint32_t)(A.g.N - ell);
-    auto fill = [&](uint32_t k) {
-        const Draw d = draw_step<DET>((uint64_t)t + 32u * (uint64_t)k + (uint64_t)lane, key, (uint32_t)ell, nd, A);
+    auto fill = [&](uint64_t k, uint32_t at) {
+        const Draw d = draw_step<DET>((uint64_t)t + 32u * k + (uint64_t)lane, key, (uint32_t)ell, nd, A);
         const uint32_t sa = perm + 2u * d.a, sb = perm + 2u * ((uint32_t)ell + d.b);
         const uint4 r = make_uint4((uint32_t)d.dmax, (uint32_t)((uint64_t)d.dmax >> 32), sa, sb);
         const uint4 q = make_uint4(r.x, r.y, sb, sa);
-        const uint32_t at = (32u * k + (uint32_t)lane) & (kRing - 1);
+        at += (uint32_t)lane;
         ring[2u * at] = r;
         ring[2u * at + 1u] = q;
         if (at < kRingMore) {
@@ -292,32 +308,33 @@ __device__ __forceinline__ void lone_draw(const WalkArgs& A, int64_t t, int ell,
             ring[2u * (kRing + at) + 1u] = q;
         }
     };
-    fill(0);
-    fill(1);
+    fill(0u, 0u);
+    fill(1u, 32u);
     lone_barrier();
-    for (uint32_t k = 2;; ++k) {
-        fill(k);
+    uint32_t at = 64u;
+    for (uint64_t k = 2u;; ++k) {            // the k-th barrier
+        fill(k, at);
+        at = at == 64u ? 0u : at + 32u;
         lone_barrier();
-        if (*done) break;
+        if (*last == k) break;
     }
 }
 
 // The walking warp: line `li` for up to A.slice_moves moves (or to its budget, or
 // to convergence); the bookkeeping between steps as in walk_line.
-template <bool TRI>
+template <bool TRI, int WORD>
 __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint8_t* sm, const uint4* ring,
-                                          uint32_t words, uint32_t* spare, volatile int32_t* done)
+                                          uint32_t* spare, volatile uint64_t* last)
 {
     const bool open = A.g.shape == kShapeOpen;
     const int ks = open ? 0 : 1;
     const int zb = open ? 8 : A.g.shape == kShapeTriangular || A.g.shape == kShapeCubic ? 6 : 4;    // Coord::zbin
-    const int kMargin = 32 * zb;         // a run of steps stays inside the window
+    const int kMargin = 16 * zb;         // a run of steps stays inside the window
     constexpr unsigned all = 0xffffffffu;
     const LineDesc D = A.desc[li];
     LineState* P = A.st + li;
-    int64_t t = P->t, F = P->F, stage = P->stage, accepts = P->accepts;
-    int64_t t_stage = P->t_stage, status = P->status, checks = P->checks;
-    const int64_t t0 = t, batches = P->batches;
+    // what only a check needs stays in memory: registers are few
+    int64_t t = P->t, F = P->F;
     const int nbins = D.nbins;
     int64_t* lng = A.lng + D.bin_off;
     hist_t* hist = A.hist + D.bin_off;
@@ -338,8 +355,8 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
     window_load<32>(wl, lng, wb, wn, m);
     __syncwarp(all);
     const uint32_t wa = (uint32_t)__cvta_generic_to_shared(wl);
-    LoneLane<TRI> L;
-    L.setup(A.g, m, words, (uint32_t)__cvta_generic_to_shared(spare));
+    LoneLane<TRI, WORD> L;
+    L.setup(A.g, m, (uint32_t)__cvta_generic_to_shared(spare));
     const uint32_t ring_at = (uint32_t)__cvta_generic_to_shared(ring) + L.swap;
     uint32_t* counter = spare + (zb == 6 ? 12 : 8);       // the first lane past the neighbours
     Lone w{};
@@ -347,6 +364,7 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
     w.u = wl[bc - wb];
     if (m == 0) *counter = 0u;
     lone_barrier();               // the first two batches are drawn
+    uint64_t barriers = 1u;
     if (t < end) {
         // the first step is pending, the second loaded, the third's slots at hand
         w.slot0 = lds64u(ring_at + 8u);
@@ -356,13 +374,14 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
         w.oth = lds16(w.slot0.y);
         w.own1 = lds16(w.slot1.x);
         w.oth1 = lds16(w.slot1.y);
-        const uint32_t wo = lds32(w.own), wt = lds32(w.oth);
-        lone_propose<TRI>(w, L, wo, wt);
+        const uint32_t wo = lds_word<WORD>(w.own), wt = lds_word<WORD>(w.oth);
+        lone_propose<TRI, WORD>(w, L, wo, wt);
     }
     __syncwarp(all);
 
     uint32_t pos = 0u;                       // steps since t0, modulo 2^32
-    uint32_t lo = 0u, hi = 0u;               // the bins a run of 32 steps may start from
+    uint32_t at = ring_at;                   // the pending step's record
+    uint32_t lo = 0u, hi = 0u;               // the bins a run of 16 steps may start from
     auto set_margins = [&]() {
         lo = wb > 0 ? wa + 8u * (uint32_t)kMargin : wa;
         hi = wa + 8u * (uint32_t)(wn - 1 - (wb + wn < nbins ? kMargin : 0));
@@ -374,40 +393,46 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
         if (seg_end - t > (1ll << 30)) seg_end = t + (1ll << 30);
         int64_t left = seg_end - t;
         while (left > 0) {
-            const uint32_t in = pos & 31u;
-            const int n = left < 32 - (int)in ? (int)left : 32 - (int)in;
-            lone_run<TRI>(w, L, ring_at + 32u * (pos & (kRing - 1)), n, F);
+            const uint32_t in = pos & 15u;
+            const int n = left < 16 - (int)in ? (int)left : 16 - (int)in;
+            lone_run<TRI, WORD>(w, L, at, n, F);
             pos += (uint32_t)n;
+            at += 32u * (uint32_t)n;
             left -= n;
             if (w.xa < lo || w.xa > hi) {
                 const uint32_t xa = w.xa;
                 bc = wb + ((int)(xa - wa) >> 3);
                 if (xa < wa || bc - wb >= wn) {
                     stop = 4;              // never: a run from inside the margins stays inside
-                    break;
+                } else {
+                    // re-centre the window
+                    __syncwarp(all);
+                    if (__any_sync(all, window_store<32>(wl, lng, hist, wb, wn, m, F))) stop = 2;
+                    __syncwarp(all);
+                    wb = window_base(bc, nbins, A.win_bins);
+                    window_load<32>(wl, lng, wb, wn, m);
+                    __syncwarp(all);
+                    const uint32_t to = wa + 8u * (uint32_t)(bc - wb);
+                    w.ta += to - xa;
+                    w.xa = to;
+                    set_margins();
                 }
-                // re-centre the window
-                __syncwarp(all);
-                if (__any_sync(all, window_store<32>(wl, lng, hist, wb, wn, m, F))) stop = 2;
-                __syncwarp(all);
-                wb = window_base(bc, nbins, A.win_bins);
-                window_load<32>(wl, lng, wb, wn, m);
-                __syncwarp(all);
-                const uint32_t to = wa + 8u * (uint32_t)(bc - wb);
-                w.ta += to - xa;
-                w.xa = to;
-                set_margins();
             }
-            if ((pos & 31u) == 0u) lone_barrier();
+            if ((pos & 31u) == 0u) {
+                lone_barrier();
+                ++barriers;
+                if (at == ring_at + 32u * kRing) at = ring_at;
+            }
             if (stop) break;
         }
         t = seg_end - left;
         bc = wb + ((int)(w.xa - wa) >> 3);
         // a segment is short enough for the 32-bit counter
         __syncwarp(all);
-        accepts += *counter;
-        __syncwarp(all);
-        if (m == 0) *counter = 0u;
+        if (m == 0) {
+            P->accepts += *counter;
+            *counter = 0u;
+        }
         __syncwarp(all);
         if (stop) break;
 
@@ -419,9 +444,9 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
                 break;
             }
             __syncwarp(all);
-            checks += 1;
+            if (m == 0) P->checks += 1;
             const bool flat = group_flat<32>(hist, nbins, m, all, A.flat_pm);
-            const bool again = !flat && A.same_f_resets > 0 && (t - t_stage) / C <= A.same_f_resets;
+            const bool again = !flat && A.same_f_resets > 0 && (t - P->t_stage) / C <= A.same_f_resets;
             if (flat || again) {
                 group_stage_step<32>(lng, hist, nbins, m, all);
                 window_load<32>(wl, lng, wb, wn, m);
@@ -429,13 +454,14 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
                 w.u = wl[bc - wb];
             }
             if (flat) {
-                stage += 1;
-                t_stage = t;
-                F >>= 2;                     // ln f -> ln f / 4
-                if (F == 0) {                // ln f < ln f_min
-                    status = 1;
-                    break;
+                __syncwarp(all);
+                if (m == 0) {
+                    P->stage += 1;
+                    P->t_stage = t;
                 }
+                __syncwarp(all);
+                F >>= 2;                     // ln f -> ln f / 4
+                if (F == 0) break;           // ln f < ln f_min
             }
             int req = 0;
             if (m == 0) {
@@ -453,58 +479,54 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
         __syncwarp(all);
         if (__ballot_sync(all, window_store<32>(wl, lng, hist, wb, wn, m, F)) && stop == 0) stop = 2;
     }
-    if (stop == 2) status = 2;
-    if (stop == 4) status = 3;
     if (m == 0) {
+        if (F == 0) P->status = 1;
+        if (stop == 2) P->status = 2;
+        if (stop == 4) P->status = 3;
         P->k = (int64_t)bc << ks;
+        P->batches += (t - P->t + 31) / 32;
         P->t = t;
         P->F = F;
-        P->stage = stage;
-        P->accepts = accepts;
-        P->t_stage = t_stage;
-        P->status = status;
-        P->checks = checks;
-        P->batches = batches + (t - t0 + 31) / 32;
         if (stop == 1) atomicOr(A.flags, 1);
         if (stop == 3) atomicOr(A.flags, 2);
         if (stop == 2) atomicOr(A.flags, 4);
         if (stop == 4) atomicOr(A.flags, 8);
-        *done = 1;
+        *last = barriers + 1u;           // the next one
     }
     __syncwarp(all);
     lone_barrier();
 }
 
-// One block per line: shared memory holds the words of the sites (and one more), the
-// list, the window, the ring of draws.
-template <bool TRI, bool DET>
-__global__ void __launch_bounds__(kLoneThreads) lone_kernel(const WalkArgs A)
+// One block per line: shared memory holds the words of the sites, the list, the window,
+// the ring of draws.
+template <bool TRI, bool DET, int WORD>
+__global__ void __launch_bounds__(kLoneThreads, WORD == 4 ? 8 : 10) lone_kernel(const WalkArgs A)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     const int th = threadIdx.x, warp = th >> 5, lane = th & 31;
-    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
-    // the words start at a whole row (cubic: plane) of addresses
-    const uint32_t row = 4u << (A.g.shape == kShapeCubic ? 2 * A.g.cshift : A.g.cshift);
-    const uint32_t words_at = (base + row - 1u) / row * row;
-    uint32_t* words = reinterpret_cast<uint32_t*>(smem + (words_at - base));
+    if ((uint32_t)__cvta_generic_to_shared(smem) != kLow) {      // never
+        if (th == 0) atomicOr(A.flags, 8);
+        return;
+    }
     uint16_t* perm = reinterpret_cast<uint16_t*>(smem + A.off_perm);
     uint4* ring = reinterpret_cast<uint4*>(smem + A.off_rec);
-    int32_t* ctl = reinterpret_cast<int32_t*>(ring + 2 * (kRing + kRingMore));    // the line; the walker is done; who walks
+    int32_t* ctl = reinterpret_cast<int32_t*>(ring + 2 * (kRing + kRingMore));    // the line; who walks; the barrier at which the walker is done
     if (th == 0) {
         // The SM deals its warps out to four schedulers in order of their slots: were
         // it always the first warp of a block that walks, all walkers would share two
         // of them.  Any choice is right; this one spreads them over all four.
         uint32_t slot;
         asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
-        ctl[2] = (int32_t)((slot >> 2) & 1u);
+        ctl[1] = (int32_t)((slot >> 2) & 1u);
     }
+    uint64_t* last = reinterpret_cast<uint64_t*>(ctl + 2);
     uint32_t* spare = reinterpret_cast<uint32_t*>(ctl + 4);
     const int N = A.g.N, pstride = A.pstride;
     for (;;) {
         if (th == 0) {
             const int qi = atomicAdd(A.qnext, 1);
             ctl[0] = qi < A.nqueue ? A.order[qi] : -1;
-            ctl[1] = 0;
+            *last = 0u;
         }
         __syncthreads();
         const int li = ctl[0];
@@ -512,32 +534,41 @@ __global__ void __launch_bounds__(kLoneThreads) lone_kernel(const WalkArgs A)
         if (A.st[li].status == 0) {
             uint16_t* gperm = reinterpret_cast<uint16_t*>(A.perm) + (size_t)li * pstride;
             uint32_t* gsp = A.spins + (size_t)li * A.g.W;
+            if (A.g.shape == kShapeOpen) {           // the border: far from either end of a byte
+                for (int x = th; x < A.off_perm; x += kLoneThreads) smem[x] = WORD == 4 && (x & 3) ? 0u : 128u;
+                __syncthreads();
+            }
             for (int n = th; n < N; n += kLoneThreads) {
-                perm[n] = (uint16_t)(words_at + 4u * site_code(A.g, gperm[n]));
+                perm[n] = (uint16_t)(WORD * site_code(A.g, gperm[n]));
                 const uint32_t u = A.g.shape == kShapeTriangular ? site_word<kTriangular>(A.g, gsp, (uint32_t)n)
                                    : A.g.shape == kShapeCubic    ? site_word<kCubic>(A.g, gsp, (uint32_t)n)
                                    : A.g.shape == kShapeOpen     ? site_word<kSquareOpen>(A.g, gsp, (uint32_t)n)
                                                                  : site_word<kSquare>(A.g, gsp, (uint32_t)n);
-                words[site_code(A.g, (uint32_t)n)] = u;
+                const uint32_t c = site_code(A.g, (uint32_t)n);
+                if constexpr (WORD == 4)
+                    reinterpret_cast<uint32_t*>(smem)[c] = u;
+                else
+                    smem[c] = (uint8_t)u;
             }
             const int64_t t = A.st[li].t;
             const int ell = A.desc[li].ell;
             __syncthreads();
-            if (warp == ctl[2])
-                lone_walk<TRI>(A, li, lane, smem, ring, words_at, spare, ctl + 1);
+            if (warp == ctl[1])
+                lone_walk<TRI, WORD>(A, li, lane, smem, ring, spare, last);
             else
-                lone_draw<DET>(A, t, ell, ring, (uint32_t)__cvta_generic_to_shared(perm), ctl + 1, lane);
+                lone_draw<DET>(A, t, ell, ring, (uint32_t)__cvta_generic_to_shared(perm), last, lane);
             __syncthreads();
             // the list, and from it the spins
-            for (int x = th; x * 32 < N; x += kLoneThreads) words[x] = 0u;
+            uint32_t* sp = reinterpret_cast<uint32_t*>(smem);
+            for (int x = th; x * 32 < N; x += kLoneThreads) sp[x] = 0u;
             __syncthreads();
             for (int n = th; n < N; n += kLoneThreads) {
-                const uint32_t s = code_site(A.g, (perm[n] - words_at) >> 2);
+                const uint32_t s = code_site(A.g, perm[n] / (uint32_t)WORD);
                 gperm[n] = (uint16_t)s;
-                if (n < ell) atomicOr(&words[s >> 5], 1u << (s & 31u));
+                if (n < ell) atomicOr(&sp[s >> 5], 1u << (s & 31u));
             }
             __syncthreads();
-            for (int x = th; x * 32 < N; x += kLoneThreads) gsp[x] = words[x];
+            for (int x = th; x * 32 < N; x += kLoneThreads) gsp[x] = sp[x];
         }
         __syncthreads();
     }

@@ -30,7 +30,8 @@ struct Slot {
     int bytes = 0, off_perm = 0, off_sites = 0, off_win = 0, off_rec = 0;
     int win = 0;                 // bins of the ln g window
     int owner_mask = 0;
-    bool stage_sites = false, stage_perm = false, lone = false;
+    bool stage_sites = false, stage_perm = false;
+    int lone = 0;            // a block per line: bytes of a site's word; else 0
 };
 
 // Launch shape of the persistent form for S lanes per walker.
