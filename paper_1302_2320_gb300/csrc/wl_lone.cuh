@@ -6,7 +6,7 @@
 // slowest line, so what counts is the latency from one decision to the next.  No step
 // is evaluated on a guess, so a line of few up spins or a tiny lattice, where
 // neighbouring steps draw the same list slots all the time, walks as fast as any other:
-// ~118 cycles a step (square 16x16 to 64x64, cubic 8^3; triangular 124).  From decision to decision there are
+// ~120 cycles a step (square 16x16 to 64x64, cubic 8^3, triangular 32x32).  From decision to decision there are
 //   - the change of the words around the two sites (below), then two loads of words;
 //   - the proposed bin, one load of ln g at it, the 64-bit compare.
 // Everything else a step needs lies off that path:
@@ -499,8 +499,13 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
 
 // One block per line: shared memory holds the words of the sites, the list, the window,
 // the ring of draws.
+//
+// Registers for 10 blocks on an SM: a burst of eight requests (square, triangular,
+// cubic, open; 10 blocks an SM) takes 29 ms, 38 with room for 8, when the last request
+// waits for the others; alone a step costs the same (119 and 120 cycles).  Triangular
+// lattices keep more (122 cycles a step against 129).
 template <bool TRI, bool DET, int WORD>
-__global__ void __launch_bounds__(kLoneThreads, WORD == 4 ? 8 : 10) lone_kernel(const WalkArgs A)
+__global__ void __launch_bounds__(kLoneThreads, TRI && WORD == 4 ? 8 : 10) lone_kernel(const WalkArgs A)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     const int th = threadIdx.x, warp = th >> 5, lane = th & 31;
