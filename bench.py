@@ -126,7 +126,8 @@ def _dist():
     return world, rank, local
 
 
-KERNEL_SOURCES = ["paper_1302_2320_gb300/csrc/wl_walk.cuh", "paper_1302_2320_gb300/csrc/wl_device.cuh"]
+KERNEL_SOURCES = ["paper_1302_2320_gb300/csrc/wl_lone.cuh", "paper_1302_2320_gb300/csrc/wl_walk.cuh",
+                  "paper_1302_2320_gb300/csrc/wl_device.cuh"]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "walk_kernel_L64_traffic.txt")
 
 
@@ -718,7 +719,7 @@ def run_ours(args):
                    "parallelism": f"replicas x{world}"},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "Tops/s",
                      "frac": achieved / alu_peak, "traffic": traffic,
-                     "kernel": "walk_kernel", "ops_per_move": INT_OPS_PER_MOVE,
+                     "kernel": "lone_kernel" if L <= 112 and args.form == 0 else "walk_kernel", "ops_per_move": INT_OPS_PER_MOVE,
                      "peak_basis": (f"measured on this GPU by wl_measure_peaks: {MUL_OPS_PER_MOVE} "
                                     f"32x32->64 products at {rates['mulwide_ops_per_s']:.3g}/s plus "
                                     f"{ALU_OPS_PER_MOVE} add/logic ops at {rates['iadd3_ops_per_s']:.3g}/s "

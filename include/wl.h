@@ -102,10 +102,11 @@ size_t wl_required_bytes(wl_lattice lattice, int L);
  *                    moves instead, so lines with more bins get longer stages
  *                    and find their rarest states before ln f shrinks (default 0)
  *   "move_budget"    per-line cap on the move counter t (default 2^62)
- *   "mapping"        lanes per walker S in {1,2,4,8,16,32}; 0 = tuned online: each
- *                    of 32, 16, 8 walks one slice (timed with CUDA events), the
- *                    fastest is kept, and they are timed again when the
- *                    acceptance rate drifts by more than 0.15 (default 0).
+ *   "mapping"        lanes per walker S in {1,2,4,8,16,32}; 0 = the library's
+ *                    choice (default): a block per line where the lines fit, else
+ *                    tuned online: each of 32, 16, 8 walks one slice (timed with
+ *                    CUDA events), the fastest is kept, and they are timed again
+ *                    when the acceptance rate drifts by more than 0.15.
  *                    Every S walks the same chain.
  *   "form"           0: one persistent launch over all lines with a device
  *                    work queue; 1: one launch per line (default 0)
@@ -114,9 +115,10 @@ size_t wl_required_bytes(wl_lattice lattice, int L);
  *   "slice_ms"       if > 0, a persistent launch also ends after this many
  *                    milliseconds of device time, so that no line waits for a
  *                    slower one at the end of a slice (default 0)
- *   "tail"           1: with no more running lines than SMs, each line gets an
- *                    SM of its own (32 lanes per walker, unless another lane
- *                    count is forced); 0: keep the throughput shape (default 1)
+ *   "tail"           1: the shape follows the number of running lines, and lines
+ *                    that fit get a block each, up to an SM of their own (32 lanes
+ *                    per walker, unless another lane count is forced); 0: batches,
+ *                    in a shape for all the lines of the run (default 1)
  *   "timeout_ms"     wall-clock limit of one wl_run, 0 = none (default 0)
  *   "hbm_budget"     refuse to allocate more than this many bytes (default 0 = none)
  *   "ell_min", "ell_max"  walk only lines in [ell_min, ell_max] (defaults 0, N/2)
@@ -130,7 +132,8 @@ size_t wl_required_bytes(wl_lattice lattice, int L);
 wl_status wl_set_option(wl_handle h, const char* key, int64_t value);
 /* Read an option back; also the read-only keys "N", "NB", "z", "k_step",
  * "lines", "bins", "device_bytes" and "tuned_mapping" (the lane count the tuner
- * settled on for this lattice and mode, 0 while it is still timing candidates). */
+ * settled on for this lattice and mode, 0 while it is still timing candidates or
+ * where no lane count is tuned). */
 wl_status wl_get_option(wl_handle h, const char* key, int64_t* value);
 
 /* The walk of the method section, on every selected line: spin-exchange
@@ -317,7 +320,7 @@ wl_status wl_server_destroy(wl_server s);
  * Walks lines ell_first .. ell_first+nlines-1 (all <= N/2; nlines <= 4096, the
  * scratch limit -- larger requests return WL_EINVAL before any launch) of the
  * periodic lattice, exactly as wl_run does with the same options (seed,
- * deterministic, check_interval, move_budget, mapping; 0 = 8 lanes per walker),
+ * deterministic, check_interval, move_budget, mapping; 0 = the library's choice),
  * on `stream` (a cudaStream_t as an integer, 0 = default stream), in slices of
  * 2^20 moves per line, and returns when every line converged (WL_OK) or
  * reached move_budget (WL_ENOTCONVERGED).  move_budget bounds the call: there

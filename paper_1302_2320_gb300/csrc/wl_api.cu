@@ -456,14 +456,13 @@ int pick_mapping_default(const wl_ctx*)
 // Persistent form: slices until every selected line converged or hit the
 // budget, or the run is stopped.
 //
-// Lane count: fixed by the "mapping" option, or (mapping = 0) tuned online
-// over real slices: each candidate (32, 16, 8 lanes per walker) walks one
-// slice, timed with CUDA events, then the fastest is used; the candidates are
-// timed again when the acceptance rate has moved by more than 0.15 since (the
-// best count depends on it).  With no more running lines than SMs the tail
-// shape (32 lanes, one walker per block) is used whatever the tuning says,
-// unless a lane count other than 32 was forced.  Every count walks the same
-// chain, so the choice never changes results.
+// Shape: a block per line where plan_shape finds that faster ("tail" = 1 and 32 lanes or
+// none given).  Otherwise batches; their lane count is fixed by the "mapping" option, or
+// (mapping = 0) tuned online over real slices: each candidate (32, 16, 8 lanes per walker)
+// walks one slice, timed with CUDA events, then the fastest is used; the candidates are
+// timed again when the acceptance rate has moved by more than 0.15 since (the best count
+// depends on it).  Every shape and count walks the same chain, so the choice never
+// changes results.
 wl_status run_persistent(wl_ctx* h, std::chrono::steady_clock::time_point t_start)
 {
     const TuneKey key{h->g.type, h->g.L, h->det};

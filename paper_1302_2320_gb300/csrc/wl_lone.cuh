@@ -1,12 +1,13 @@
-// wl_lone.cuh -- the walker for a surface's lines while an SM has few of them: one block
-// per line, made for the time of one step (arXiv:1302.2320, the procedure around Eq. 3
-// and Eq. 4).
+// wl_lone.cuh -- the walker for lines whose state fits a share of an SM's shared memory:
+// one block per line, made for the time of one step (arXiv:1302.2320, the procedure
+// around Eq. 3 and Eq. 4).  plan_shape chooses between it and batches (wl_walk.cuh).
 //
 // The chain of a line is serial, and the time to the end of a surface is that of its
 // slowest line, so what counts is the latency from one decision to the next.  No step
 // is evaluated on a guess, so a line of few up spins or a tiny lattice, where
 // neighbouring steps draw the same list slots all the time, walks as fast as any other:
-// ~120 cycles a step (square 16x16 to 64x64, cubic 8^3, triangular 32x32).  From decision to decision there are
+// ~120 cycles a step (square 16x16 to 64x64, cubic 8^3, triangular 32x32; batches: 160
+// to 1000, and the walker before both 180 to 420).  From decision to decision there are
 //   - the change of the words around the two sites (below), then two loads of words;
 //   - the proposed bin, one load of ln g at it, the 64-bit compare.
 // Everything else a step needs lies off that path:
@@ -27,10 +28,14 @@
 //
 // Sites are kept as the addresses of their words past the start of the shared memory;
 // rows have a power-of-two stride, (y << s) | x, so that coordinates need no division
-// and a list entry no address arithmetic.  A word is a
-// byte, so that a line takes little shared memory: on an SM with many lines the walkers
-// fill each other's gaps, and what bounds them together is the shared-memory pipe (14
-// of its cycles a step).
+// and a list entry no address arithmetic.
+//
+// WORD: bytes of a site's word.  With 4 a step is shorter (119 cycles against 126: no
+// shift into place); with 1 a line takes little shared memory, so that more of them
+// share an SM and fill each other's gaps (96x96: 6 instead of 2 an SM, 27 cycles a move
+// and SM; 64x64, 7 an SM with either: 23 and 24), and 256x256 fits.  What bounds 7 to 12
+// walkers on an SM together is issue (57 to 70 % of its slots, ~51 instructions a step
+// with the drawing warp's) and the shared-memory pipe (63 to 74 %, 14 cycles a step).
 #pragma once
 
 #include "wl_walk.cuh"

@@ -76,7 +76,7 @@ struct wl_ctx {
     int ell_min = 0, ell_max = 0;
     std::vector<uint8_t> sel;   // lines chosen by wl_select_lines (empty: every line in [ell_min, ell_max])
     int same_f_resets = 0;
-    int tail = 1;            // option "tail": few active lines get the one-walker-per-SM shape
+    int tail = 1;            // option "tail": the shape follows the running lines, a block per line where that is faster
     // state
     bool allocated = false, initialized = false, assembled = false;
     double u = 0.0;

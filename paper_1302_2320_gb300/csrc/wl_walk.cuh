@@ -40,6 +40,12 @@
 // back when the walker nears an edge of it, at every check and at the end.  A
 // visit adds F to a bin's ln g and 1 to its count, so the counts are not kept
 // while walking: storing the window recovers them as (ln g - ln g before) / F.
+//
+// Lattices too large for a block per line walk in this form (plan_shape), and "tail" = 0,
+// other lane counts than 32 and one launch per line.  A line of many up spins takes
+// 160 cycles a move alone (256x256, where resolving the accepted steps with all lanes
+// took 500), 17 a move and SM when there are enough lines to fill it; a line of few up
+// spins, whose batches keep running into themselves, up to 1000.
 #pragma once
 
 #include "wl_device.cuh"
