@@ -376,12 +376,30 @@ wl_status persistent_shape(wl_ctx* h, int S, int active, Shape* sh)
     return plan_shape(k, sh);
 }
 
+// More lines than blocks: they take turns, so that all blocks have work until the end of
+// the slice and not the last round's few (2^18 moves each, 1569 lines of 56x56 on 1520
+// blocks: 37.7 -> 26.7 ms; 2049 lines of 64x64 on 1520: 40.4 -> 33.2).
+// Turns of 2^14 moves and more: loading and storing a line takes ~50 us, a turn 1.3 ms.
+static void set_turns(wl_ctx* h, const Shape& sh, WalkArgs* a)
+{
+    a->turns = 1;
+    if (!sh.slot.lone || h->nqueue <= (int)sh.grid.x) return;
+    const int64_t moves = std::min(a->slice_moves, a->budget);
+    if (moves > (1 << 26)) return;       // turns of more than a second
+    a->turns = (int)std::max<int64_t>(1, std::min<int64_t>(8, moves >> 14));
+    a->turn = h->d_qheads;
+}
+
 // One slice of the persistent form on stream h->s (capturable).
 wl_status enqueue_slice(wl_ctx* h, int S, const Shape& sh)
 {
     WalkArgs a = base_args(h);
     set_slot(sh.slot, &a);
-    CU(cudaMemsetAsync(a.qnext, 0, 4, h->s));
+    set_turns(h, sh, &a);
+    if (a.turns > 1)
+        CU(cudaMemsetAsync(h->d_qheads, 0, (size_t)(h->lo.nlines + 1) * 4, h->s));     // with qnext
+    else
+        CU(cudaMemsetAsync(a.qnext, 0, 4, h->s));
     if (h->slice_ms > 0) CU(launch_set_deadline(h->d_deadline + 1, (uint64_t)h->slice_ms * 1000000ull, h->s));
     CU(launch_walk(kernel_lattice(h), S, h->det != 0, h->lo.idx16, sh.grid, sh.block, sh.smem, h->s, a));
     CU(launch_summary(h->d_st, h->lo.nlines, h->budget, h->d_flags, h->d_summary, h->s));
@@ -399,6 +417,7 @@ wl_status run_slice(wl_ctx* h, int S, const Shape& sh, bool use_graph)
     }
     WalkArgs now = base_args(h);
     set_slot(sh.slot, &now);
+    set_turns(h, sh, &now);
     const bool same = h->graph && h->graph_S == S && h->graph_grid == sh.grid.x && h->graph_block == sh.block.x &&
                       memcmp(&h->graph_args, &now, sizeof now) == 0;
     if (!same) {
@@ -720,15 +739,15 @@ static bool plan_lone(const ShapeKey& k, int word, size_t room, Slot* o)
 
 // Cycles a move takes its walker (GB300).
 // A block per line (wl_lone.cuh), words of 4 bytes or of one: 119 and 126 with up to 4 on
-// an SM, one for each scheduler; 153 .. 168 with up to 8; 217 with 10 (64x64).  So a
-// third more for every further walker on a scheduler.
+// an SM, one for each scheduler; 153 and 159 with 5 or 6, 162 and 168 with 7 or 8, 217
+// (words of a byte; 197 where they take turns) with 9 or 10 (64x64).
 // Batches (wl_walk.cuh): 191 with 7 on an SM and the lists staged (96x96), 272 with 16
 // on an SM and the lists in global memory (96x96) or 12 and staged (64x64); and what a
 // surface's lines of few up spins take longer, whose batches keep running into
 // themselves.  Whole surfaces, cycles for a move of all lines, block per line against
-// batches: 64x64 320 and 1189, 96x96 827 and 1367, 112x112 1260 and ~1350,
+// batches: 64x64 262 and 1189, 96x96 795 and 1367, 112x112 1260 and ~1350,
 // 128x128 1920 and 1536.
-constexpr double kLoneCycles[2] = {119.0, 126.0}, kLoneCrowd = 0.33, kBatchIssue = 17.0, kBatchSlowest = 600.0;
+constexpr double kLoneCycles[2] = {119.0, 126.0}, kLoneCrowd[4] = {1.0, 1.2, 1.27, 1.58}, kBatchIssue = 17.0, kBatchSlowest = 600.0;
 
 // Either a block of two warps per line, or one warp per block with 32 / S walkers,
 // whichever takes its walkers less time for a move of all of them.  The shape spreads the walkers over
@@ -758,19 +777,18 @@ wl_status plan_shape(const ShapeKey& k, Shape* sh)
     for (int word : {4, 1}) {
         if (!k.lone) break;
         auto cycles = [&](int on_sm) {
-            return kLoneCycles[word == 1] * (1.0 + kLoneCrowd * ((on_sm + 3) / 4 - 1));
+            return kLoneCycles[word == 1] * kLoneCrowd[std::min(3, std::max(0, (on_sm - 3) / 2))];
         };
-        int b = std::min((k.lines + sms - 1) / sms, 32), bps = 0;
-        Slot slot;
-        while (b > 0 && !plan_lone(k, word, room_of(b), &slot)) --b;
-        if (b > 0) CU(walk_attrs(k, slot, slot.bytes, 64, &bps));
-        b = std::min(b, bps);
-        if (b < 1) continue;
-        // whole rounds, and one of what is left
-        const int rest = (k.lines % (sms * b) + sms - 1) / sms;
-        const double cost = k.lines / (sms * b) * cycles(b) + (rest > 0 ? cycles(rest) : 0.0);
-        if (best_blocks == 0 || cost < best) {
+        const int want = std::min((k.lines + sms - 1) / sms, 32);
+        for (int b = want; b > 0; --b) {
+            Slot slot;
+            int bps = 0;
             if (!plan_lone(k, word, room_of(b), &slot)) continue;
+            CU(walk_attrs(k, slot, slot.bytes, 64, &bps));
+            if (bps < b) continue;
+            // lines that take turns keep all blocks busy to the end
+            const double cost = std::max(1.0, (double)k.lines / (sms * b)) * cycles(b);
+            if (best_blocks != 0 && cost >= best) continue;
             best = cost;
             best_blocks = b;
             sh->slot = slot;

@@ -97,6 +97,8 @@ struct WalkArgs {
     int32_t owner_mask;      // sites not staged: owner table entries - 1
     int32_t stage_perm;      // 1: the list is staged at the start of the slot
     int32_t stage_sites;     // 1: one byte per site staged (selects the kernel)
+    int32_t turns;           // block per line: turns a line's moves are walked in; 0 or 1: one
+    int32_t* turn;           // turns > 1: per line, the turns done in this launch
     int32_t lone;            // not 0: one block per line, bytes of a site's word (selects the kernel)
     int32_t pstride;         // list entries per line, N rounded up to 16 bytes
     int32_t same_f_resets;   // R > 0: extra histogram resets at unchanged f (see walk_line)

@@ -343,7 +343,9 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
     const int nbins = D.nbins;
     int64_t* lng = A.lng + D.bin_off;
     hist_t* hist = A.hist + D.bin_off;
-    int64_t end = t + A.slice_moves;
+    // a turn's share of the moves of this launch
+    const int64_t moves = A.turns > 1 && A.slice_moves > A.budget ? A.budget : A.slice_moves;
+    int64_t end = t + (A.turns > 1 ? (moves + A.turns - 1) / A.turns : moves);
     if (end > A.budget) end = A.budget;
     const int64_t C = A.C_per_bin > 0 && A.C_per_bin * nbins > A.C ? A.C_per_bin * nbins : A.C;
 
@@ -502,6 +504,29 @@ __device__ __forceinline__ void lone_walk(const WalkArgs& A, int li, int m, uint
     lone_barrier();
 }
 
+// Turn r of a line: once the block that has the turn before it, an earlier entry of the
+// queue and so running or done, is through with it.  Not taken when the slice is over,
+// or when that takes a second: the line goes on in the next slice.
+__device__ __noinline__ bool lone_turn(const WalkArgs& A, int li, int r)
+{
+    for (int n = 0; n < (1 << 20); ++n) {
+        const uint64_t now = globaltimer_ns();
+        if (A.slice_end_ns && *A.slice_end_ns && now > *A.slice_end_ns) return false;
+        if (A.deadline_ns && *A.deadline_ns && now > *A.deadline_ns) return false;
+        if (A.abort_flag && *A.abort_flag) return false;
+        int done;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(done) : "l"(A.turn + li) : "memory");
+        if (done >= r) return true;
+        __nanosleep(1000);
+    }
+    return false;
+}
+__device__ __forceinline__ void turn_done(int32_t* turn, int done)
+{
+    __threadfence();
+    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(turn), "r"(done) : "memory");
+}
+
 // One block per line: shared memory holds the words of the sites, the list, the window,
 // the ring of draws.
 //
@@ -532,16 +557,21 @@ __global__ void __launch_bounds__(kLoneThreads, TRI && WORD == 4 ? 8 : 10) lone_
     uint64_t* last = reinterpret_cast<uint64_t*>(ctl + 2);
     uint32_t* spare = reinterpret_cast<uint32_t*>(ctl + 4);
     const int N = A.g.N, pstride = A.pstride;
+    int turn = 0;
     for (;;) {
         if (th == 0) {
             const int qi = atomicAdd(A.qnext, 1);
-            ctl[0] = qi < A.nqueue ? A.order[qi] : -1;
+            const int r = A.turns > 1 ? qi / A.nqueue : 0;       // the line's turn
+            int li = A.turns > 1 ? (r < A.turns ? A.order[qi - r * A.nqueue] : -1) : qi < A.nqueue ? A.order[qi] : -1;
+            if (li >= 0 && r > 0 && !lone_turn(A, li, r)) li = -2;
+            ctl[0] = li;
             *last = 0u;
+            turn = r;
         }
         __syncthreads();
         const int li = ctl[0];
-        if (li < 0) break;
-        if (A.st[li].status == 0) {
+        if (li == -1) break;
+        if (li >= 0 && A.st[li].status == 0) {
             uint16_t* gperm = reinterpret_cast<uint16_t*>(A.perm) + (size_t)li * pstride;
             uint32_t* gsp = A.spins + (size_t)li * A.g.W;
             if (A.g.shape == kShapeOpen) {           // the border: far from either end of a byte
@@ -581,6 +611,7 @@ __global__ void __launch_bounds__(kLoneThreads, TRI && WORD == 4 ? 8 : 10) lone_
             for (int x = th; x * 32 < N; x += kLoneThreads) gsp[x] = sp[x];
         }
         __syncthreads();
+        if (th == 0 && li >= 0 && A.turns > 1) turn_done(A.turn + li, turn + 1);
     }
 }
 

@@ -78,6 +78,20 @@ def test_more_lines_than_resident_blocks(lattice, L):
     h.close()
 
 
+@pytest.mark.parametrize("slice_ms,budget", [(0, 100_003), (2, 70_001)])
+def test_lines_that_take_turns(slice_ms, budget):
+    """More lines than resident blocks, with moves enough for several turns of each;
+    a time limit ends a slice between the turns."""
+    h = wl.Handle("square", 56, seed=3, check_interval=1500, move_budget=budget, slice_ms=slice_ms)
+    h.run(1e-6, 0.8)
+    ells = [0, 1, 2, 50, 400, 1000, 1567, 1568]
+    ref = oracle_lines(LAT["square"], 56, ells, 3, 1e-6, 1500, budget)
+    for ell in ells:
+        assert_line_equal(h, ell, ref[ell], f"slice_ms={slice_ms}")
+    assert h.stats()["moves"] == budget * 1568 or h.stats()["lines_converged"] > 1
+    h.close()
+
+
 @pytest.mark.parametrize("lattice,L,tail", [("square", 10, 1), ("square", 10, 0), ("triangular", 6, 1), ("cubic", 4, 1),
                                             ("square_open", 6, 1), ("square", 130, 1)])
 def test_slices_of_odd_lengths(lattice, L, tail):
