@@ -750,11 +750,11 @@ static bool plan_lone(const ShapeKey& k, int word, size_t room, Slot* o)
 constexpr double kLoneCycles[2] = {119.0, 126.0}, kLoneCrowd[4] = {1.0, 1.2, 1.27, 1.58}, kBatchIssue = 17.0, kBatchSlowest = 600.0;
 
 // Either a block of two warps per line, or one warp per block with 32 / S walkers,
-// whichever takes its walkers less time for a move of all of them.  The shape spreads the walkers over
-// the SMs and gives each the shared memory its share of an SM leaves.  When the
-// walkers do not all fit at once with their lists staged, the lists stay in
-// global memory if that takes fewer rounds: they are read once per batch, so
-// they cost a batch one L2 latency, while a round more costs a whole walk.
+// whichever takes its walkers less time for a move of all of them.  The shape spreads the
+// walkers over the SMs and gives each the shared memory its share of an SM leaves.  When
+// walkers in batches do not all fit at once with their lists staged, the lists stay in
+// global memory if that takes fewer rounds: they are read once per batch, so they cost a
+// batch one L2 latency, while a round more costs a whole walk.
 wl_status plan_shape(const ShapeKey& k, Shape* sh)
 {
     int dev = 0, sms = 0, per_block = 0, per_sm = 0, reserved = 0;
