@@ -418,7 +418,10 @@ wl_status run_slice(wl_ctx* h, int S, const Shape& sh, bool use_graph)
     WalkArgs now = base_args(h);
     set_slot(sh.slot, &now);
     set_turns(h, sh, &now);
-    const bool same = h->graph && h->graph_S == S && h->graph_grid == sh.grid.x && h->graph_block == sh.block.x &&
+    // everything baked into the graph: the kernel (S, the acceptance rule, fields of its
+    // arguments), its launch, its arguments, and the time limit set before it
+    const bool same = h->graph && h->graph_S == S && h->graph_det == h->det && h->graph_grid == sh.grid.x &&
+                      h->graph_block == sh.block.x && h->graph_smem == sh.smem && h->graph_slice_ms == h->slice_ms &&
                       memcmp(&h->graph_args, &now, sizeof now) == 0;
     if (!same) {
         if (h->graph) cudaGraphExecDestroy(h->graph);
@@ -433,8 +436,11 @@ wl_status run_slice(wl_ctx* h, int S, const Shape& sh, bool use_graph)
         cudaGraphDestroy(g);
         if (e != cudaSuccess) return fail(WL_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
         h->graph_S = S;
+        h->graph_det = h->det;
         h->graph_grid = sh.grid.x;
         h->graph_block = sh.block.x;
+        h->graph_smem = sh.smem;
+        h->graph_slice_ms = h->slice_ms;
         memcpy(&h->graph_args, &now, sizeof now);
     }
     CU(cudaGraphLaunch(h->graph, h->s));

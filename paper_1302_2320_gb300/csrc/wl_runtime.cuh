@@ -119,8 +119,10 @@ struct wl_ctx {
     int nqueue = 0;
     // captured slice graph
     cudaGraphExec_t graph = nullptr;
-    int graph_S = -1;
+    int graph_S = -1, graph_det = -1;
     unsigned graph_grid = 0, graph_block = 0;
+    size_t graph_smem = 0;
+    int64_t graph_slice_ms = 0;
     wl::WalkArgs graph_args{};          // arguments baked into the captured graph
 };
 

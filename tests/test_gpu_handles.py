@@ -1,0 +1,50 @@
+"""A handle that is kept: options that change between its walks.
+
+Every walk is a function of its lattice, options and seed alone, so a handle that
+has walked before gives what a fresh one gives, and an option set between two
+walks holds for the second.
+"""
+import numpy as np
+import pytest
+
+import paper_1302_2320_gb300 as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    wl.build()
+
+
+def _assert_same(a, b, ells, what):
+    for ell in ells:
+        x, y = a.line_state(ell), b.line_state(ell)
+        for key in x:
+            assert np.array_equal(x[key], y[key]), (what, ell, key)
+
+
+@pytest.mark.parametrize("lattice,L,mapping", [("square", 8, 0), ("triangular", 6, 32), ("square", 8, 8)])
+@pytest.mark.parametrize("first", [0, 1])
+def test_both_acceptance_rules_on_one_handle(lattice, L, mapping, first):
+    opt = dict(seed=3, check_interval=500, move_budget=30_000, mapping=mapping)
+    kept = wl.Handle(lattice, L, deterministic=first, **opt)
+    kept.run(1e-6, 0.8)
+    kept.reset()
+    kept.set_option("deterministic", 1 - first)
+    kept.run(1e-6, 0.8)
+    fresh = wl.Handle(lattice, L, deterministic=1 - first, **opt)
+    fresh.run(1e-6, 0.8)
+    _assert_same(kept, fresh, range(1, kept.lines, 5), f"deterministic {first} then {1 - first}")
+
+
+def test_a_shorter_time_limit_of_a_slice_holds_from_the_next_walk_on():
+    """2^18 moves a line take 15 ms or more: one slice of 10 s, and many of 1 ms (two
+    launches a slice, two for the initialisation)."""
+    h = wl.Handle("square", 16, seed=2, check_interval=1000, move_budget=1 << 18, slice_moves=1 << 40, slice_ms=10_000)
+    h.run(1e-6, 0.8)
+    assert h.stats()["launches"] == 4
+    h.reset()
+    h.set_option("slice_ms", 1)
+    h.run(1e-6, 0.8)
+    assert h.stats()["launches"] >= 2 + 2 * 4
