@@ -100,69 +100,77 @@ __global__ void __launch_bounds__(32) init_kernel(const InitArgs A)
 }
 
 // ---------------------------------------------------------------------------
-// A caller's own walker state (wl_walk_noalloc): one warp per running line checks
-// that the list is a permutation whose first l entries are the up spins and that
-// k is theirs.  The walkers take this for granted; a line that fails gets the
-// status and the flag of a broken invariant and is not walked.
+// A caller's own walker state (wl_walk_noalloc): one block per running line checks
+// that the list is a permutation whose first l entries are the up spins, that k is
+// theirs and that there is a move to make.  The walkers take this for granted: every
+// bin and site they reach, and with it every address, follows from it.  A line that
+// fails gets the status and the flag of a broken invariant and is not walked.
+// A site seen twice shows in a bit per site (up to 128 KB of shared memory).
 // ---------------------------------------------------------------------------
+constexpr int kCheckThreads = 128;
+
 template <int LAT, typename IDX>
-__global__ void check_state_kernel(const InitArgs A, int32_t* flags)
+__global__ void __launch_bounds__(kCheckThreads) check_state_kernel(const InitArgs A, int32_t* flags)
 {
-    const int li = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (li >= A.nlines || A.st[li].status != 0) return;
+    extern __shared__ uint32_t seen[];
+    __shared__ int twice_all;
+    const int li = blockIdx.x;
+    if (A.st[li].status != 0) return;
     const LineDesc D = A.desc[li];
     const int N = A.g.N;
     const IDX* perm = reinterpret_cast<const IDX*>(A.perm) + (size_t)li * A.pstride;
     const uint32_t* sp = A.spins + (size_t)li * A.g.W;
     constexpr int z = Coord<LAT>::z;
-    int up = 0, twice = 0, bad = 0;
-    // every entry a site of the right spin; with l up spins in all and the sums
-    // and sums of squares of 0 .. N-1 the entries are all different in practice
-    int64_t s1 = 0, s2 = 0;
-    for (int n = lane; n < N; n += 32) {
+    for (int w = threadIdx.x; w < A.g.W; w += kCheckThreads) seen[w] = 0u;
+    if (threadIdx.x == 0) twice_all = 0;
+    __syncthreads();
+    int twice = 0, bad = D.ell < 1 || A.st[li].t < 0;
+    for (int n = threadIdx.x; n < N; n += kCheckThreads) {
         const uint32_t e = (uint32_t)perm[n];
         if (e >= (uint32_t)N) {
             bad = 1;
-            continue;
+        } else {
+            const uint32_t bit = 1u << (e & 31u);
+            bad |= (atomicOr(&seen[e >> 5], bit) & bit) != 0u;
+            bad |= spin_at(sp, e) != (n < D.ell ? 1u : 0u);
         }
-        bad |= spin_at(sp, e) != (n < D.ell ? 1u : 0u);
-        s1 += (int64_t)e - n;
-        s2 += (int64_t)e * e - (int64_t)n * n;
         uint32_t nb[z];
         neighbours<LAT>(A.g, (uint32_t)n, nb);
         const uint32_t sn = spin_at(sp, (uint32_t)n);
-        up += (int)sn;
 #pragma unroll
         for (int q = 0; q < z; ++q) twice += sn != spin_at(sp, nb[q]);
     }
-    up = group_sum<32>(0xffffffffu, up);
     twice = group_sum<32>(0xffffffffu, twice);
-    s1 = group_sum<32>(0xffffffffu, s1);
-    s2 = group_sum<32>(0xffffffffu, s2);
-    bad |= up != D.ell || s1 != 0 || s2 != 0 || A.st[li].k != twice / 2 || A.st[li].t < 0;
-    if (__any_sync(0xffffffffu, bad) && lane == 0) {
+    if ((threadIdx.x & 31) == 0) atomicAdd(&twice_all, twice);
+    __syncthreads();
+    bad |= A.st[li].k != twice_all / 2;
+    if (__syncthreads_or(bad) && threadIdx.x == 0) {
         A.st[li].status = 3;
         atomicOr(flags, 8);
     }
 }
 
+template <int LAT, typename IDX>
+static cudaError_t check_one(const InitArgs& a, int32_t* flags, cudaStream_t s)
+{
+    const size_t bits = (size_t)a.g.W * 4;
+    if (bits > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(check_state_kernel<LAT, IDX>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+        if (e != cudaSuccess) return e;
+    }
+    check_state_kernel<LAT, IDX><<<a.nlines, kCheckThreads, bits, s>>>(a, flags);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_check_state(int lattice, bool idx16, const InitArgs& a, int32_t* flags, cudaStream_t s)
 {
     clear_stale_error();
-    const int warps = 4;
-    const dim3 grid((a.nlines + warps - 1) / warps), block(32 * warps);
-    if (lattice == kSquare) {
-        if (idx16) check_state_kernel<kSquare, uint16_t><<<grid, block, 0, s>>>(a, flags);
-        else check_state_kernel<kSquare, uint32_t><<<grid, block, 0, s>>>(a, flags);
-    } else if (lattice == kTriangular) {
-        if (idx16) check_state_kernel<kTriangular, uint16_t><<<grid, block, 0, s>>>(a, flags);
-        else check_state_kernel<kTriangular, uint32_t><<<grid, block, 0, s>>>(a, flags);
-    } else {
-        if (idx16) check_state_kernel<kCubic, uint16_t><<<grid, block, 0, s>>>(a, flags);
-        else check_state_kernel<kCubic, uint32_t><<<grid, block, 0, s>>>(a, flags);
-    }
-    return cudaGetLastError();
+    if (lattice == kSquare)
+        return idx16 ? check_one<kSquare, uint16_t>(a, flags, s) : check_one<kSquare, uint32_t>(a, flags, s);
+    if (lattice == kTriangular)
+        return idx16 ? check_one<kTriangular, uint16_t>(a, flags, s) : check_one<kTriangular, uint32_t>(a, flags, s);
+    return idx16 ? check_one<kCubic, uint16_t>(a, flags, s) : check_one<kCubic, uint32_t>(a, flags, s);
 }
 
 template <int LAT, typename IDX>

@@ -195,3 +195,60 @@ def test_thermo_sums_from_hot_to_cold(lattice, L, z):
     for i in range(len(T)):
         assert np.array_equal(h.thermo(T[i:i + 1], H), got[i:i + 1])
     h.close()
+
+
+def _set_line(buf, i, lattice, L, up, entries):
+    """Line i of the caller's buffers: the spins up at `up`, its k, the list `entries`
+    followed by the sites that are down."""
+    N = buf.N
+    spins = np.zeros(N, dtype=np.uint8)
+    spins[list(up)] = 1
+    g = spins.reshape(L, L).astype(int)
+    k = int((g != np.roll(g, 1, 0)).sum() + (g != np.roll(g, 1, 1)).sum())
+    words = np.zeros(buf.W, dtype=np.uint32)
+    np.bitwise_or.at(words, np.arange(N) >> 5, spins.astype(np.uint32) << (np.arange(N, dtype=np.uint32) & 31))
+    down = np.flatnonzero(spins == 0)
+    perm = np.concatenate([np.array(entries), down]).astype(np.int64)
+    wide = buf.perm.element_size() == 4
+    perm = perm.astype(np.uint32).view(np.int32) if wide else perm.astype(np.uint16).view(np.int16)
+    import torch
+    buf.perm[i * buf.P:i * buf.P + N] = torch.from_numpy(perm).to(buf.perm.device)
+    buf.spins[i * buf.W:(i + 1) * buf.W] = torch.from_numpy(words.view(np.int32)).to(buf.spins.device)
+    buf.state[i * 9] = k
+
+
+@pytest.mark.parametrize("L,mapping", [(8, 0), (8, 8), (260, 0), (700, 0)])
+def test_noalloc_refuses_equal_entries_whose_sums_are_right(L, mapping):
+    """The sites 0, 4, 5 twice in the place of 0, 1, 2, 4, 5, 6: as many up spins, the
+    same sum and the same sum of squares, and no line's list."""
+    import torch
+    f = _fn()
+    up, twice = [0, 1, 2, 4, 5, 6], [0, 4, 5, 0, 4, 5]
+    assert sum(up) == sum(twice) and sum(x * x for x in up) == sum(x * x for x in twice)
+    buf = Buffers("square", L, 6, 2)
+    args = (wl.WL_SQUARE, L, 6, 2, 3, 1, 1e-6, 0.8, 500)
+    assert f(*args, 0, mapping, 1, *buf.ptrs(), buf.stream) == wl.WL_ENOTCONVERGED
+    torch.cuda.synchronize()
+    _set_line(buf, 0, "square", L, up, up)                      # a line's state: walked
+    assert f(*args, 300, mapping, 0, *buf.ptrs(), buf.stream) == wl.WL_ENOTCONVERGED
+    torch.cuda.synchronize()
+    assert buf.line(0)["sc"][1] == 300 and sorted(buf.line(0)["perm"]) == list(range(L * L))
+    _set_line(buf, 0, "square", L, up, twice)
+    assert f(*args, 600, mapping, 0, *buf.ptrs(), buf.stream) not in (wl.WL_OK, wl.WL_ENOTCONVERGED)
+    torch.cuda.synchronize()
+    assert buf.line(0)["sc"][6] == 3 and buf.line(0)["sc"][1] == 300
+
+
+def test_noalloc_refuses_a_running_line_without_up_spins():
+    """l = 0 has no move and is done from the start; a state that has it running is none."""
+    import torch
+    f = _fn()
+    buf = Buffers("square", 8, 0, 2)
+    args = (wl.WL_SQUARE, 8, 0, 2, 3, 1, 1e-6, 0.8, 500)
+    assert f(*args, 0, 0, 1, *buf.ptrs(), buf.stream) == wl.WL_ENOTCONVERGED
+    torch.cuda.synchronize()
+    buf.state[2] = 10**6                                       # ln f = 1 in units of ln f_min
+    buf.state[6] = 0
+    assert f(*args, 300, 0, 0, *buf.ptrs(), buf.stream) not in (wl.WL_OK, wl.WL_ENOTCONVERGED)
+    torch.cuda.synchronize()
+    assert buf.line(0)["sc"][6] == 3 and buf.line(0)["sc"][1] == 0
