@@ -88,8 +88,6 @@ int line_nbins(const LatInfo& g, int ell)
     return (int)(khi / g.kstep + 1);
 }
 
-size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
-
 Layout make_layout(const LatInfo& g)
 {
     Layout lo;
@@ -383,7 +381,7 @@ wl_status persistent_shape(wl_ctx* h, int S, int active, Shape* sh)
 static void set_turns(wl_ctx* h, const Shape& sh, WalkArgs* a)
 {
     a->turns = 1;
-    if (!sh.slot.lone || h->nqueue <= (int)sh.grid.x) return;
+    if (!sh.slot.lone || h->nqueue <= (int)sh.grid) return;
     const int64_t moves = std::min(a->slice_moves, a->budget);
     if (moves > (1 << 26)) return;       // turns of more than a second
     a->turns = (int)std::max<int64_t>(1, std::min<int64_t>(8, moves >> 14));
@@ -420,8 +418,8 @@ wl_status run_slice(wl_ctx* h, int S, const Shape& sh, bool use_graph)
     set_turns(h, sh, &now);
     // everything baked into the graph: the kernel (S, the acceptance rule, fields of its
     // arguments), its launch, its arguments, and the time limit set before it
-    const bool same = h->graph && h->graph_S == S && h->graph_det == h->det && h->graph_grid == sh.grid.x &&
-                      h->graph_block == sh.block.x && h->graph_smem == sh.smem && h->graph_slice_ms == h->slice_ms &&
+    const bool same = h->graph && h->graph_S == S && h->graph_det == h->det && h->graph_grid == sh.grid &&
+                      h->graph_block == sh.block && h->graph_smem == sh.smem && h->graph_slice_ms == h->slice_ms &&
                       memcmp(&h->graph_args, &now, sizeof now) == 0;
     if (!same) {
         if (h->graph) cudaGraphExecDestroy(h->graph);
@@ -437,8 +435,8 @@ wl_status run_slice(wl_ctx* h, int S, const Shape& sh, bool use_graph)
         if (e != cudaSuccess) return fail(WL_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
         h->graph_S = S;
         h->graph_det = h->det;
-        h->graph_grid = sh.grid.x;
-        h->graph_block = sh.block.x;
+        h->graph_grid = sh.grid;
+        h->graph_block = sh.block;
         h->graph_smem = sh.smem;
         h->graph_slice_ms = h->slice_ms;
         memcpy(&h->graph_args, &now, sizeof now);
@@ -663,35 +661,6 @@ wl_status prepare(wl_ctx* h, double ln_f_min, double flatness, cudaStream_t afte
     return WL_OK;
 }
 
-// A walker's slot: the list (staged or not), the sites, the window, the step
-// records.  The window is what is left of `room` bytes, up to the whole line; a
-// guard on both sides of it keeps every address inside the slot even where a
-// caller's own state (wl_walk_noalloc) is not one of the line's.
-static bool plan_slot(const ShapeKey& k, bool sites, bool perm, size_t room, Slot* o)
-{
-    constexpr int kGuard = 8 * 8 * (12 + 1);      // kSub steps of the largest bin step, in bytes
-    constexpr int kOwners = 4096;
-    // room for the margins of both edges and a walk between them
-    const int min_win = std::min(k.max_bins, k.lattice == kTriangular || k.lattice == kCubic ? 384 : 256);
-    Slot s;
-    size_t at = perm ? (size_t)k.pstride * (k.idx16 ? 2 : 4) : 0;
-    s.stage_perm = perm;
-    s.stage_sites = sites;
-    s.off_sites = (int)at;
-    s.owner_mask = kOwners - 1;
-    at += sites ? ((size_t)k.N + 31) / 32 * 32 : (size_t)kOwners;
-    at = std::max<size_t>(align16(at), kGuard);
-    s.off_win = (int)at;
-    const size_t after = std::max<size_t>(align16((size_t)k.S * kStepBytes), kGuard);
-    if (at + (size_t)min_win * 8 + 16 + after > room) return false;
-    s.win = (int)std::min<size_t>((size_t)k.max_bins, (room - 16 - at - after) / 8);
-    at += align16((size_t)s.win * 8);
-    s.off_rec = (int)at;
-    s.bytes = (int)align16(at + after);
-    *o = s;
-    return true;
-}
-
 void set_slot(const Slot& slot, WalkArgs* a)
 {
     a->slot_bytes = slot.bytes;
@@ -714,128 +683,26 @@ static cudaError_t walk_attrs(const ShapeKey& k, const Slot& slot, size_t smem, 
     return walk_kernel_attrs(k.lattice, k.S, k.det, k.idx16, smem, threads, a, bps);
 }
 
-// The slot of a line with a block of its own (wl_lone.cuh): the words of the sites
-// by code, the list, the window, the ring.
-static bool plan_lone(const ShapeKey& k, int word, size_t room, Slot* o)
-{
-    if (!k.idx16) return false;
-    const bool open = k.lattice == kSquareOpen;      // with a border around it
-    size_t stride = 1;
-    while (stride < (size_t)k.L + (open ? 1 : 0)) stride <<= 1;
-    const size_t codes = (k.lattice == kCubic ? stride : 1) * stride * ((size_t)k.L + (open ? 2 : 0));
-    if (word * codes > 65536) return false;          // a list entry holds an address
-    // two margins of 16 steps of the largest bin step, and 64 bins to walk between them
-    const int zb = k.lattice == kSquareOpen ? 8 : k.lattice == kTriangular || k.lattice == kCubic ? 6 : 4;
-    const int min_win = std::min(k.max_bins, 32 * zb + 64);
-    Slot s;
-    s.lone = word;
-    size_t at = align16(word * codes);
-    s.off_perm = (int)at;
-    at += (size_t)k.pstride * 2;
-    s.off_win = (int)at;
-    const size_t ring = (96 + 3) * 32 + 16 + 128;   // the draws, control words, spare words
-    if (at + (size_t)min_win * 8 + 16 + ring > room) return false;
-    s.win = (int)std::min<size_t>((size_t)k.max_bins, (room - 16 - at - ring) / 8);
-    at += align16((size_t)s.win * 8);
-    s.off_rec = (int)at;
-    s.bytes = (int)(at + ring);
-    *o = s;
-    return true;
-}
-
-// Cycles a move takes its walker (GB300).
-// A block per line (wl_lone.cuh), words of 4 bytes or of one: 119 and 126 with up to 4 on
-// an SM, one for each scheduler; 153 and 159 with 5 or 6, 162 and 168 with 7 or 8, 217
-// (words of a byte; 197 where they take turns) with 9 or 10 (64x64).
-// Batches (wl_walk.cuh): 191 with 7 on an SM and the lists staged (96x96), 272 with 16
-// on an SM and the lists in global memory (96x96) or 12 and staged (64x64); and what a
-// surface's lines of few up spins take longer, whose batches keep running into
-// themselves.  Whole surfaces, cycles for a move of all lines, block per line against
-// batches: 64x64 262 and 1189, 96x96 795 and 1367, 112x112 1260 and ~1350,
-// 128x128 1920 and 1536.
-constexpr double kLoneCycles[2] = {119.0, 126.0}, kLoneCrowd[4] = {1.0, 1.2, 1.27, 1.58}, kBatchIssue = 17.0, kBatchSlowest = 600.0;
-
-// Either a block of two warps per line, or one warp per block with 32 / S walkers,
-// whichever takes its walkers less time for a move of all of them.  The shape spreads the
-// walkers over the SMs and gives each the shared memory its share of an SM leaves.  When
-// walkers in batches do not all fit at once with their lists staged, the lists stay in
-// global memory if that takes fewer rounds: they are read once per batch, so they cost a
-// batch one L2 latency, while a round more costs a whole walk.
 wl_status plan_shape(const ShapeKey& k, Shape* sh)
 {
-    int dev = 0, sms = 0, per_block = 0, per_sm = 0, reserved = 0;
+    int dev = 0;
+    Gpu gpu{};
     CU(cudaGetDevice(&dev));
-    CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    CU(cudaDeviceGetAttribute(&per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    CU(cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
-    CU(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
-    const int groups = 32 / k.S;
-    const int need = (k.lines + groups - 1) / groups;       // blocks wanted
-    const int want = std::min((need + sms - 1) / sms, 32);  // per SM
-    auto room_of = [&](int blocks) {   // bytes of a block with this many on an SM
-        const int b = std::min(per_block, per_sm / blocks - reserved - 128) / 128 * 128;
-        return b > 0 ? (size_t)b : (size_t)0;
-    };
-    double best = 0.0;
-    int best_blocks = 0;
-    // a block per line: as many as fit, each with its share of the shared memory; words of
-    // a byte where that makes room for enough more of them (wl_lone.cuh)
-    for (int word : {4, 1}) {
-        if (!k.lone) break;
-        auto cycles = [&](int on_sm) {
-            return kLoneCycles[word == 1] * kLoneCrowd[std::min(3, std::max(0, (on_sm - 3) / 2))];
-        };
-        const int want = std::min((k.lines + sms - 1) / sms, 32);
-        for (int b = want; b > 0; --b) {
-            Slot slot;
-            int bps = 0;
-            if (!plan_lone(k, word, room_of(b), &slot)) continue;
-            CU(walk_attrs(k, slot, slot.bytes, 64, &bps));
-            if (bps < b) continue;
-            // lines that take turns keep all blocks busy to the end
-            const double cost = std::max(1.0, (double)k.lines / (sms * b)) * cycles(b);
-            if (best_blocks != 0 && cost >= best) continue;
-            best = cost;
-            best_blocks = b;
-            sh->slot = slot;
-            sh->grid = dim3(std::min(k.lines, sms * b));
-            sh->block = dim3(64);
-            sh->smem = slot.bytes;
-        }
-    }
-    auto room = [&](int blocks) {      // bytes per walker with this many blocks on an SM
-        const int b = std::min(per_block, per_sm / blocks - reserved) / 128 * 128;
-        return b > 0 ? (size_t)b / groups / 16 * 16 : (size_t)0;
-    };
-    struct Mode {
-        bool sites, perm;
-        double cycles;                 // a lone walker's cycles per move, to weigh rounds
-    };
-    const Mode modes[3] = {{true, true, 190.0}, {true, false, 200.0}, {false, false, 250.0}};
-    for (const Mode& m : modes) {
-        if (m.sites && !k.idx16) continue;
-        int b = want;
-        Slot slot;
-        while (b > 0 && !plan_slot(k, m.sites, m.perm, room(b), &slot)) --b;
-        if (b == 0) continue;
+    CU(cudaDeviceGetAttribute(&gpu.sms, cudaDevAttrMultiProcessorCount, dev));
+    CU(cudaDeviceGetAttribute(&gpu.per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    CU(cudaDeviceGetAttribute(&gpu.per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    CU(cudaDeviceGetAttribute(&gpu.reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
+    cudaError_t e = cudaSuccess;
+    auto resident = [&](const Slot& slot, size_t smem, int threads) {
         int bps = 0;
-        CU(walk_attrs(k, slot, (size_t)groups * slot.bytes, 32, &bps));
-        b = std::min(b, bps);
-        if (b < 1) continue;
-        const double rounds = (double)((need + sms * b - 1) / (sms * b));
-        const double cost = rounds * std::max(m.cycles, kBatchIssue * b * groups) + kBatchSlowest;
-        if (best_blocks == 0 || cost < best) {
-            if (!plan_slot(k, m.sites, m.perm, room(b), &slot)) continue;
-            best = cost;
-            best_blocks = b;
-            sh->slot = slot;
-            sh->grid = dim3(std::max(1, std::min(need, sms * b)));
-            sh->block = dim3(32);
-            sh->smem = (size_t)groups * slot.bytes;
-        }
+        e = walk_attrs(k, slot, smem, threads, &bps);
+        return e == cudaSuccess ? bps : -1;
+    };
+    switch (plan_shape(k, gpu, resident, sh)) {
+    case Planned::ok: return WL_OK;
+    case Planned::none_fits: return fail(WL_ECUDA, "no walker shape fits shared memory (S=%d)", k.S);
+    default: return fail(WL_ECUDA, "walker attributes: %s", cudaGetErrorString(e));
     }
-    if (best_blocks == 0) return fail(WL_ECUDA, "no walker shape fits shared memory (S=%d)", k.S);
-    return WL_OK;
 }
 
 wl_status choose_shape(wl_ctx* h, int* S, Shape* sh)

@@ -7,18 +7,14 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "wl_plan.h"
+
 namespace wl {
 
 using hist_t = uint64_t;                       // histogram word: count, bit 63 = ever visited
 constexpr hist_t kVisited = 1ull << 63;
 constexpr int kTableN = 4096;
 constexpr int kTableBytes = kTableN * 4;     // entries 1..4095 as u32; entry 0 is 2^32
-
-// kSquareP2: the square lattice when L is a power of two (coordinates by
-// shift and mask); the same lattice and bond set as kSquare.
-// kSquareOpen: the square lattice with open boundaries (sites on an edge have
-// fewer neighbours; k takes every value, so bins have step 1).
-enum LatticeType : int { kSquare = 0, kTriangular = 1, kCubic = 2, kSquareP2 = 3, kSquareOpen = 4 };
 
 // Per-line scalar state (device, one per walked line).
 struct LineState {
@@ -33,16 +29,11 @@ struct LineState {
     int64_t batches;   // speculative batches evaluated (diagnostic)
 };
 
-constexpr int kStepBytes = 40;     // shared bytes of a lane's step record (Steps in wl_walk.cuh)
-
 struct LineDesc {
     int64_t bin_off;   // first bin of this line in the ragged lng/hist arrays
     int32_t ell;       // number of up spins
     int32_t nbins;     // bins k = 0, 2, ..., 2*(nbins-1)
 };
-
-// A lattice at run time, whatever its kernel specialisation.
-enum LatticeShape : int { kShapeSquare = 0, kShapeTriangular = 1, kShapeCubic = 2, kShapeOpen = 3 };
 
 struct Geo {
     int type, L, N, NB, W;   // W = 32-bit words of packed spins per line (multiple of 4)
@@ -90,7 +81,7 @@ struct WalkArgs {
     float inv_u;             // 1 / u, production acceptance
     uint32_t seed;
     int32_t flat_pm;         // flatness fraction x in 1/1000
-    // a walker's slot of shared memory (plan_slot in wl_api.cu)
+    // a walker's slot of shared memory (plan_slot, plan_lone in wl_plan.h)
     int32_t slot_bytes;
     int32_t off_perm, off_sites, off_win, off_rec;
     int32_t win_bins;        // bins of ln g held in the window

@@ -25,34 +25,6 @@ struct Layout {
     std::vector<LineDesc> desc;
 };
 
-// A walker's slot of shared memory.
-struct Slot {
-    int bytes = 0, off_perm = 0, off_sites = 0, off_win = 0, off_rec = 0;
-    int win = 0;                 // bins of the ln g window
-    int owner_mask = 0;
-    bool stage_sites = false, stage_perm = false;
-    int lone = 0;            // a block per line: bytes of a site's word; else 0
-};
-
-// Launch shape of the persistent form for S lanes per walker.
-struct Shape {
-    dim3 grid, block;
-    size_t smem = 0;
-    Slot slot;
-};
-
-// What the shape of a launch depends on.
-struct ShapeKey {
-    int lattice;         // kernel specialisation (LatticeType)
-    int S;               // lanes per walker
-    bool det, idx16;
-    int L, N, pstride;
-    int max_bins;        // bins of the largest line
-    int lines;           // walkers wanted at once
-    bool lone;           // few lines may get a block each (wl_lone.cuh)
-};
-
-
 }  // namespace rt
 }  // namespace wl
 

@@ -733,7 +733,7 @@ __device__ __forceinline__ void sites_store(uint32_t* sp, const uint8_t* own, in
 // Persistent walker: every group pops lines from the work queue until it is
 // empty.  With one group and a one-entry queue the same kernel is the plain
 // one-launch-per-line form.  A group's slot of shared memory: the list (when
-// staged), the window, the sites, the step records (plan_slot in wl_api.cu).
+// staged), the window, the sites, the step records (plan_slot in wl_plan.h).
 template <int LAT, int S, bool DET, typename IDX, bool BYTES>
 __global__ void walk_kernel(const WalkArgs A)
 {
