@@ -62,12 +62,11 @@ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 // records.  The window is what is left of `room` bytes, up to the whole line; a
 // guard on both sides of it keeps every address inside the slot even where a
 // caller's own state (wl_walk_noalloc) is not one of the line's.
-inline bool plan_slot(const ShapeKey& k, bool sites, bool perm, size_t room, Slot* o)
+inline bool plan_slot(const ShapeKey& k, bool sites, bool perm, size_t room, int least_win, Slot* o)
 {
     constexpr int kGuard = 8 * 8 * (12 + 1);      // kSub steps of the largest bin step, in bytes
     constexpr int kOwners = 4096;
-    // room for the margins of both edges and a walk between them
-    const int min_win = std::min(k.max_bins, k.lattice == kTriangular || k.lattice == kCubic ? 384 : 256);
+    const int min_win = std::min(k.max_bins, least_win);
     Slot s;
     size_t at = perm ? (size_t)k.pstride * (k.idx16 ? 2 : 4) : 0;
     s.stage_perm = perm;
@@ -186,26 +185,35 @@ Planned plan_shape(const ShapeKey& k, const Gpu& gpu, Resident&& resident, Shape
         double cycles;                 // a lone walker's cycles per move, to weigh rounds
     };
     const Mode modes[3] = {{true, true, 190.0}, {true, false, 200.0}, {false, false, 250.0}};
-    for (const Mode& m : modes) {
-        if (m.sites && !k.idx16) continue;
-        int b = want;
-        Slot slot;
-        while (b > 0 && !plan_slot(k, m.sites, m.perm, room(b), &slot)) --b;
-        if (b == 0) continue;
-        const int bps = resident(slot, (size_t)groups * slot.bytes, 32);
-        if (bps < 0) return Planned::unknown;
-        b = std::min(b, bps);
-        if (b < 1) continue;
-        const double rounds = (double)((need + sms * b - 1) / (sms * b));
-        const double cost = rounds * std::max(m.cycles, kBatchIssue * b * groups) + kBatchSlowest;
-        if (best_blocks == 0 || cost < best) {
-            if (!plan_slot(k, m.sites, m.perm, room(b), &slot)) continue;
-            best = cost;
-            best_blocks = b;
-            sh->slot = slot;
-            sh->grid = (unsigned)std::max(1, std::min(need, sms * b));
-            sh->block = 32;
-            sh->smem = (size_t)groups * slot.bytes;
+    // Windows of 384 bins where there are six neighbours, 256 otherwise; with one lane a
+    // walker, of which 32 share a block, 384 may leave room for none (triangular from
+    // 58x58 on, cubic from 15^3): then 256, still more than twice the two margins of 56.
+    const bool six = k.lattice == kTriangular || k.lattice == kCubic;
+    bool fits = false;
+    for (const int least_win : {six ? 384 : 256, 256}) {
+        if (fits) break;
+        for (const Mode& m : modes) {
+            if (m.sites && !k.idx16) continue;
+            int b = want;
+            Slot slot;
+            while (b > 0 && !plan_slot(k, m.sites, m.perm, room(b), least_win, &slot)) --b;
+            if (b == 0) continue;
+            const int bps = resident(slot, (size_t)groups * slot.bytes, 32);
+            if (bps < 0) return Planned::unknown;
+            b = std::min(b, bps);
+            if (b < 1) continue;
+            fits = true;
+            const double rounds = (double)((need + sms * b - 1) / (sms * b));
+            const double cost = rounds * std::max(m.cycles, kBatchIssue * b * groups) + kBatchSlowest;
+            if (best_blocks == 0 || cost < best) {
+                if (!plan_slot(k, m.sites, m.perm, room(b), least_win, &slot)) continue;
+                best = cost;
+                best_blocks = b;
+                sh->slot = slot;
+                sh->grid = (unsigned)std::max(1, std::min(need, sms * b));
+                sh->block = 32;
+                sh->smem = (size_t)groups * slot.bytes;
+            }
         }
     }
     return best_blocks ? Planned::ok : Planned::none_fits;

@@ -252,3 +252,29 @@ def test_noalloc_refuses_a_running_line_without_up_spins():
     assert f(*args, 300, 0, 0, *buf.ptrs(), buf.stream) not in (wl.WL_OK, wl.WL_ENOTCONVERGED)
     torch.cuda.synchronize()
     assert buf.line(0)["sc"][6] == 3 and buf.line(0)["sc"][1] == 0
+
+
+# one lane a walker, with more sites than 32 walkers' windows of 384 bins leave room for
+@pytest.mark.parametrize("lattice,L", [("triangular", 58), ("cubic", 15), ("triangular", 128)])
+@pytest.mark.parametrize("form", [0, 1])
+def test_one_lane_with_six_neighbours(lattice, L, form):
+    N = L ** 3 if lattice == "cubic" else L * L
+    ells = [1, 40, N // 2]
+    h = walk(lattice, L, ells, 5, 1e-6, 300, 2_001, mapping=1, form=form)
+    ref = oracle_lines(LAT[lattice], L, ells, 5, 1e-6, 300, 2_001)
+    for ell in ells:
+        assert_line_equal(h, ell, ref[ell], f"{lattice} {L} form={form}")
+    h.close()
+
+
+def test_noalloc_with_one_lane_and_six_neighbours():
+    import torch
+    f = _fn()
+    buf = Buffers("cubic", 15, 1200, 3)
+    assert f(wl.WL_SIMPLE_CUBIC, 15, 1200, 3, 5, 1, 1e-6, 0.8, 300, 2_001, 1, 1, *buf.ptrs(), buf.stream) == wl.WL_ENOTCONVERGED
+    torch.cuda.synchronize()
+    ref = oracle_lines(oracle.CUBIC, 15, range(1200, 1203), 5, 1e-6, 300, 2_001)
+    for i in range(3):
+        got = buf.line(i)
+        for key in ("perm", "spins", "lng", "hist", "visited"):
+            assert np.array_equal(got[key], getattr(ref[1200 + i], key)), (i, key)
