@@ -47,7 +47,6 @@ namespace wl {
 constexpr int kRing = 96;                  // steps (3 batches of 32)
 constexpr int kRingMore = 3;               // the first records again past the end: a step reads up to 3 ahead
 constexpr int kLoneThreads = 64;           // one warp walks, one draws
-constexpr uint32_t kLow = 1024u;           // address at which the shared memory of a block starts
 
 // The lattice is a run-time matter but for the second axis of the triangular one's
 // diagonals (TRI): requests for different lattices that share an SM then run the same
@@ -539,7 +538,7 @@ __global__ void __launch_bounds__(kLoneThreads, TRI && WORD == 4 ? 8 : 10) lone_
 {
     extern __shared__ __align__(16) uint8_t smem[];
     const int th = threadIdx.x, warp = th >> 5, lane = th & 31;
-    if ((uint32_t)__cvta_generic_to_shared(smem) != kLow) {      // never
+    if ((uint32_t)__cvta_generic_to_shared(smem) != kLow) {      // never: plan_shape
         if (th == 0) atomicOr(A.flags, 8);
         return;
     }

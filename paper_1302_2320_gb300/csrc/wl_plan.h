@@ -20,6 +20,7 @@ enum LatticeType : int { kSquare = 0, kTriangular = 1, kCubic = 2, kSquareP2 = 3
 enum LatticeShape : int { kShapeSquare = 0, kShapeTriangular = 1, kShapeCubic = 2, kShapeOpen = 3 };
 
 constexpr int kStepBytes = 40;     // shared bytes of a lane's step record (Steps in wl_walk.cuh)
+constexpr uint32_t kLow = 1024u;   // address at which a block's shared memory starts (wl_lone.cuh): behind the system's share
 
 namespace rt {
 
@@ -154,7 +155,7 @@ Planned plan_shape(const ShapeKey& k, const Gpu& gpu, Resident&& resident, Shape
     // a block per line: as many as fit, each with its share of the shared memory; words of
     // a byte where that makes room for enough more of them (wl_lone.cuh)
     for (int word : {4, 1}) {
-        if (!k.lone) break;
+        if (!k.lone || gpu.reserved != (int)kLow) break;      // its addresses count from kLow
         auto cycles = [&](int on_sm) {
             return kLoneCycles[word == 1] * kLoneCrowd[std::min(3, std::max(0, (on_sm - 3) / 2))];
         };

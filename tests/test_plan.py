@@ -78,3 +78,12 @@ def test_every_lane_count_has_a_shape(planner, lattice, L, S):
         zb = {"square": 4, "square_open": 8}.get(lattice, 6)
         N = L ** 3 if lattice == "cubic" else L * L
         assert sh.slot.win >= min(Z[lattice] * (N // 2) // 2 + 1, 2 * 8 * (zb + 1) + 32)
+
+
+def test_a_block_per_line_only_where_shared_memory_starts_at_its_address(planner):
+    """Its list entries are addresses past 1024, the share the system keeps of a block."""
+    for lattice, L in (("square", 16), ("square_p2", 64), ("triangular", 32), ("cubic", 8), ("square_open", 15)):
+        assert planner(lattice, L, 100).slot.lone != 0
+        for reserved in (0, 2048):
+            sh = planner(lattice, L, 100, reserved=reserved)
+            assert sh is not None and sh.slot.lone == 0
