@@ -216,7 +216,7 @@ wl_status allocate(wl_ctx* h)
     if (!e) e = alloc((void**)&h->d_ident, lo.nlines * 4);
     if (!e) e = alloc((void**)&h->d_qheads, (lo.nlines + 1) * 4);
     if (!e) e = alloc((void**)&h->d_flags, 16);
-    if (!e) e = alloc((void**)&h->d_deadline, 16);
+    if (!e) e = alloc((void**)&h->d_deadline, 32);
     if (!e) e = alloc((void**)&h->d_summary, sizeof(Summary));
     if (!e) e = cudaHostAlloc((void**)&h->h_summary, sizeof(Summary), cudaHostAllocDefault);
     if (!e) e = cudaHostAlloc((void**)&h->h_abort, 16, cudaHostAllocMapped);
@@ -233,7 +233,7 @@ wl_status allocate(wl_ctx* h)
     std::vector<int32_t> ident(lo.nlines);
     for (int l = 0; l < lo.nlines; ++l) ident[l] = l;
     CU(cudaMemcpyAsync(h->d_ident, ident.data(), lo.nlines * 4, cudaMemcpyHostToDevice, h->s));
-    CU(cudaMemsetAsync(h->d_deadline, 0, 16, h->s));
+    CU(cudaMemsetAsync(h->d_deadline, 0, 32, h->s));
     CU(cudaStreamSynchronize(h->s));
     h->allocated = true;
     return WL_OK;
@@ -241,9 +241,12 @@ wl_status allocate(wl_ctx* h)
 
 Geo make_geo(const wl_ctx* h) { return wl::make_geo(h->g.type, (LatticeShape)h->g.type, h->g.L, h->g.N, h->g.NB, h->lo.W); }
 
-// The work queue: selected lines, slowest first.  A slice takes every line the same
-// number of moves further, and a move takes longest where few up spins make
-// neighbouring steps draw the same list slot.
+int32_t* queue_place(const wl_ctx* h) { return reinterpret_cast<int32_t*>(h->d_deadline + 2); }
+
+// The work queue: selected lines by ascending l.  A slice that ends by moves takes every
+// line equally far; batches take longest over a move where few up spins make neighbouring
+// steps draw the same list slot, so these lines go first.  One that ends by time goes
+// through the queue from its other end (queue_line).
 wl_status upload_queue(wl_ctx* h)
 {
     std::vector<int32_t> order;
@@ -251,6 +254,7 @@ wl_status upload_queue(wl_ctx* h)
         if (line_selected(h, l)) order.push_back(l);
     h->nqueue = (int)order.size();
     CU(cudaMemcpyAsync(h->d_order, order.data(), order.size() * 4, cudaMemcpyHostToDevice, h->s));
+    CU(cudaMemsetAsync(queue_place(h), 0, 8, h->s));
     return WL_OK;
 }
 
@@ -388,17 +392,28 @@ static void set_turns(wl_ctx* h, const Shape& sh, WalkArgs* a)
     a->turn = h->d_qheads;
 }
 
-// One slice of the persistent form on stream h->s (capturable).
-wl_status enqueue_slice(wl_ctx* h, int S, const Shape& sh)
+// The walker's arguments for a slice of the persistent form.
+WalkArgs slice_args(wl_ctx* h, const Shape& sh)
 {
     WalkArgs a = base_args(h);
     set_slot(sh.slot, &a);
     set_turns(h, sh, &a);
+    if (h->slice_ms > 0) a.first = queue_place(h);
+    return a;
+}
+
+// One slice of the persistent form on stream h->s (capturable).
+wl_status enqueue_slice(wl_ctx* h, int S, const Shape& sh)
+{
+    const WalkArgs a = slice_args(h, sh);
     if (a.turns > 1)
         CU(cudaMemsetAsync(h->d_qheads, 0, (size_t)(h->lo.nlines + 1) * 4, h->s));     // with qnext
     else
         CU(cudaMemsetAsync(a.qnext, 0, 4, h->s));
-    if (h->slice_ms > 0) CU(launch_set_deadline(h->d_deadline + 1, (uint64_t)h->slice_ms * 1000000ull, h->s));
+    const int walkers = (int)(sh.grid * (sh.slot.lone ? 1u : sh.block / (unsigned)S));
+    if (h->slice_ms > 0)
+        CU(launch_begin_slice(h->d_deadline + 1, (uint64_t)h->slice_ms * 1000000ull, queue_place(h), walkers,
+                              h->nqueue, h->s));
     CU(launch_walk(kernel_lattice(h), S, h->det != 0, h->lo.idx16, sh.grid, sh.block, sh.smem, h->s, a));
     CU(launch_summary(h->d_st, h->lo.nlines, h->budget, h->d_flags, h->d_summary, h->s));
     CU(cudaMemcpyAsync(h->h_summary, h->d_summary, sizeof(Summary), cudaMemcpyDeviceToHost, h->s));
@@ -413,9 +428,7 @@ wl_status run_slice(wl_ctx* h, int S, const Shape& sh, bool use_graph)
         h->launches += 2;
         return WL_OK;
     }
-    WalkArgs now = base_args(h);
-    set_slot(sh.slot, &now);
-    set_turns(h, sh, &now);
+    const WalkArgs now = slice_args(h, sh);
     // everything baked into the graph: the kernel (S, the acceptance rule, fields of its
     // arguments), its launch, its arguments, and the time limit set before it
     const bool same = h->graph && h->graph_S == S && h->graph_det == h->det && h->graph_grid == sh.grid &&

@@ -73,9 +73,10 @@ struct WalkArgs {
     int64_t* lng;            // ragged ln g / u
     hist_t* hist;            // ragged histogram | kVisited
     const uint32_t* table;   // exp threshold table (kTableN words)
-    const int32_t* order;    // work queue: line indices, most expensive first
+    const int32_t* order;    // work queue: line indices by ascending l, and so by bins
     int32_t* qnext;          // work queue head
     int32_t nqueue;
+    const int32_t* first;    // where a time-limited launch starts in the queue (queue_line); null: at its head
     int32_t q;               // table shift
     float seg_per_log2;      // ln 2 / (2^q u): table segments per halving of exp(-u d)
     float inv_u;             // 1 / u, production acceptance
@@ -306,6 +307,18 @@ struct Draw {
     uint32_t a, b;
     int64_t dmax;
 };
+
+// The line of entry x of the work queue.  A launch that ends by time may leave lines
+// at the end of the queue with a single check's moves.  Such launches go from the
+// longest line to the shortest, each on from where the one before had no walker left
+// (*first entries from the end), and around: every line has its share of the time.
+__device__ __forceinline__ int queue_line(const WalkArgs& A, int x)
+{
+    if (!A.first) return A.order[x];
+    x += *A.first;
+    if (x >= A.nqueue) x -= A.nqueue;
+    return A.order[A.nqueue - 1 - x];
+}
 
 // ---------------------------------------------------------------------------
 // Group helpers: S consecutive lanes of a warp serve one walker.

@@ -673,6 +673,22 @@ cudaError_t launch_set_deadline(uint64_t* deadline, uint64_t timeout_ns, cudaStr
     return cudaGetLastError();
 }
 
+__global__ void begin_slice_kernel(uint64_t* slice_end, uint64_t slice_ns, int32_t* first, int walkers, int nqueue)
+{
+    *slice_end = globaltimer_ns() + slice_ns;
+    const int at = first[1];
+    first[0] = at;
+    first[1] = (at + walkers) % nqueue;
+}
+
+cudaError_t launch_begin_slice(uint64_t* slice_end, uint64_t slice_ns, int32_t* first, int walkers, int nqueue,
+                               cudaStream_t s)
+{
+    clear_stale_error();
+    begin_slice_kernel<<<1, 1, 0, s>>>(slice_end, slice_ns, first, walkers, nqueue);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_walk(int lattice, int S, bool det, bool idx16, dim3 grid, dim3 block,
                         size_t smem, cudaStream_t s, const WalkArgs& a)
 {

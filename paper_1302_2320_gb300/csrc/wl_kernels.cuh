@@ -73,6 +73,10 @@ cudaError_t launch_dmax(size_t n, const uint32_t* r, int det, const uint32_t* ta
 cudaError_t launch_summary(const LineState* st, int nlines, int64_t budget, const int32_t* flags,
                            Summary* out, cudaStream_t s);
 cudaError_t launch_set_deadline(uint64_t* deadline, uint64_t timeout_ns, cudaStream_t s);
+// The start of a time-limited slice of `walkers` walkers over a queue of nqueue lines:
+// its end in device time, and its place in the queue (first[0]; first[1]: the next one's).
+cudaError_t launch_begin_slice(uint64_t* slice_end, uint64_t slice_ns, int32_t* first, int walkers, int nqueue,
+                               cudaStream_t s);
 cudaError_t launch_thermo(const LineDesc* desc, int nlines, const double* lng, int N, int NB,
                           int kstep, const double* T, int nT, const double* H, int nH, double* out,
                           void* scratch, cudaStream_t s);

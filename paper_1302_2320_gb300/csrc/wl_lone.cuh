@@ -561,7 +561,8 @@ __global__ void __launch_bounds__(kLoneThreads, TRI && WORD == 4 ? 8 : 10) lone_
         if (th == 0) {
             const int qi = atomicAdd(A.qnext, 1);
             const int r = A.turns > 1 ? qi / A.nqueue : 0;       // the line's turn
-            int li = A.turns > 1 ? (r < A.turns ? A.order[qi - r * A.nqueue] : -1) : qi < A.nqueue ? A.order[qi] : -1;
+            const int x = qi - r * A.nqueue;
+            int li = r < (A.turns > 1 ? A.turns : 1) && x < A.nqueue ? queue_line(A, x) : -1;
             if (li >= 0 && r > 0 && !lone_turn(A, li, r)) li = -2;
             ctl[0] = li;
             *last = 0u;

@@ -78,7 +78,7 @@ struct wl_ctx {
     int32_t* d_ident = nullptr;
     int32_t* d_qheads = nullptr;
     int32_t* d_flags = nullptr;
-    uint64_t* d_deadline = nullptr;
+    uint64_t* d_deadline = nullptr;       // the run's deadline, the slice's end, the place in the queue (two words)
     wl::Summary* d_summary = nullptr;
     void* d_thermo = nullptr;             // workspace of wl_thermo, from its first call on
     size_t thermo_bytes = 0;

@@ -761,7 +761,7 @@ __global__ void walk_kernel(const WalkArgs A)
         if (m == 0) qi = atomicAdd(A.qnext, 1);
         qi = __shfl_sync(gmask, qi, gbase);
         if (qi >= A.nqueue) break;
-        const int li = A.order[qi];
+        const int li = queue_line(A, qi);
         if (A.st[li].status != 0) continue;
         IDX* gperm = reinterpret_cast<IDX*>(A.perm) + (size_t)li * pstride;
         uint32_t* gsp = A.spins + (size_t)li * W;

@@ -48,3 +48,17 @@ def test_a_shorter_time_limit_of_a_slice_holds_from_the_next_walk_on():
     h.set_option("slice_ms", 1)
     h.run(1e-6, 0.8)
     assert h.stats()["launches"] >= 2 + 2 * 4
+
+
+@pytest.mark.parametrize("L,tail", [(64, 1), (96, 0)])
+def test_slices_that_end_by_time_take_every_line_along(L, tail):
+    """More lines than walkers at once and no budget that ends a line's slice: after some
+    60 slices no line that still walks has a fraction of another's moves."""
+    h = wl.Handle("square", L, seed=5, check_interval=1000, move_budget=1 << 40, slice_moves=1 << 40, slice_ms=4,
+                  timeout_ms=240, tail=tail, mapping=32)
+    assert h.run(1e-6, 0.8, allow=(wl.WL_ETIMEOUT,)) == wl.WL_ETIMEOUT
+    states = [h.line_state(ell)["sc"] for ell in range(64, h.lines, h.lines // 64)]
+    moves = [int(sc[1]) for sc in states if sc[6] == 0]
+    assert len(moves) > 48
+    assert min(moves) * 3 > max(moves), (min(moves), max(moves))
+    h.close()
