@@ -378,18 +378,10 @@ wl_status persistent_shape(wl_ctx* h, int S, int active, Shape* sh)
     return plan_shape(k, sh);
 }
 
-// More lines than blocks: they take turns, so that all blocks have work until the end of
-// the slice and not the last round's few (2^18 moves each, 1569 lines of 56x56 on 1520
-// blocks: 37.7 -> 26.7 ms; 2049 lines of 64x64 on 1520: 40.4 -> 33.2).
-// Turns of 2^14 moves and more: loading and storing a line takes ~50 us, a turn 1.3 ms.
 static void set_turns(wl_ctx* h, const Shape& sh, WalkArgs* a)
 {
-    a->turns = 1;
-    if (!sh.slot.lone || h->nqueue <= (int)sh.grid) return;
-    const int64_t moves = std::min(a->slice_moves, a->budget);
-    if (moves > (1 << 26)) return;       // turns of more than a second
-    a->turns = (int)std::max<int64_t>(1, std::min<int64_t>(8, moves >> 14));
-    a->turn = h->d_qheads;
+    a->turns = line_turns(sh, h->running, std::min(h->slice_moves, h->budget));
+    if (a->turns > 1) a->turn = h->d_qheads;
 }
 
 // The walker's arguments for a slice of the persistent form.
@@ -459,9 +451,10 @@ wl_status run_slice(wl_ctx* h, int S, const Shape& sh, bool use_graph)
     return WL_OK;
 }
 
-// Device-side stop conditions recorded during a launch.
+// What a slice's summary says: the lines that still run, and stop conditions on the device.
 wl_status check_flags(wl_ctx* h, const Summary& sm)
 {
+    h->running = sm.active;
     if (sm.flags & 8) return fail(WL_ECUDA, "walker state invariant broken (k' outside its bins)");
     if (sm.overflow || (sm.flags & 4)) return fail(WL_EOVERFLOW, "a histogram bin exceeded 2^63-1 within one stage");
     if (sm.flags & 3) {
@@ -670,6 +663,7 @@ wl_status prepare(wl_ctx* h, double ln_f_min, double flatness, cudaStream_t afte
     } else if (ln_f_min != h->u || flat_pm != h->flat_pm) {
         return fail(WL_EINVAL, "a continued run must use the same ln_f_min and flatness");
     }
+    h->running = h->nqueue;
     h->assembled = false;
     return WL_OK;
 }

@@ -89,6 +89,7 @@ struct wl_ctx {
     double table_u = 0.0;                 // the ln f_min it is for (0: none)
     bool table_checked = false;           // equal to the host's own build of it
     int nqueue = 0;
+    int running = 0;                      // lines of the queue that were not done after the last slice
     // captured slice graph
     cudaGraphExec_t graph = nullptr;
     int graph_S = -1, graph_det = -1;

@@ -6,6 +6,8 @@
 using namespace wl;
 using namespace wl::rt;
 
+extern "C" int turns_of(const Shape* sh, long long running, long long moves) { return line_turns(*sh, running, moves); }
+
 extern "C" int plan_shapes(const ShapeKey* k, const Gpu* gpu, int max_lone, int max_batch, Shape* out)
 {
     auto resident = [&](const Slot& slot, size_t smem, int) {

@@ -62,6 +62,7 @@ def planner():
             return None
         assert s.smem <= g.per_block and s.grid >= 1 and s.slot.win >= 1
         return s
+    plan.turns = lambda sh, running, moves: lib.turns_of(ctypes.byref(sh), ctypes.c_longlong(running), ctypes.c_longlong(moves))
     return plan
 
 
@@ -87,3 +88,13 @@ def test_a_block_per_line_only_where_shared_memory_starts_at_its_address(planner
         for reserved in (0, 2048):
             sh = planner(lattice, L, 100, reserved=reserved)
             assert sh is not None and sh.slot.lone == 0
+
+
+def test_turns_are_for_running_lines_without_a_block(planner):
+    sh = planner("square_p2", 64, 2049)
+    assert sh.slot.lone and 1400 < sh.grid < 2049
+    assert planner.turns(sh, 2049, 1 << 20) == 8
+    assert planner.turns(sh, 2049, 1 << 15) == 2 and planner.turns(sh, 2049, 5000) == 1
+    assert planner.turns(sh, 2049, (1 << 26) + 1) == 1
+    assert planner.turns(sh, sh.grid, 1 << 20) == 1             # the others are done
+    assert planner.turns(planner("square_p2", 64, 2049, lone=False), 5000, 1 << 20) == 1
