@@ -131,7 +131,8 @@ size_t wl_required_bytes(wl_lattice lattice, int L);
  * line range after a run requires wl_reset().  Errors: WL_EINVAL (unknown key or bad value), WL_ESTATE. */
 wl_status wl_set_option(wl_handle h, const char* key, int64_t value);
 /* Read an option back; also the read-only keys "N", "NB", "z", "k_step",
- * "lines", "bins", "device_bytes" and "tuned_mapping" (the lane count the tuner
+ * "lines", "bins", "device_bytes" (wl_required_bytes and what wl_thermo has kept)
+ * and "tuned_mapping" (the lane count the tuner
  * settled on for this lattice and mode, 0 while it is still timing candidates or
  * where no lane count is tuned). */
 wl_status wl_get_option(wl_handle h, const char* key, int64_t* value);
@@ -202,7 +203,9 @@ wl_status wl_get_stats(wl_handle h, wl_stats* out);
  * field H[c], per spin, out[(a*nH + c)*6 + 0..5] = ln Z / N, <E>/N,
  * C/N = (<E^2> - <E>^2) / (N T^2), <M>/N, <|M|>/N, chi/N = (<M^2> - <M>^2)/(N T),
  * with M = 2l - N (l up spins; lines l > N/2 are their mirrors).  Host arrays.
- * Needs wl_assemble over every line l = 0..N/2 (else WL_ESTATE).  FP64. */
+ * Needs wl_assemble over every line l = 0..N/2 (else WL_ESTATE).  FP64.
+ * Workspace: up to 4 MB stay with the handle where "hbm_budget" leaves room for
+ * them, and count in "device_bytes"; more is given back before the call returns. */
 wl_status wl_thermo(wl_handle h, const double* T, int nT, const double* H, int nH, double* out);
 
 /* The walker of one line as the method section defines it (current k, the

@@ -131,6 +131,8 @@ void host_table(double u, int q, std::vector<uint64_t>& t)
     for (int i = 0; i < kTableN; ++i) t[i] = wl::rt::table_entry(u, q, i);
 }
 
+constexpr size_t kThermoKept = (size_t)4 << 20;      // the largest workspace of wl_thermo that stays with a handle
+
 struct TuneKey {
     int type, L, det;
     bool operator<(const TuneKey& o) const
@@ -893,7 +895,7 @@ wl_status wl_get_option(wl_handle h, const char* key, int64_t* v)
     else if (k == "k_step") *v = h->g.kstep;
     else if (k == "lines") *v = h->lo.nlines;
     else if (k == "bins") *v = h->lo.nbins_total;
-    else if (k == "device_bytes") *v = (int64_t)required_bytes(h->g, h->lo);
+    else if (k == "device_bytes") *v = (int64_t)(required_bytes(h->g, h->lo) + h->thermo_bytes);
     else return fail(WL_EINVAL, "unknown option '%s'", key);
     return WL_OK;
 }
@@ -1138,22 +1140,28 @@ wl_status wl_thermo(wl_handle h, const double* T, int nT, const double* H, int n
         if (!(T[a] > 0.0)) return fail(WL_EINVAL, "temperatures must be > 0");
     const size_t nd = (size_t)nT + (size_t)nH + 6 * (size_t)nT * (size_t)nH;
     const size_t need = nd * sizeof(double) + thermo_scratch_bytes(h->lo.nlines, nT);
-    // the workspace is kept with the handle: to map and unmap it on every call takes
-    // longer than a scan of a small surface
-    if (h->thermo_bytes < need) {
+    // A small workspace is kept with the handle, inside its memory budget: to map and unmap
+    // it on every call takes longer than a scan of a small surface.  A large one is given
+    // back at the end of the call.
+    const size_t held = required_bytes(h->g, h->lo);
+    const bool keep = need <= kThermoKept && (h->hbm_budget == 0 || held + need <= (size_t)h->hbm_budget);
+    if (keep && h->thermo_bytes < need) {
         if (h->d_thermo) CU(cudaFree(h->d_thermo));
         h->d_thermo = nullptr;
         h->thermo_bytes = 0;
         CU(cudaMalloc(&h->d_thermo, need));
         h->thermo_bytes = need;
     }
-    double* d = static_cast<double*>(h->d_thermo);
+    void* once = nullptr;
+    if (!keep) CU(cudaMallocAsync(&once, need, h->s));
+    double* d = static_cast<double*>(keep ? h->d_thermo : once);
     cudaError_t e = cudaMemcpyAsync(d, T, nT * sizeof(double), cudaMemcpyHostToDevice, h->s);
     if (!e) e = cudaMemcpyAsync(d + nT, H, nH * sizeof(double), cudaMemcpyHostToDevice, h->s);
     if (!e) e = launch_thermo(h->d_desc, h->lo.nlines, h->d_out, h->g.N, h->g.NB, h->g.kstep, d, nT,
                               d + nT, nH, d + nT + nH, d + nd, h->s);
     if (!e) e = cudaMemcpyAsync(out, d + nT + nH, 6 * (size_t)nT * nH * sizeof(double),
                                 cudaMemcpyDeviceToHost, h->s);
+    if (once) cudaFreeAsync(once, h->s);
     if (!e) e = cudaStreamSynchronize(h->s);
     if (e) return fail(WL_ECUDA, "wl_thermo: %s", cudaGetErrorString(e));
     return WL_OK;

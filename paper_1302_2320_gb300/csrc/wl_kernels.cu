@@ -640,9 +640,10 @@ __global__ void __launch_bounds__(256) thermo_points_kernel(const LineDesc* desc
 
 size_t thermo_scratch_bytes(int nlines, int nT)
 {
-    // temperatures are taken in groups whose line sums fit 64 MB (one at least)
+    // temperatures are taken in groups whose line sums fit 2 MB (one at least): a group of
+    // a large surface has work for all SMs all the same
     const size_t one = (size_t)nlines * sizeof(LineSum);
-    return one * std::min<size_t>((size_t)nT, std::max<size_t>(1, ((size_t)64 << 20) / one));
+    return one * std::min<size_t>((size_t)nT, std::max<size_t>(1, ((size_t)2 << 20) / one));
 }
 
 cudaError_t launch_thermo(const LineDesc* desc, int nlines, const double* lng, int N, int NB,

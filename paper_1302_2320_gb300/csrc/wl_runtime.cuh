@@ -80,7 +80,7 @@ struct wl_ctx {
     int32_t* d_flags = nullptr;
     uint64_t* d_deadline = nullptr;       // the run's deadline, the slice's end, the place in the queue (two words)
     wl::Summary* d_summary = nullptr;
-    void* d_thermo = nullptr;             // workspace of wl_thermo, from its first call on
+    void* d_thermo = nullptr;             // workspace of wl_thermo, kept where it is small
     size_t thermo_bytes = 0;
     wl::Summary* h_summary = nullptr;         // pinned
     int32_t* h_abort = nullptr;           // pinned, mapped

@@ -62,3 +62,25 @@ def test_slices_that_end_by_time_take_every_line_along(L, tail):
     assert len(moves) > 48
     assert min(moves) * 3 > max(moves), (min(moves), max(moves))
     h.close()
+
+
+def test_workspace_of_thermodynamics_is_counted_and_within_the_budget():
+    """A small one stays with the handle and shows in device_bytes, unless the budget has
+    no room for it; a large one is given back.  The values do not depend on it."""
+    need = wl.wl_required_bytes(wl.LATTICES["square"], 16)
+    T, H = np.linspace(1.0, 5.0, 600), np.linspace(0.0, 2.0, 200)       # 5.8 MB of results
+    got = {}
+    for name, budget in (("free", 0), ("tight", need)):
+        h = wl.Handle("square", 16, seed=2, check_interval=1000, move_budget=20_000, hbm_budget=budget)
+        h.run(1e-6, 0.8)
+        h.assemble()
+        assert h.get_option("device_bytes") == need
+        large = h.thermo(T, H)
+        assert h.get_option("device_bytes") == need
+        small = h.thermo(T[:3], H[:2])
+        held = h.get_option("device_bytes") - need
+        assert held == 0 if name == "tight" else 0 < held <= 4 << 20
+        assert np.array_equal(small, large[:3, :2]) and np.isfinite(large).all()
+        got[name] = small
+        h.close()
+    assert np.array_equal(got["free"], got["tight"])
