@@ -495,10 +495,11 @@ cudaError_t launch_summary(const LineState* st, int nlines, int64_t budget, cons
 // (T, line) and the fields are then a sum over lines: bins x nT exponentials and not
 // 2 x bins x nT x nH, spread over (lines x nT) warps and not nT x nH blocks.  FP64 is
 // slow on this GPU, and most bins of a line weigh nothing at a given T, so the line's
-// maximum is found first and only bins within e^-46 of it (1e-20, so that a line of
-// 4097 bins loses less than a rounding of its sum) take an exponential.  Moments are kept about the line's
-// likeliest bin and then about the mean, where the variances of C and chi do not
-// cancel.  32x32, 64 T x 3 H: 7.8 ms as one block per point with an exponential for
+// maximum is found first and only bins within e^-46 of it (1e-20) take an exponential:
+// a line of 4097 bins loses less than a rounding of its sum, and of its second moment
+// less than 1e-20 (2 N_B)^2 a bin, 3e-12 at 64x64, where squares of energies that cancel
+// lose more.  Moments are kept about the line's likeliest bin and then about the mean,
+// where the variances of C and chi do not cancel.  32x32, 64 T x 3 H: 7.8 ms as one block per point with an exponential for
 // every bin and mirror, 0.6 ms this way.
 // ---------------------------------------------------------------------------
 struct LineSum {
