@@ -655,6 +655,7 @@ def run_ours(args):
     torch.cuda.synchronize()
     if dist:
         dist.barrier()
+    block_per_line = bool(h.get_option("block_per_line"))
     step_ms = [a.elapsed_time(b) for a, b in ev]
     total_ms = sum(step_ms)
 
@@ -719,7 +720,7 @@ def run_ours(args):
                    "parallelism": f"replicas x{world}"},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "Tops/s",
                      "frac": achieved / alu_peak, "traffic": traffic,
-                     "kernel": "lone_kernel" if L <= 112 and args.form == 0 else "walk_kernel", "ops_per_move": INT_OPS_PER_MOVE,
+                     "kernel": "lone_kernel" if block_per_line else "walk_kernel", "ops_per_move": INT_OPS_PER_MOVE,
                      "peak_basis": (f"measured on this GPU by wl_measure_peaks: {MUL_OPS_PER_MOVE} "
                                     f"32x32->64 products at {rates['mulwide_ops_per_s']:.3g}/s plus "
                                     f"{ALU_OPS_PER_MOVE} add/logic ops at {rates['iadd3_ops_per_s']:.3g}/s "
@@ -737,7 +738,7 @@ def run_ours(args):
         "gpu_launches": launches,
         "clocks": clk,
         "walk_ms_per_step": walk_ms / args.steps,
-        "accept_rate": acc_rate, "moves_per_batch": moves / max(batches, 1),
+        "accept_rate": acc_rate, "moves_per_batch": None if block_per_line else moves / max(batches, 1),
     }
     print(json.dumps(line), flush=True)
     h.close()

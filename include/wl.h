@@ -63,7 +63,7 @@ typedef struct {
     int64_t moves;            /* move attempts made, summed over lines          */
     int64_t accepts;          /* accepted exchange proposals                    */
     int64_t checks;           /* flatness checks made                           */
-    int64_t batches;          /* batches of moves (moves per batch = moves / batches) */
+    int64_t batches;          /* batches of moves (a block per line: draws of 32)     */
     int32_t lines;            /* lines walked (l = 0..N/2)                      */
     int32_t lines_converged;  /* lines with ln f < ln f_min                     */
     int32_t min_stage;        /* fewest completed stages over lines             */
@@ -131,10 +131,11 @@ size_t wl_required_bytes(wl_lattice lattice, int L);
  * line range after a run requires wl_reset().  Errors: WL_EINVAL (unknown key or bad value), WL_ESTATE. */
 wl_status wl_set_option(wl_handle h, const char* key, int64_t value);
 /* Read an option back; also the read-only keys "N", "NB", "z", "k_step",
- * "lines", "bins", "device_bytes" (wl_required_bytes and what wl_thermo has kept)
- * and "tuned_mapping" (the lane count the tuner
- * settled on for this lattice and mode, 0 while it is still timing candidates or
- * where no lane count is tuned). */
+ * "lines", "bins", "device_bytes" (wl_required_bytes and what wl_thermo has kept),
+ * "tuned_mapping" (the lane count the tuner settled on for this lattice and mode, 0
+ * while it is still timing candidates or where no lane count is tuned) and
+ * "block_per_line" (1: the last slice of the last wl_run walked with a block per
+ * line; 0: in batches). */
 wl_status wl_get_option(wl_handle h, const char* key, int64_t* value);
 
 /* The walk of the method section, on every selected line: spin-exchange

@@ -543,6 +543,7 @@ wl_status run_persistent(wl_ctx* h, std::chrono::steady_clock::time_point t_star
         CU(cudaStreamSynchronize(h->s));
         const Summary sm = *h->h_summary;
         h->last_mapping = curS;
+        h->last_lone = sh.slot.lone != 0;
         const int64_t dm = sm.moves - prev_moves;
         if (dm > 0) last_accept = (double)(sm.accepts - prev_accepts) / (double)dm;
         if (tried >= 0 && dm > 0) {
@@ -585,6 +586,7 @@ wl_status run_plain(wl_ctx* h)
 {
     int S = h->mapping ? h->mapping : pick_mapping_default(h);
     h->last_mapping = S;
+    h->last_lone = false;
     const int npool = 128;      // the device runs at most 128 kernels at once
     while ((int)h->pool.size() < npool) {
         cudaStream_t st;
@@ -884,6 +886,7 @@ wl_status wl_get_option(wl_handle h, const char* key, int64_t* v)
         auto it = g_tune_cache.find({h->g.type, h->g.L, h->det});
         *v = it != g_tune_cache.end() ? it->second.best : 0;
     }
+    else if (k == "block_per_line") *v = h->last_lone;
     else if (k == "hbm_budget") *v = h->hbm_budget;
     else if (k == "ell_min") *v = h->ell_min;
     else if (k == "same_f_resets") *v = h->same_f_resets;

@@ -55,6 +55,7 @@ struct wl_ctx {
     int flat_pm = 0;
     int q = 0;
     int last_mapping = 0;
+    bool last_lone = false;      // the last slice walked with a block per line
     int64_t launches = 0;
     double walk_ms = 0, assemble_ms = 0;
     int64_t init_moves = 0;

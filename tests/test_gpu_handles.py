@@ -84,3 +84,12 @@ def test_workspace_of_thermodynamics_is_counted_and_within_the_budget():
         got[name] = small
         h.close()
     assert np.array_equal(got["free"], got["tight"])
+
+
+@pytest.mark.parametrize("opt,expect", [({}, 1), ({"mapping": 32}, 1), ({"mapping": 8}, 0), ({"tail": 0}, 0),
+                                        ({"form": 1}, 0)])
+def test_the_library_names_the_walker_that_ran(opt, expect):
+    h = wl.Handle("square", 16, seed=2, check_interval=1000, move_budget=5_000, **opt)
+    h.run(1e-6, 0.8)
+    assert h.get_option("block_per_line") == expect
+    h.close()
