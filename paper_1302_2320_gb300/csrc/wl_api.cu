@@ -5,10 +5,9 @@
 // symmetry), ragged per-line ln g / histogram arrays over the even k, packed
 // spins and up/down index lists, all resident on the device across calls.
 // wl_run drives the walk in slices: each slice is one persistent launch over a
-// device work queue (lines ordered by estimated cost, most expensive first),
-// followed by a summary kernel whose result is read back; the slice is
-// captured once as a CUDA graph and replayed.  The alternative "plain" form
-// issues one launch per line over a pool of streams.
+// device work queue of lines (queue_line), followed by a summary kernel whose
+// result is read back; the slice is captured once as a CUDA graph and replayed.
+// The alternative "plain" form issues one launch per line over a pool of streams.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -477,8 +476,8 @@ int kernel_lattice(const wl_ctx* h)
     return h->g.type;
 }
 
-// 32 lanes per walker: on the 64x64 lattice a batch commits ~26 moves and this
-// mapping was fastest for every lattice measured.
+// 32 lanes per walker: the fastest batches of every lattice measured (64x64: 3.7e9 moves/s
+// with 32 lanes, 3.5e9 with 16, 2.6e9 with 8; 128x128: 1.24e10, 6.0e9, 5.2e9).
 int pick_mapping_default(const wl_ctx*)
 {
     return 32;

@@ -176,7 +176,7 @@ cudaError_t launch_check_state(int lattice, bool idx16, const InitArgs& a, int32
 template <int LAT, typename IDX>
 static cudaError_t init_one(InitArgs a, cudaStream_t s)
 {
-    // up to 64 KB of list per block, or the whole of an SM's shared memory for a line
+    // any list that fits a block's shared memory
     const size_t list = (size_t)a.pstride * sizeof(IDX);
     int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);

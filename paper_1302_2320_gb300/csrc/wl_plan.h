@@ -72,9 +72,9 @@ inline int line_turns(const Shape& sh, int64_t running, int64_t moves)
 inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 // A walker's slot: the list (staged or not), the sites, the window, the step
-// records.  The window is what is left of `room` bytes, up to the whole line; a
-// guard on both sides of it keeps every address inside the slot even where a
-// caller's own state (wl_walk_noalloc) is not one of the line's.
+// records.  The window is what is left of `room` bytes, up to the whole line; the
+// chain loads ln g before it knows that a step is out of date, a few bins off at most:
+// a guard on both sides keeps that inside the slot.
 inline bool plan_slot(const ShapeKey& k, bool sites, bool perm, size_t room, int least_win, Slot* o)
 {
     constexpr int kGuard = 8 * 8 * (12 + 1);      // kSub steps of the largest bin step, in bytes
@@ -100,7 +100,9 @@ inline bool plan_slot(const ShapeKey& k, bool sites, bool perm, size_t room, int
 }
 
 // The slot of a line with a block of its own (wl_lone.cuh): the words of the sites
-// by code, the list, the window, the ring.
+// by code, the list, the window, the ring.  The window needs no guard: a step is
+// evaluated from the state it is taken from, and every state is a line's own, by the
+// library's initialisation or by the exact check of a caller's (check_state_kernel).
 inline bool plan_lone(const ShapeKey& k, int word, size_t room, Slot* o)
 {
     if (!k.idx16) return false;
@@ -128,16 +130,30 @@ inline bool plan_lone(const ShapeKey& k, int word, size_t room, Slot* o)
     return true;
 }
 
-// Cycles a move takes its walker (GB300).
+// Cycles a move takes its walker (GB300), for the choice between shapes.
 // A block per line (wl_lone.cuh), words of 4 bytes or of one: 119 and 126 with up to 4 on
-// an SM, one for each scheduler; 153 and 159 with 5 or 6, 162 and 168 with 7 or 8, 217
-// (words of a byte; 197 where they take turns) with 9 or 10 (64x64).
+// an SM, one for each scheduler.  With more on an SM a move alone takes 153 and 159 (5 or
+// 6), 162 and 168 (7 or 8), 197 (9 or 10, in turns; 64x64).  In a whole surface the loads
+// of lines, checks and windows weigh as well, and more of them hide more of that: with 4
+// and 5 on an SM 112x112 takes 163 and 173 cycles a move.  kLoneCrowd is what ranks whole
+// surfaces rightly: the ratios of moves alone (1.29, 1.36, 1.58) in its place choose 4 and
+// not 5 on an SM at 112x112 (26.6 and not 22.7 ms for 2^15 moves) and cubic 20^3 (17.0 and
+// 14.3), and 10 and not 8 at 56x56 (28.2 and 27.2 ms, 2^18).
+// Rounds of a block per line are lines / blocks as they are, also where lines take no
+// turns: the lines of the last round have an SM to fewer, and are faster.  Counted whole
+// they gain 3 % at 64x64 (a continuation without allocation, 7 and not 10 on an SM) and
+// lose 5 % at 56x56, 7 % at triangular 58x58 and 18 % at cubic 20^3.
 // Batches (wl_walk.cuh): 191 with 7 on an SM and the lists staged (96x96), 272 with 16
 // on an SM and the lists in global memory (96x96) or 12 and staged (64x64); and what a
 // surface's lines of few up spins take longer, whose batches keep running into
-// themselves.  Whole surfaces, cycles for a move of all lines, block per line against
-// batches: 64x64 262 and 1189, 96x96 795 and 1367, 112x112 1260 and ~1350,
-// 128x128 1920 and 1536.
+// themselves.
+// Where the line between the two lies, block per line and batches, ms for 2^15 moves of
+// all lines: square 112x112 21.7 and 24.4, 116x116 27.4 and 24.4, 128x128 33.6 and 23.0;
+// triangular 112x112 23.2 and 24.6, 120x120 30.3 and 26.7; cubic 23^3 24.9 and 26.5, 24^3
+// 37.2 and 26.1.  With production acceptance a block per line is the same within 1 % and
+// batches take from 4 % more to 13 % less there (116x116: 29.9).  Open boundaries cross
+// earlier, between 100x100 (17.1 and 20.1) and 108x108 (20.6 and 18.4; 112x112: 25.8 and
+// 17.3), which the figures below, those of square lattices, do not know.
 inline constexpr double kLoneCycles[2] = {119.0, 126.0}, kLoneCrowd[4] = {1.0, 1.2, 1.27, 1.58}, kBatchIssue = 17.0, kBatchSlowest = 600.0;
 
 // Either a block of two warps per line, or one warp per block with 32 / S walkers,
@@ -178,7 +194,7 @@ Planned plan_shape(const ShapeKey& k, const Gpu& gpu, Resident&& resident, Shape
             const int bps = resident(slot, (size_t)slot.bytes, 64);
             if (bps < 0) return Planned::unknown;
             if (bps < b) continue;
-            // lines that take turns keep all blocks busy to the end
+            // rounds as a fraction (above)
             const double cost = std::max(1.0, (double)k.lines / (sms * b)) * cycles(b);
             if (best_blocks != 0 && cost >= best) continue;
             best = cost;
